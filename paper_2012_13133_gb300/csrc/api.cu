@@ -126,6 +126,7 @@ void ctx_trim(kry_ctx* ctx) {
         // the whole-grid index lists are rebuilt on demand unless a site map needs them
         ctx->rowptr_full.release();
         ctx->colidx_full.release();
+        ctx->cellbits_full.release();
         ctx->full_n1 = ctx->full_n2 = 0;
     }
 }
@@ -178,9 +179,10 @@ __global__ void k_interior_count(const uint8_t* __restrict__ mask, int n1, int n
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, (unsigned long long)c);
 }
 
-// Ordered compaction of one row: colidx and cellidx of its observed cells.
+// Ordered compaction of one row: colidx and cellidx of its observed cells, and
+// per 32 cells their observation bits with the index of the first observed one.
 __global__ void k_row_fill(const uint8_t* __restrict__ mask, int n2, const int* __restrict__ rowptr,
-                           int* __restrict__ colidx, int* __restrict__ cellidx) {
+                           int* __restrict__ colidx, int* __restrict__ cellidx, uint2* __restrict__ bits) {
     const int row = blockIdx.x;
     __shared__ int wsum[32];
     __shared__ int base;
@@ -196,6 +198,8 @@ __global__ void k_row_fill(const uint8_t* __restrict__ mask, int n2, const int* 
         int off = 0;
         for (int k = 0; k < w; ++k) off += wsum[k];
         const int pos = base + off + __popc(bal & ((1u << lane) - 1u));
+        if (lane == 0 && j < n2)
+            bits[(int64_t)row * ((n2 + 31) / 32) + (j >> 5)] = make_uint2(bal, (unsigned)(base + off));
         if (f) {
             colidx[pos] = j;
             cellidx[pos] = row * n2 + j;
@@ -260,10 +264,12 @@ static void check_embed(kry_ctx* ctx, const kry_embed* e) {
     require_mask(ctx);
 }
 
-// True if FP32 matvecs on this embedding run the length-specialised passes
-// (their column pass reads the permuted eigenvalue copy lam32P).
-static bool spec_column_pass(const kry_ctx* ctx, const kry_embed* e) {
-    return ctx->use_spec && e->M1 >= 64 && e->M2 >= 64 && e->M1 <= 8192 && e->M2 <= 8192;
+// FP32 eigenvalues of ntheta settings: the permuted form that the specialised
+// passes read (torus sides from 64), or the plain transposed one.
+static void alloc_lam32(kry_ctx* ctx, kry_embed* e, size_t ntheta) {
+    const size_t bytes = ntheta * e->M1 * e->M2 * sizeof(float);
+    const bool spec = e->M1 >= 64 && e->M2 >= 64;
+    dev_alloc((void**)(spec ? &e->lam32P : &e->lam32T), bytes, ctx->stream);
 }
 
 // True if FP32 iterates resolve the covariance whose embedding eigenvalues span
@@ -298,8 +304,7 @@ static kry_embed* make_embed(kry_ctx* ctx, const kry_cov* cov, kry_prec prec, bo
         }
         const size_t MM = (size_t)e->M1 * e->M2;
         dev_alloc((void**)&e->lam64T, MM * sizeof(double), ctx->stream);
-        if (prec == KRY_F32) dev_alloc((void**)&e->lam32T, MM * sizeof(float), ctx->stream);
-        if (prec == KRY_F32 && spec_column_pass(ctx, e)) dev_alloc((void**)&e->lam32P, MM * sizeof(float), ctx->stream);
+        if (prec == KRY_F32) alloc_lam32(ctx, e, 1);
         kry::store_embedding(ctx, e, 0);
     } catch (...) {
         if (e->lam64T) cudaFreeAsync(e->lam64T, ctx->stream);
@@ -348,8 +353,7 @@ static kry_embed* make_precond_embed(kry_ctx* ctx, const kry_cov* cov, const kry
         kry::invert_eigs(ctx, e->M1, e->M2, cov->tau2);
         const size_t MM = (size_t)e->M1 * e->M2;
         dev_alloc((void**)&e->lam64T, MM * sizeof(double), ctx->stream);
-        dev_alloc((void**)&e->lam32T, MM * sizeof(float), ctx->stream);
-        if (spec_column_pass(ctx, e)) dev_alloc((void**)&e->lam32P, MM * sizeof(float), ctx->stream);
+        alloc_lam32(ctx, e, 1);
         kry::store_embedding(ctx, e, 0);
     } catch (...) {
         if (e->lam64T) cudaFreeAsync(e->lam64T, ctx->stream);
@@ -403,9 +407,7 @@ static kry_embed* make_embed_batch(kry_ctx* ctx, const kry_cov* thetas, int nthe
     e->lam_stride = (int64_t)MM;
     try {
         dev_alloc((void**)&e->lam64T, ntheta * MM * sizeof(double), ctx->stream);
-        if (prec == KRY_F32) dev_alloc((void**)&e->lam32T, ntheta * MM * sizeof(float), ctx->stream);
-        if (prec == KRY_F32 && spec_column_pass(ctx, e))
-            dev_alloc((void**)&e->lam32P, ntheta * MM * sizeof(float), ctx->stream);
+        if (prec == KRY_F32) alloc_lam32(ctx, e, ntheta);
         dev_alloc((void**)&e->tau2_dev, ntheta * sizeof(double), ctx->stream);
         std::vector<double> t2(ntheta);
         for (int t = 0; t < ntheta; ++t) {
@@ -446,9 +448,9 @@ kry_status kry_create(kry_ctx** out, int device, void* cuda_stream) {
         KRY_CUDA(cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
         // every scratch buffer is stream-ordered on the context stream; keep freed
         // pool memory cached in this process instead of returning it at each sync
-        DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->tw32, &ctx->tw64, &ctx->twt32, &ctx->slab32,
+        DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->tw64, &ctx->spec_tab, &ctx->slab32,
                           &ctx->slab64, &ctx->scal, &ctx->eig_c, &ctx->eig_z, &ctx->eig_d, &ctx->red, &ctx->tolbuf,
-                          &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full,
+                          &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full, &ctx->cellbits_full,
                       &ctx->sites.corner, &ctx->sites.w64, &ctx->sites.w32, &ctx->sites.cellptr, &ctx->sites.ent_site,
                       &ctx->sites.ent_w64, &ctx->sites.ent_w32, &ctx->sites.cnt, &ctx->sites.grid32, &ctx->sites.grid64};
         for (DevBuf* b : bufs) b->stream = ctx->stream;
@@ -476,9 +478,9 @@ void kry_destroy(kry_ctx* ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     else cudaDeviceSynchronize();
-    DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->tw32, &ctx->tw64, &ctx->twt32, &ctx->slab32,
+    DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->tw64, &ctx->spec_tab, &ctx->slab32,
                       &ctx->slab64, &ctx->scal, &ctx->eig_c, &ctx->eig_z, &ctx->eig_d, &ctx->red, &ctx->tolbuf,
-                      &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full,
+                      &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full, &ctx->cellbits_full,
                       &ctx->sites.corner, &ctx->sites.w64, &ctx->sites.w32, &ctx->sites.cellptr, &ctx->sites.ent_site,
                       &ctx->sites.ent_w64, &ctx->sites.ent_w32, &ctx->sites.cnt, &ctx->sites.grid32, &ctx->sites.grid64};
     for (DevBuf* b : bufs) b->release();
@@ -503,6 +505,7 @@ kry_status kry_set_mask(kry_ctx* ctx, const kry_grid* grid, const uint8_t* mask_
         ctx->rowptr.ensure((size_t)(n1 + 1) * sizeof(int));
         ctx->colidx.ensure((size_t)n1 * n2 * sizeof(int));
         ctx->cellidx.ensure((size_t)n1 * n2 * sizeof(int));
+        ctx->cellbits.ensure((size_t)n1 * ((n2 + 31) / 32) * sizeof(uint2));
         ctx->red.ensure((size_t)(n1 + 4) * sizeof(int) + sizeof(unsigned long long));
         int* counts = ctx->red.as<int>();
         k_row_counts<<<n1, 256, 0, ctx->stream>>>(mask_dev, n2, counts);
@@ -510,7 +513,7 @@ kry_status kry_set_mask(kry_ctx* ctx, const kry_grid* grid, const uint8_t* mask_
         k_rowptr<<<1, 32, 0, ctx->stream>>>(counts, n1, ctx->rowptr.as<int>());
         KRY_CHECK_LAUNCH();
         k_row_fill<<<n1, 256, 0, ctx->stream>>>(mask_dev, n2, ctx->rowptr.as<int>(), ctx->colidx.as<int>(),
-                                                ctx->cellidx.as<int>());
+                                                ctx->cellidx.as<int>(), ctx->cellbits.as<uint2>());
         KRY_CHECK_LAUNCH();
         unsigned long long* icount = reinterpret_cast<unsigned long long*>(ctx->red.as<int>() + ((n1 + 2) & ~1));
         KRY_CUDA(cudaMemsetAsync(icount, 0, sizeof(unsigned long long), ctx->stream));

@@ -35,6 +35,23 @@ struct DFAcc {
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// (hi, lo) += (ohi, olo), double-float.
+__device__ __forceinline__ void df_add(float& hi, float& lo, float ohi, float olo) {
+    float s, t;
+    two_sum(hi, ohi, s, t);
+    hi = s;
+    lo = __fadd_rn(__fadd_rn(lo, olo), t);
+}
+
+// Sum of (hi, lo) over a warp's lanes in a fixed tree order; valid in lane 0.
+__device__ __forceinline__ void df_warp_sum(float& hi, float& lo) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_down_sync(0xffffffffu, hi, o), l = __shfl_down_sync(0xffffffffu, lo, o);
+        df_add(hi, lo, h, l);
+    }
+}
+
 // Dot-product accumulator of the vector precision: double-float for FP32
 // vectors, plain FP64 FMAs for FP64 vectors.
 template <typename T>

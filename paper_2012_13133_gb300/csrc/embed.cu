@@ -35,8 +35,8 @@ void init_twiddles(kry_ctx* ctx) {
     ctx->tw32.ensure(KRY_TWN * sizeof(float2));
     k_twiddles<<<(KRY_TWN + 255) / 256, 256, 0, ctx->stream>>>(ctx->tw64.as<double2>(), ctx->tw32.as<float2>());
     KRY_CHECK_LAUNCH();
-    ctx->twt32.ensure((size_t)kspec::TWT_ROWS * 16 * sizeof(float2));
-    kspec::fill_stage_twiddles(ctx->twt32.as<float2>(), ctx->stream);
+    ctx->spec_tab.ensure((size_t)kspec::TABLE_WORDS * sizeof(float4));
+    kspec::fill_tables(ctx->spec_tab.as<float4>(), ctx->stream);
 }
 
 // ------------------------------------------------------------------ lag covariance
@@ -386,11 +386,10 @@ void bccb_logdet(kry_ctx* ctx, const kry_cov& cov, bool deriv, double* logdet, d
 }
 
 // lamT[j][k] = lam[k][j] * scale (FP64 and optionally FP32), 32 x 32 tiles.
-// With t32p != NULL also the column-permuted FP32 copy: row k = t + m M1/16 of
-// column j goes to t32p[j M1 + 16 t + m].
+// With t32p != NULL also the column-permuted FP32 copy (kspec::lam_slot).
 __global__ void k_transpose_scale(const double* __restrict__ lam, int M1, int M2, double scale,
-                                  double* __restrict__ t64, float* __restrict__ t32, float* __restrict__ t32p) {
-    const int lt = M1 >> 4;
+                                  double* __restrict__ t64, float* __restrict__ t32, float* __restrict__ t32p,
+                                  int lt) {
     __shared__ double tile[32][33];
     const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -404,7 +403,7 @@ __global__ void k_transpose_scale(const double* __restrict__ lam, int M1, int M2
             const double v = tile[threadIdx.x][r] * scale;
             t64[(int64_t)j * M1 + k] = v;
             if (t32) t32[(int64_t)j * M1 + k] = (float)v;
-            if (t32p) t32p[(int64_t)j * M1 + (k % lt) * 16 + k / lt] = (float)v;
+            if (t32p) t32p[(int64_t)j * M1 + kspec::lam_slot(k, M1, lt)] = (float)v;
         }
     }
 }
@@ -416,7 +415,8 @@ void store_embedding(kry_ctx* ctx, kry_embed* e, int slot) {
     k_transpose_scale<<<grid, blk, 0, ctx->stream>>>(ctx->eig_c.as<double>(), e->M1, e->M2,
                                                      1.0 / ((double)e->M1 * (double)e->M2), e->lam64T + off,
                                                      e->lam32T ? e->lam32T + off : nullptr,
-                                                     e->lam32P ? e->lam32P + off : nullptr);
+                                                     e->lam32P ? e->lam32P + off : nullptr,
+                                                     e->lam32P ? kspec::transform_threads(e->M1) : 0);
     KRY_CHECK_LAUNCH();
 }
 

@@ -36,11 +36,17 @@ int matvec_num_partials(kry_ctx* ctx, const kry_embed* e, bool dbl, int nvec);
 
 namespace {
 
-__global__ void k_full_index(int* __restrict__ rowptr, int* __restrict__ colidx, int n1, int n2) {
+__global__ void k_full_index(int* __restrict__ rowptr, int* __restrict__ colidx, uint2* __restrict__ bits, int n1,
+                             int n2) {
     const int64_t N = (int64_t)n1 * n2;
+    const int wpr = (n2 + 31) / 32;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         colidx[i] = (int)(i % n2);
         if (i % n2 == 0) rowptr[i / n2] = (int)i;
+        if (i % n2 % 32 == 0) {
+            const int left = n2 - (int)(i % n2);
+            bits[i / n2 * wpr + i % n2 / 32] = make_uint2(left >= 32 ? 0xffffffffu : (1u << left) - 1u, (unsigned)i);
+        }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) rowptr[n1] = (int)N;
 }
@@ -52,11 +58,13 @@ struct FullGrid {
     explicit FullGrid(kry_ctx* c) : ctx(c), p_saved(c->p) {
         std::swap(ctx->rowptr, ctx->rowptr_full);
         std::swap(ctx->colidx, ctx->colidx_full);
+        std::swap(ctx->cellbits, ctx->cellbits_full);
         ctx->p = (int64_t)ctx->n1 * ctx->n2;
     }
     ~FullGrid() {
         std::swap(ctx->rowptr, ctx->rowptr_full);
         std::swap(ctx->colidx, ctx->colidx_full);
+        std::swap(ctx->cellbits, ctx->cellbits_full);
         ctx->p = p_saved;
     }
 };
@@ -223,15 +231,7 @@ void genhybr_t(kry_ctx* ctx, const kry_cov& cov, const double* b, int k, bool re
     KRY_REQUIRE(N <= 4096 * 4096, KRY_EUNSUPPORTED, "grid too large for the whole-grid matvec");
     // whole-grid index lists (built once per mask)
     KRY_REQUIRE(k >= 1, KRY_EINVAL, "k must be >= 1");
-    if (ctx->rowptr_full.p == nullptr || ctx->full_n1 != n1 || ctx->full_n2 != n2) {
-        ctx->rowptr_full.ensure((size_t)(n1 + 1) * sizeof(int));
-        ctx->colidx_full.ensure((size_t)N * sizeof(int));
-        k_full_index<<<grid_for(N), 256, 0, ctx->stream>>>(ctx->rowptr_full.as<int>(), ctx->colidx_full.as<int>(), n1,
-                                                           n2);
-        KRY_CHECK_LAUNCH();
-        ctx->full_n1 = n1;
-        ctx->full_n2 = n2;
-    }
+    if (ctx->rowptr_full.p == nullptr || ctx->full_n1 != n1 || ctx->full_n2 != n2) build_full_lists(ctx, n1, n2);
     kry_cov corr = cov;
     corr.sigma2 = 1.0;
     corr.tau2 = 0.0;
@@ -390,6 +390,18 @@ void genhybr_t(kry_ctx* ctx, const kry_cov& cov, const double* b, int k, bool re
 }
 
 }  // namespace
+
+void build_full_lists(kry_ctx* ctx, int n1, int n2) {
+    const int64_t N = (int64_t)n1 * n2;
+    ctx->rowptr_full.ensure((size_t)(n1 + 1) * sizeof(int));
+    ctx->colidx_full.ensure((size_t)N * sizeof(int));
+    ctx->cellbits_full.ensure((size_t)n1 * ((n2 + 31) / 32) * sizeof(uint2));
+    k_full_index<<<grid_for(N), 256, 0, ctx->stream>>>(ctx->rowptr_full.as<int>(), ctx->colidx_full.as<int>(),
+                                                       ctx->cellbits_full.as<uint2>(), n1, n2);
+    KRY_CHECK_LAUNCH();
+    ctx->full_n1 = n1;
+    ctx->full_n2 = n2;
+}
 
 void genhybr_opt(kry_ctx* ctx, const kry_cov& cov, kry_prec prec, bool reorth, const double* b, int k, double* x_out,
                  double* alphas, double* betas, double* z2_out, double* psi2_out, double* pl_out, double* grad,

@@ -132,13 +132,11 @@ struct kry_ctx {
     DevBuf rowptr;   // int32 [n1 + 1]: first observed index of each row
     DevBuf colidx;   // int32 [p]: column of each observed cell
     DevBuf cellidx;  // int32 [p]: row-major cell index of each observed cell
+    DevBuf cellbits; // uint2 [n1][ceil(n2 / 32)]: observation bits of 32 cells, index of the first observed one
 
-    // shared twiddle tables, W[k] = exp(-2 pi i k / KRY_TWN), and the FP32
-    // stage table of the specialised passes (row Ns - 1 + k: W_{16 Ns}^{k m})
-    DevBuf tw32, tw64, twt32;
-    // FP32 matvecs use the length-specialised passes where they apply (the
-    // generic radix-16 passes compute the same transform for the other shapes)
-    bool use_spec = true;
+    // shared twiddle tables, W[k] = exp(-2 pi i k / KRY_TWN), and the tables of
+    // the specialised FP32 passes (kspec::fill_tables)
+    DevBuf tw32, tw64, spec_tab;
 
     // scratch
     DevBuf slab32, slab64;        // FFT intermediates
@@ -151,7 +149,7 @@ struct kry_ctx {
     DevBuf zbuf, gbuf;            // [y, X] and its solve; kriging grid and weights
     DevBuf boot;                  // bootstrap replicates: fields, predictions, right-hand sides, solves
     DevBuf gk;                    // genGK bases and work vectors
-    DevBuf rowptr_full, colidx_full;   // index lists of the whole grid (genGK's and the sites' Sigma matvec)
+    DevBuf rowptr_full, colidx_full, cellbits_full;   // index lists of the whole grid (genGK's and the sites' Sigma matvec)
     int full_n1 = 0, full_n2 = 0;
     // the FFT passes add no nugget (set while the sites' whole-grid Sigma matvec runs)
     bool no_nugget = false;
@@ -200,13 +198,12 @@ struct kry_embed {
     kry_prec prec = KRY_F32;
     cudaStream_t stream = nullptr;   // stream of the creating context (stream-ordered frees)
     // eigenvalues transposed to [M2][M1] (column-pass order) and scaled by
-    // 1 / (M1 M2), FP64 always and FP32 when prec = KRY_F32
+    // 1 / (M1 M2), FP64 always and FP32 (one of the two forms below) when prec = KRY_F32
     double* lam64T = nullptr;
     float* lam32T = nullptr;
-    // FP32 eigenvalues for the length-specialised column pass: the same
-    // [M2][M1] blocks with each column permuted so that the 16 values one
-    // thread multiplies (rows t + m M1/16, m < 16) are contiguous at 16 t + m
-    // (NULL when that pass does not apply)
+    // FP32 eigenvalues for the specialised column pass: the same [M2][M1]
+    // blocks with each column permuted (kspec::lam_slot); lam32T serves torus
+    // sides below 64, which that pass does not cover
     float* lam32P = nullptr;
     double lam_min = 0, lam_max = 0;
     // several covariance settings in one embedding (batched likelihood
@@ -250,6 +247,9 @@ void sample_field(kry_ctx* ctx, const kry_cov& cov, int M1, int M2, const double
 void boot_rhs(kry_ctx* ctx, const double* G, int64_t N, const double* eps, double tau, double* R, int nrep);
 void boot_mse(kry_ctx* ctx, const double* G, const double* H, int64_t N, int nrep, const int64_t* cells,
               int64_t ncell, double* var, int* bad);
+
+// Index lists of the whole n1 x n2 grid (rowptr_full, colidx_full, cellbits_full).
+void build_full_lists(kry_ctx* ctx, int n1, int n2);
 
 // Irregular sites (sites.cu, Sec. 2 Wendland mapping A): build ctx->sites for
 // nsite device coordinate pairs (false if a site lies outside the domain);

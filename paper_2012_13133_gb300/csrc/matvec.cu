@@ -600,22 +600,37 @@ const MvSched& sched_for(kry_ctx* ctx, int M1, int M2, bool dbl, int nvec) {
     return dbl ? ctx->sched64 : ctx->sched32;
 }
 
-// Rows per block (pass A/C) and columns per block (pass B, = slab tile width).
+// Rows per block (pass A/C) and columns per block (pass B; for FP64 also the
+// slab tile width).
 static void sched16(kry_ctx* ctx, int M1, int M2, bool dbl, int nvec, int* G, int* C) {
     const MvSched& want = sched_for(ctx, M1, M2, dbl, nvec);
+    if (!dbl) {
+        // Specialised passes: blocks of 128 threads (four and more per SM, so that one block's
+        // loads run behind another's butterflies), 256 for the longest columns, whose slab rows
+        // would otherwise be read 8 bytes at a time; down to two warps (one for columns) while the
+        // launch has fewer blocks than two per SM (128^2, 4 vectors: 11.0 us, with 128 threads 12).
+        const int ltr = kspec::transform_threads(M2), ltc = kspec::transform_threads(M1);
+        const int np = (nvec + 1) / 2;
+        auto fill = [&](int lt, int th, int least, int64_t transforms) {
+            while (th > least && th > lt && transforms * lt / th < 2 * ctx->num_sms) th /= 2;
+            return std::max(1, th / lt);
+        };
+        const int g = want.g16 > 0 ? want.g16 : fill(ltr, 128, 64, (int64_t)(M1 / 2) * np);
+        const int c = want.c16 > 0 ? want.c16 : fill(ltc, M1 >= 4096 ? 256 : 128, 32, (int64_t)M2 * np);
+        *G = kspec::block_threads(M2, g, 64) / ltr;
+        *C = kspec::block_threads(M1, c, M2) / ltc;
+        return;
+    }
     const size_t lim = (size_t)ctx->max_smem_optin - 1024;   // leave room for static shared memory
-    // the length-specialised FP32 passes run up to 8 transforms per block
-    const int ntmax = (!dbl && ctx->use_spec) ? 8 : 16;
     auto fit = [&](int L, int nt) {
-        nt = std::max(1, std::min(nt, ntmax));
-        while (nt > 1 && (nt * (L >> 4) > (ntmax == 8 ? 1024 : 512) || smem16(L, nt, dbl) > lim)) nt >>= 1;
+        nt = std::max(1, std::min(nt, 16));
+        while (nt > 1 && (nt * (L >> 4) > 512 || smem16(L, nt, dbl) > lim)) nt >>= 1;
         return nt;
     };
     int g = want.g16 > 0 ? want.g16 : std::max(1, 256 / (M2 >> 4));
     int c = want.c16 > 0 ? want.c16 : std::max(1, 512 / (M1 >> 4));
     *G = fit(M2, g);
     *C = std::min(fit(M1, c), M2);
-    if (ntmax == 8) *C = std::min(*C, std::max(1, M2 >> 4));   // specialised pass A/C need C <= M2 / 16
 }
 
 #define KRY_DISPATCH_NT(NTV, ...)                                  \
@@ -639,36 +654,37 @@ static void run_matvec16(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t
     int G, C;
     sched16(ctx, M1, M2, dbl, nvec, &G, &C);
     const int npairs = (nvec + 1) / 2;
-    const T* lamT = dbl ? reinterpret_cast<const T*>(e->lam64T) : reinterpret_cast<const T*>(e->lam32T);
     const int* rowptr = ctx->rowptr.as<int>();
     const int* colidx = ctx->colidx.as<int>();
     const void* tw32 = ctx->tw32.p;
     const void* tw64 = ctx->tw64.p;
     cudaStream_t st = ctx->stream;
+    if constexpr (sizeof(T) == 4) {
+        KRY_REQUIRE(mode == 0 && e->lam32P != nullptr, KRY_EINVAL, "embedding lacks the permuted eigenvalues");
+        kspec::SpecArgs a{};
+        a.vin = vin; a.ld_in = ld_in; a.scale = scale; a.vout = vout; a.ld_out = ld_out;
+        a.nvec = nvec; a.bits = ctx->cellbits.as<uint2>(); a.wpr = (n2 + 31) / 32;
+        a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2; a.G = G; a.C = C;
+        a.logCs = ilog2(std::max(4, C));   // tile rows of at least a 32-byte sector
+        a.slab = slab; a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
+        a.tau2 = tau2; a.tau2v = ctx->no_nugget ? nullptr : e->tau2_dev; a.dots = dots; a.nds = nds;
+        a.twf = ctx->spec_tab.as<float4>();
+        a.twi = a.twf + kspec::TWF_WORDS;
+        a.post = reinterpret_cast<const float2*>(a.twi + kspec::TWI_WORDS);
+        a.skip = skip;
+        for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
+            a.pair0 = pair0;
+            a.np = std::min(ppb, npairs - pair0);
+            KRY_REQUIRE(kspec::launch_a(a, st) && kspec::launch_b(a, st) && kspec::launch_c(a, st),
+                        KRY_EUNSUPPORTED, "no specialised matvec pass for this shape");
+        }
+    } else {
+    const T* lamT = e->lam64T;
     const int psA = pad_shift(M2, G), psB = pad_shift(M1, C);
     const int thrA = G * (M2 >> 4), thrB = C * (M1 >> 4);
     const size_t smA = smem16(M2, G, dbl), smB = smem16(M1, C, dbl);
     const int nbx = (n1 + G - 1) / G;
     const int logC = ilog2(C);
-    if constexpr (sizeof(T) == 4) {
-        if (mode == 0 && ctx->use_spec && kspec::supported(M1, M2, G, C)) {
-            kspec::SpecArgs a{};
-            a.vin = vin; a.ld_in = ld_in; a.scale = scale; a.vout = vout; a.ld_out = ld_out;
-            a.nvec = nvec; a.rowptr = rowptr; a.colidx = colidx;
-            a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2; a.G = G; a.C = C; a.logC = logC;
-            KRY_REQUIRE(e->lam32P != nullptr, KRY_EINVAL, "embedding lacks the permuted eigenvalues");
-            a.slab = slab; a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
-            a.tau2 = tau2; a.tau2v = ctx->no_nugget ? nullptr : e->tau2_dev; a.dots = dots; a.nds = nds;
-            a.twt = ctx->twt32.as<float4>(); a.skip = skip;
-            for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
-                a.pair0 = pair0;
-                a.np = std::min(ppb, npairs - pair0);
-                KRY_REQUIRE(kspec::launch_a(a, st) && kspec::launch_b(a, st) && kspec::launch_c(a, st),
-                            KRY_EUNSUPPORTED, "no specialised matvec pass for this shape");
-            }
-            return;
-        }
-    }
     for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
         const int np = std::min(ppb, npairs - pair0);
         dim3 gA(nbx, np), gB(M2 / C, np);
@@ -706,6 +722,7 @@ static void run_matvec16(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t
             });
         }
     }
+    }
 }
 
 template <typename T>
@@ -735,6 +752,7 @@ static void run_matvec_sites(kry_ctx* ctx, const kry_embed* e, const T* vin, int
         explicit Scope(kry_ctx* x) : c(x), p(x->p) {
             std::swap(c->rowptr, c->rowptr_full);
             std::swap(c->colidx, c->colidx_full);
+            std::swap(c->cellbits, c->cellbits_full);
             c->p = (int64_t)c->n1 * c->n2;
             c->sites.active = false;
             c->no_nugget = true;
@@ -742,6 +760,7 @@ static void run_matvec_sites(kry_ctx* ctx, const kry_embed* e, const T* vin, int
         ~Scope() {
             std::swap(c->rowptr, c->rowptr_full);
             std::swap(c->colidx, c->colidx_full);
+            std::swap(c->cellbits, c->cellbits_full);
             c->p = p;
             c->sites.active = true;
             c->no_nugget = false;
@@ -1117,12 +1136,14 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
     const bool had = ctx->tuned.count(key) > 0;
     const MvSched prev = had ? ctx->tuned[key] : bs;
     if (use16(M1, M2)) {
-        const bool spec = !dbl && ctx->use_spec;
-        const int tmax = spec ? 1024 : 512;
+        auto feasible = [&](int M, int nt, int most) {
+            return dbl ? nt * (M >> 4) <= 512 && smem16(M, nt, dbl) <= lim && nt <= most
+                       : kspec::block_threads(M, nt, most) == nt * kspec::transform_threads(M);
+        };
         for (int g : {1, 2, 4, 8, 16}) {
-            if (g * (M2 >> 4) > tmax || smem16(M2, g, dbl) > lim || (spec && g > 8)) continue;
+            if (!feasible(M2, g, 64)) continue;
             for (int c : {1, 2, 4, 8, 16}) {
-                if (c * (M1 >> 4) > tmax || smem16(M1, c, dbl) > lim || c > M2 || (spec && (c > 8 || c > (M2 >> 4)))) continue;
+                if (!feasible(M1, c, M2)) continue;
                 for (int ppb : ppbs) {
                     MvSched cand = bs;
                     cand.g16 = g;

@@ -1,16 +1,20 @@
 // The three FP32 matvec passes (Sec. 3: K v = A F^-1 (Lambda . F (A^T v)) +
-// tau^2 v on the circulant embedding) specialised for transform length
-// L = 2^B and NT transforms per block; see fftspec.cuh.  Each translation
-// unit mvspec_{a,b,c}.cu instantiates one pass for every supported (B, NT)
+// tau^2 v on the circulant embedding) specialised for torus side L = 2^B and
+// a block of TH threads; see fftspec.cuh for the transforms.  Each translation
+// unit mvspec_{a,b,c}.cu instantiates one pass for every supported (B, TH)
 // and exposes a runtime dispatcher; matvec.cu calls them for FP32 batches.
 //
-// Layouts (identical to the generic radix-16 passes, so the two can be mixed):
+// Layouts:
 //  * slab: per complex pair an n1 x M2 complex intermediate, stored in column
-//    tiles slab[pair][tile][i][c], c < C, tile = column / C;
-//  * lamP: eigenvalues transposed to [M2][M1], scaled by 1 / (M1 M2), each
-//    column permuted so that row t + m L/16 sits at 16 t + m;
-//  * twt: stage twiddle table, row Ns - 1 + k (Ns a power of two <= 512,
-//    k < Ns) holds W_{16 Ns}^{k m}, m = 0..15, W_n = exp(-2 pi i / n).
+//    tiles slab[pair][tile][i][c], c < Cs, tile = column / Cs (Cs even, so the
+//    two columns 2k, 2k + 1 that a row transform produces in its two lanes
+//    are one 16-byte word);
+//  * lamP: eigenvalues per column j at j M1, scaled by 1 / (M1 M2), permuted
+//    so that the values a column-pass thread multiplies are 16-byte words
+//    consecutive over threads (lam_slot);
+//  * bits: per 32 cells of a grid row, the observation bits and the index of
+//    the first observed cell among them, so that a thread finds the vector
+//    index of any cell with one load and a bit count.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -20,264 +24,282 @@
 #include "fftspec.cuh"
 #include "kry_internal.cuh"
 
-#ifndef KRY_KS_MAXREG
-#define KRY_KS_MAXREG 64   // register cap per thread of the specialised passes
-#endif
-
 namespace kspec {
 
-constexpr int tpb(int B, int NT) { return NT * ((1 << B) >> 4); }
-// Minimum resident blocks per SM that caps registers at KRY_KS_MAXREG (at most
-// 32, the SM's block limit; tiny blocks are then capped less tightly).
-constexpr int minb(int B, int NT) {
-    return 65536 / (KRY_KS_MAXREG * tpb(B, NT)) < 1    ? 1
-           : 65536 / (KRY_KS_MAXREG * tpb(B, NT)) > 32 ? 32
-                                                       : 65536 / (KRY_KS_MAXREG * tpb(B, NT));
-}
+// Threads per transform of torus side 2^B, transforms per block of TH threads.
+__host__ __device__ constexpr int lt_of(int B) { return (1 << (B - 1)) / 16; }
+constexpr int nt_of(int B, int TH) { return TH / lt_of(B); }
+// Registers: 64 of a thread's 128 hold the transform: 512 threads per SM.
+// (Measured on the 64-vector 1024^2 call: 96 registers and 640 threads 1195 us
+// against 913 us; 32 values a thread, one shared-memory exchange fewer, but 8
+// warps per SM, 982 us.)
+constexpr int minb(int B, int TH) { return TH >= 512 ? 1 : 512 / TH; }
 
 // Shared-memory bytes of a block.
-constexpr size_t smem_bytes(int B, int NT) {
-    return (size_t)((1 << B) + ((1 << B) >> pad_shift(1 << B, NT))) * NT * sizeof(float2);
+constexpr size_t smem_bytes(int B, int TH) {
+    return (size_t)((1 << (B - 1)) + ((1 << (B - 1)) >> pad_shift(1 << (B - 1)))) * nt_of(B, TH) * 16;
+}
+
+// Offset within a column of M1 eigenvalues of torus row k1 = 2 k + q, k = t +
+// s lt, lt = threads per transform: word (s/2) lt + t holds (s even: q = 0, 1;
+// s odd: q = 0, 1).
+__host__ __device__ __forceinline__ int lam_slot(int k1, int M1, int lt) {
+    const int q = k1 & 1, k = k1 >> 1, t = k & (lt - 1), s = k / lt;
+    return ((s >> 1) * lt + t) * 4 + (s & 1) * 2 + q;
+}
+
+// Vector indices of a thread's E cells j = t + m LT of a row with wpr
+// observation words w, -1 where the cell is not observed (or beyond the row:
+// the bits of a row's last word end at its last cell).  All loads are
+// unconditional, at clamped addresses: behind branches the compiler issues
+// the dependent load chains one after the other (pass A 473 us instead of
+// 209, 64 vectors on 1024^2).
+template <int LT, int E>
+__device__ __forceinline__ void cell_indices(const uint2* __restrict__ w, int wpr, bool live, int t, int (&q)[E]) {
+    uint2 b[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) b[m] = __ldg(w + min((t + m * LT) >> 5, wpr - 1));
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int j = t + m * LT;
+        const unsigned bit = 1u << (j & 31);
+        const bool on = live && (b[m].x & bit) != 0u && (j >> 5) < wpr;
+        q[m] = on ? (int)(b[m].y + __popc(b[m].x & (bit - 1u))) : -1;
+    }
 }
 
 // ---------------------------------------------------------------- pass A
-// Scatter the observed values of NT rows (two real vectors as re/im) into
-// zeroed rows, forward row FFT (half-input first stage: columns >= n2 are
-// zero), store the n1 x M2 slab in column tiles of width C (C <= L/16).
-template <int B, int NT>
-__global__ void __launch_bounds__(tpb(B, NT), minb(B, NT))
+// Row transforms of NT rows: every thread picks its cells' values straight
+// from the observed vectors (two real vectors as re/im; the observed cells of
+// a row are in column order, so neighbouring threads read neighbouring
+// values), forward FFT, columns 2k and 2k + 1 to the slab as one word.
+template <int B, int TH>
+__global__ void __launch_bounds__(TH, minb(B, TH))
     ks_pass_a(const float* __restrict__ vin, int64_t ld, const double* __restrict__ scale, int nvec, int pair0,
-              const int* __restrict__ rowptr, const int* __restrict__ colidx, int n1, int n2, int C, int logC,
-              float2* __restrict__ slab, const float4* __restrict__ twt, const int* __restrict__ skip) {
+              const uint2* __restrict__ bits, int wpr, int n1, int n2, int logCs, float4* __restrict__ slab,
+              const float4* __restrict__ twf, const int* __restrict__ skip) {
     using P = Plan<B>;
-    constexpr int L = P::L, LT = P::LT, PS = pad_shift(L, NT);
+    constexpr int H = P::H, E = P::E, LT = P::LT, NT = nt_of(B, TH), PS = pad_shift(H);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_wait();   // the vectors and skip flags come from the kernel before
-    pdl_launch_dependents();
     const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    StageTw<16> tw1;   // constant tables: their latency lies behind the kernel before
+    load_twiddles<E, P::R0, false>(tw1, twf, t);
+    pdl_wait();        // the vectors and skip flags come from the kernel before
+    pdl_launch_dependents();
     const int row = blockIdx.x * NT + n;
     const int pair = pair0 + blockIdx.y;
     const int va = 2 * pair, vb = 2 * pair + 1;
     const bool has_b = vb < nvec;
     if (skip && skip[va] && (!has_b || skip[vb])) return;   // both columns finished (whole block)
-    float2* sb = reinterpret_cast<float2*>(smem_raw) + n;
-    const float2 zero = make_float2(0.f, 0.f);
-    const int tb = soff<PS, NT>(t);
+    const bool live = row < n1;
+    c2* sb = reinterpret_cast<c2*>(smem_raw) + n;
 
-    // The row's observed cells are loaded into registers first (a row holds at
-    // most n2 <= L/2 = 8 L/16 of them, so a fixed-trip predicated loop covers
-    // it), and their latency overlaps the zero fill.
-    int col[8];
-    float2 val[8];
-    if (row < n1) {
+    float2 x[E];
+    {
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
-        const int q0 = rowptr[row] + t, q1 = rowptr[row + 1];
         const float* pa = vin + (int64_t)va * ld;
-        const float* pb = vin + (int64_t)vb * ld;
+        const float* pb = has_b ? vin + (int64_t)vb * ld : pa;
+        int q[E];
+        cell_indices<LT, E>(bits + (int64_t)min(row, n1 - 1) * wpr, wpr, live, t, q);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int q = q0 + i * LT;
-            col[i] = q < q1 ? colidx[q] : -1;
-            val[i] = q < q1 ? make_float2(pa[q] * sa, has_b ? pb[q] * sbv : 0.f) : zero;
-        }
-    } else {
+        for (int m = 0; m < E; ++m) x[m] = make_float2(pa[max(q[m], 0)], pb[max(q[m], 0)]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) col[i] = -1;
+        for (int m = 0; m < E; ++m)
+            x[m] = make_float2(q[m] >= 0 ? x[m].x * sa : 0.f, q[m] >= 0 && has_b ? x[m].y * sbv : 0.f);
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i)   // positions t + i L/16 cover [0, L/2), which holds [0, n2)
-        if (t + i * LT < n2) sb[tb + soff<PS, NT>(i * LT)] = zero;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (col[i] >= 0) sb[soff<PS, NT>(col[i])] = val[i];
-    __syncthreads();
-
-    // global store of output position p = t + c (c a multiple of L/16 >= C)
-    const int64_t tstride = (int64_t)n1 * C;
-    float2* out = slab + (int64_t)blockIdx.y * n1 * (int64_t)(L) + (int64_t)row * C +
-                  (int64_t)(t >> logC) * tstride + (t & (C - 1));
-    const int64_t gstep = (int64_t)(LT >> logC) * tstride;
-    const bool live = row < n1;
-
-    auto ld0 = [&](int c) { return (t + c < n2) ? sb[tb + soff<PS, NT>(c)] : zero; };
+    const int tb = soff<PS, NT>(t);
     auto lds = [&](int c) { return sb[tb + soff<PS, NT>(c)]; };
-    auto sts = [&](int bo, int c, float2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
-    auto stg = [&](int, int c, float2 z) {
-        if (live) out[(c / LT) * gstep] = z;
-    };
-    float2 v[16];
-    stage<L, P::R0, 1, false, true, false, true, false>(v, t, twt, ld0, sts);
-    __syncthreads();
-    middle_stages<B, 1, false>(v, t, twt, lds, sts);
-    stage<L, 16, LT, false, false, false, false, false>(v, t, twt, lds, stg);
+    auto sts = [&](int bo, int c, c2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
+    first_forward<B>(x, t, sts);
+    c2 v[E];
+    later_stages<B, 1, false>(v, tw1, t, twf, lds, sts);
+    if (!live) return;
+    // word of columns 2k, 2k + 1, k = t + s LT
+    const int logk = logCs - 1;   // words per tile row
+    float4* out = slab + (((int64_t)blockIdx.y * n1) << (B - 1));
+#pragma unroll
+    for (int s = 0; s < E; ++s) {
+        const int k = t + s * LT;
+        const c2 z = v[brev(s, P::LE)];
+        const float2 re = upk(z.r), im = upk(z.i);
+        out[(((int64_t)(k >> logk) * n1 + row) << logk) + (k & ((1 << logk) - 1))] = make_float4(re.x, im.x, re.y, im.y);
+    }
 }
 
 // ---------------------------------------------------------------- pass B
-// Per column (NT columns = one slab tile per block): forward column FFT
-// (half-input: rows >= n1 are zero) ending in registers, multiply by Lambda,
-// inverse column FFT starting from registers, keep rows < n1.
-template <int B, int NT>
-__global__ void __launch_bounds__(tpb(B, NT), minb(B, NT))
-    ks_pass_b(float2* __restrict__ slab, const float* __restrict__ lamP, int n1, int M2,
-              const float4* __restrict__ twt, int pair0, int64_t lam_stride, int vpt, const int* __restrict__ skip,
-              int nvec) {
+// Column transforms of NT columns: forward, multiply by Lambda in registers,
+// inverse, keep rows < n1 (in place in the slab).
+template <int B, int TH>
+__global__ void __launch_bounds__(TH, minb(B, TH))
+    ks_pass_b(float2* __restrict__ slab, const float* __restrict__ lamP, int n1, int M2, int logCs,
+              const float4* __restrict__ twf, const float4* __restrict__ twi, const float2* __restrict__ post, int pair0,
+              int64_t lam_stride, int vpt, const int* __restrict__ skip, int nvec) {
     using P = Plan<B>;
-    constexpr int L = P::L, LT = P::LT, PS = pad_shift(L, NT);
+    constexpr int L = P::L, H = P::H, E = P::E, LT = P::LT, NT = nt_of(B, TH), PS = pad_shift(H);
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    const int col = blockIdx.x * NT + n;
+    // constant tables: their latency lies behind the kernel before
+    StageTw<16> tw1;
+    load_twiddles<E, P::R0, false>(tw1, twf, t);
+    const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
+    const float4* lam = reinterpret_cast<const float4*>(lamP + theta * lam_stride + (int64_t)col * L) + t;
+    const float2* pw = post + (H - 32) + t;
     pdl_wait();   // the slab comes from pass A
     pdl_launch_dependents();
     if (skip) {
         const int va = 2 * (pair0 + (int)blockIdx.y), vb = va + 1;
         if (skip[va] && (vb >= nvec || skip[vb])) return;
     }
-    const int c = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
-    const int tile = blockIdx.x;
-    float2* sb = reinterpret_cast<float2*>(smem_raw) + c;
-    float2* blk = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)tile * n1 * NT + (int64_t)t * NT + c;
-    const float2 zero = make_float2(0.f, 0.f);
+    c2* sb = reinterpret_cast<c2*>(smem_raw) + n;
+    float2* blk = slab + (int64_t)blockIdx.y * n1 * M2 + (((int64_t)(col >> logCs) * n1 + t) << logCs) +
+                  (col & ((1 << logCs) - 1));
     const int tb = soff<PS, NT>(t);
-
-    auto ldg = [&](int cc) { return (t + cc < n1) ? blk[cc * NT] : zero; };
-    auto lds = [&](int cc) { return sb[tb + soff<PS, NT>(cc)]; };
-    auto sts = [&](int bo, int cc, float2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(cc)] = z; };
-    auto none = [&](int, int, float2) {};
-    auto stg = [&](int, int cc, float2 z) {
-        if (t + cc < n1) blk[cc * NT] = z;
-    };
-    float2 v[16];
-    // forward, ending with slot m = row t + m L/16
-    stage<L, P::R0, 1, false, true, false, false, false>(v, t, twt, ldg, sts);
-    __syncthreads();
-    middle_stages<B, 1, false>(v, t, twt, lds, sts);
-    stage<L, 16, LT, false, false, false, true, true>(v, t, twt, lds, none);
-
-    // eigenvalue multiply
-    const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
-    // column-permuted eigenvalues: slot m of thread t at 16 t + m
-    const float4* lam = reinterpret_cast<const float4*>(lamP + theta * lam_stride + (int64_t)(tile * NT + c) * L) + 4 * t;
+    auto lds = [&](int c) { return sb[tb + soff<PS, NT>(c)]; };
+    auto sts = [&](int bo, int c, c2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
+    c2 v[E];
+    {
+        float2 x[E];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 l = __ldg(lam + q);
-        v[4 * q] = make_float2(v[4 * q].x * l.x, v[4 * q].y * l.x);
-        v[4 * q + 1] = make_float2(v[4 * q + 1].x * l.y, v[4 * q + 1].y * l.y);
-        v[4 * q + 2] = make_float2(v[4 * q + 2].x * l.z, v[4 * q + 2].y * l.z);
-        v[4 * q + 3] = make_float2(v[4 * q + 3].x * l.w, v[4 * q + 3].y * l.w);
+        for (int m = 0; m < E; ++m)
+            x[m] = (t + m * LT < n1) ? blk[(int64_t)(m * LT) << logCs] : make_float2(0.f, 0.f);
+        first_forward<B>(x, t, sts);
     }
+    later_stages<B, 1, false>(v, tw1, t, twf, lds, sts);
 
-    // inverse, first stage fed from registers: input position t + c lives in slot c / (L/16)
-    float2 w[16];
+    c2 w[E];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) w[m] = v[m];
-    auto ldr = [&](int cc) { return w[cc / LT]; };
-    stage<L, P::R0, 1, true, false, false, false, false>(v, t, twt, ldr, sts);
-    __syncthreads();
-    middle_stages<B, 1, true>(v, t, twt, lds, sts);
-    stage<L, 16, LT, true, false, true, false, false>(v, t, twt, lds, stg);
+    for (int s = 0; s < E; s += 2) {
+        const float4 l = __ldg(lam + (s >> 1) * LT);
+        const c2 a = v[brev(s, P::LE)], b = v[brev(s + 1, P::LE)];
+        const u64 la = pk(l.x, l.y), lb = pk(l.z, l.w);
+        w[s] = {mul2(a.r, la), mul2(a.i, la)};
+        w[s + 1] = {mul2(b.r, lb), mul2(b.i, lb)};
+    }
+    __syncthreads();   // every read of the forward transform's last stage is done
+    first_inverse<B>(w, t, sts);
+    load_twiddles<E, P::R0, true>(tw1, twi, t);
+    later_stages<B, 1, true>(v, tw1, t, twi, lds, sts);
+#pragma unroll
+    for (int s = 0; s < E; ++s) {
+        if (t + s * LT < n1) {
+            const c2 z = v[brev(s, P::LE)];
+            const float2 re = upk(z.r), im = upk(z.i), f = __ldg(pw + s * LT);
+            blk[(int64_t)(s * LT) << logCs] = make_float2(fmaf(f.x, re.y, fmaf(-f.y, im.y, re.x)),
+                                                          fmaf(f.x, im.y, fmaf(f.y, re.y, im.x)));
+        }
+    }
 }
 
 // ---------------------------------------------------------------- pass C
-// Inverse row FFT of NT slab rows (last stage keeps columns < n2), gather the
-// observed cells, add the nugget, write K v, and (dots != NULL) per-block FP64
-// partials of v . K v.
-template <int B, int NT>
-__global__ void __launch_bounds__(tpb(B, NT), minb(B, NT))
-    ks_pass_c(const float2* __restrict__ slab, const float* __restrict__ vin, int64_t ld_in,
+// Inverse row transforms of NT slab rows; every thread then writes its observed
+// cells of K v straight from registers, adds the nugget and (dots != NULL)
+// accumulates v . K v, one FP64 partial per block.
+template <int B, int TH>
+__global__ void __launch_bounds__(TH, minb(B, TH))
+    ks_pass_c(const float4* __restrict__ slab, const float* __restrict__ vin, int64_t ld_in,
               const double* __restrict__ scale, float* __restrict__ vout, int64_t ld_out, int nvec, int pair0,
-              const int* __restrict__ rowptr, const int* __restrict__ colidx, int n1, int n2, int C, int logC,
-              double tau2, double* __restrict__ dots, int ndot_stride, const float4* __restrict__ twt,
-              const double* __restrict__ tau2v, int vpt, const int* __restrict__ skip) {
+              const uint2* __restrict__ bits, int wpr, int n1, int n2, int logCs, double tau2,
+              double* __restrict__ dots, int ndot_stride, const float4* __restrict__ twi,
+              const float2* __restrict__ post, const double* __restrict__ tau2v, int vpt,
+              const int* __restrict__ skip) {
     using P = Plan<B>;
-    constexpr int L = P::L, LT = P::LT, PS = pad_shift(L, NT);
+    constexpr int H = P::H, E = P::E, LT = P::LT, NT = nt_of(B, TH), PS = pad_shift(H);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[2][32];
+    __shared__ float2 red[2][TH / 32];
+    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    StageTw<16> tw1;   // constant tables: their latency lies behind the kernel before
+    load_twiddles<E, P::R0, true>(tw1, twi, t);
+    const float2* pw = post + (H - 32) + t;
     pdl_wait();   // the slab comes from pass B
     pdl_launch_dependents();
-    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
     const int row = blockIdx.x * NT + n;
     const int pair = pair0 + blockIdx.y;
     const int va = 2 * pair, vb = 2 * pair + 1;
     const bool has_b = vb < nvec;
     if (skip && skip[va] && (!has_b || skip[vb])) return;   // both columns finished (whole block)
-    float2* sb = reinterpret_cast<float2*>(smem_raw) + n;
-    const float2 zero = make_float2(0.f, 0.f);
-    const int tb = soff<PS, NT>(t);
     const bool live = row < n1;
-    const int q0 = live ? rowptr[row] + t : 0, q1 = live ? rowptr[row + 1] : 0;   // read early
-
-    const int64_t tstride = (int64_t)n1 * C;
-    const float2* in = slab + (int64_t)blockIdx.y * n1 * (int64_t)(L) + (int64_t)row * C +
-                       (int64_t)(t >> logC) * tstride + (t & (C - 1));
-    const int64_t gstep = (int64_t)(LT >> logC) * tstride;
-    auto ldg = [&](int c) { return live ? in[(c / LT) * gstep] : zero; };
+    c2* sb = reinterpret_cast<c2*>(smem_raw) + n;
+    const int tb = soff<PS, NT>(t);
     auto lds = [&](int c) { return sb[tb + soff<PS, NT>(c)]; };
-    auto sts = [&](int bo, int c, float2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
-    auto stn = [&](int, int c, float2 z) {
-        if (t + c < n2) sb[tb + soff<PS, NT>(c)] = z;
-    };
-    float2 v[16];
-    stage<L, P::R0, 1, true, false, false, false, false>(v, t, twt, ldg, sts);
-    __syncthreads();
-    middle_stages<B, 1, true>(v, t, twt, lds, sts);
-    stage<L, 16, LT, true, false, true, true, false>(v, t, twt, lds, stn);
-    __syncthreads();
+    auto sts = [&](int bo, int c, c2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
+    c2 v[E];
+    {
+        const int logk = logCs - 1;
+        const float4* in = slab + (((int64_t)blockIdx.y * n1) << (B - 1));
+        c2 w[E];
+#pragma unroll
+        for (int s = 0; s < E; ++s) {
+            const int k = t + s * LT;
+            const float4 f = in[(((int64_t)(k >> logk) * n1 + min(row, n1 - 1)) << logk) + (k & ((1 << logk) - 1))];
+            w[s] = {pk(f.x, f.z), pk(f.y, f.w)};
+        }
+        first_inverse<B>(w, t, sts);
+    }
+    later_stages<B, 1, true>(v, tw1, t, twi, lds, sts);
 
-    kry::DotAcc<float> acc_a, acc_b;
-    if (live) {
+    kry::DFAcc acc_a, acc_b;
+    {
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
         const float t2 = (float)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
         const float* pa = vin + (int64_t)va * ld_in;
-        const float* pb = vin + (int64_t)vb * ld_in;
+        const float* pb = has_b ? vin + (int64_t)vb * ld_in : pa;
         float* oa = vout + (int64_t)va * ld_out;
         float* ob = vout + (int64_t)vb * ld_out;
-        // at most n2 <= 8 L/16 cells per row: fixed-trip predicated loop
+        const uint2* w = bits + (int64_t)min(row, n1 - 1) * wpr;
+        constexpr int CH = 16;   // cells at a time (their indices and inputs are live together)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int q = q0 + i * LT;
-            if (q < q1) {
-                const float2 z = sb[soff<PS, NT>(colidx[q])];
-                const float xa = pa[q] * sa;
-                const float ya = z.x + t2 * xa;
-                oa[q] = ya;
-                acc_a.add_prod(xa, ya);
-                if (has_b) {
-                    const float xb = pb[q] * sbv;
-                    const float yb = z.y + t2 * xb;
-                    ob[q] = yb;
-                    acc_b.add_prod(xb, yb);
+        for (int s0 = 0; s0 < E; s0 += CH) {
+            int q[CH];
+            cell_indices<LT, CH>(w, wpr, live, t + s0 * LT, q);
+            float2 x[CH], y[CH];
+#pragma unroll
+            for (int i = 0; i < CH; ++i) x[i] = make_float2(pa[max(q[i], 0)], pb[max(q[i], 0)]);
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                const c2 z = v[brev(s0 + i, P::LE)];
+                const float2 re = upk(z.r), im = upk(z.i), f = __ldg(pw + (s0 + i) * LT);
+                y[i] = make_float2(fmaf(f.x, re.y, fmaf(-f.y, im.y, re.x)), fmaf(f.x, im.y, fmaf(f.y, re.y, im.x)));
+            }
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                x[i] = make_float2(x[i].x * sa, x[i].y * sbv);
+                y[i] = make_float2(y[i].x + t2 * x[i].x, y[i].y + t2 * x[i].y);
+            }
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                if (q[i] >= 0) oa[q[i]] = y[i].x;
+                if (q[i] >= 0 && has_b) ob[q[i]] = y[i].y;
+            }
+            if (dots) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) {
+                    const bool on = q[i] >= 0;   // what lies in unobserved cells stays out of the sums
+                    acc_a.add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
+                    acc_b.add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
                 }
             }
         }
     }
     if (dots != nullptr) {
-        double da = acc_a.value(), db = acc_b.value();
-        // fixed-order block reduction (rows interleaved across lanes, n fastest)
+        // fixed-order block reduction in double-float: FP64 shuffle trees would
+        // hold the FP64 pipe (one warp instruction per 64 cycles) for longer
+        // than the pass's stores take
+        kry::df_warp_sum(acc_a.hi, acc_a.lo);
+        kry::df_warp_sum(acc_b.hi, acc_b.lo);
         const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        if (blockDim.x >= 32) {
-            for (int o = 16; o > 0; o >>= 1) {
-                da += __shfl_down_sync(0xffffffffu, da, o);
-                db += __shfl_down_sync(0xffffffffu, db, o);
-            }
-            if (lane == 0) {
-                red[0][w] = da;
-                red[1][w] = db;
-            }
-        } else {
-            red[0][threadIdx.x] = da;
-            red[1][threadIdx.x] = db;
+        if (lane == 0) {
+            red[0][w] = make_float2(acc_a.hi, acc_a.lo);
+            red[1][w] = make_float2(acc_b.hi, acc_b.lo);
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double s0 = 0.0, s1 = 0.0;
-            const int nw = (blockDim.x >= 32) ? (blockDim.x >> 5) : blockDim.x;
-            for (int k = 0; k < nw; ++k) {
-                s0 += red[0][k];
-                s1 += red[1][k];
-            }
-            dots[(int64_t)va * ndot_stride + blockIdx.x] = s0;
-            if (has_b) dots[(int64_t)vb * ndot_stride + blockIdx.x] = s1;
+        if (threadIdx.x < 2 && (threadIdx.x == 0 || has_b)) {
+            float hi = 0.f, lo = 0.f;
+#pragma unroll
+            for (int k = 0; k < TH / 32; ++k) kry::df_add(hi, lo, red[threadIdx.x][k].x, red[threadIdx.x][k].y);
+            dots[(int64_t)(threadIdx.x ? vb : va) * ndot_stride + blockIdx.x] = (double)hi + (double)lo;
         }
     }
 }
@@ -292,10 +314,10 @@ struct SpecArgs {
     float* vout;
     int64_t ld_out;
     int nvec, pair0, np;
-    const int* rowptr;
-    const int* colidx;
+    const uint2* bits;
+    int wpr;
     int n1, n2, M1, M2;
-    int G, C, logC;
+    int G, C, logCs;   // rows per block (A, C), columns per block (B), log2 of the slab tile width
     float2* slab;
     const float* lamP;   // column-permuted FP32 eigenvalues (kry_embed::lam32P)
     int64_t lam_stride;
@@ -304,56 +326,67 @@ struct SpecArgs {
     const double* tau2v;
     double* dots;
     int nds;
-    const float4* twt;
+    const float4* twf;
+    const float4* twi;
+    const float2* post;
     const int* skip;
 };
 
-// True if the specialised kernels cover this shape: 64 <= M <= 8192, rows and
-// columns per block in {1, 2, 4, 8} within 1024 threads, slab tile width C
-// at most M2 / 16.
-bool supported(int M1, int M2, int G, int C);
+// Largest block compiled for torus side 2^B.
+constexpr int max_threads(int B) { return B >= 12 ? 512 : B >= 8 ? 256 : 128; }
 
-// Launch pass A, B or C (returns false if the (B, NT) pair is not compiled).
+// Threads per transform of torus side M.
+int transform_threads(int M);
+
+// Threads per block of a pass that puts nt transforms of torus side M in a
+// block: at least a warp, at most max_threads, never more transforms than
+// `most`.
+int block_threads(int M, int nt, int most);
+
+// Launch pass A, B or C (false if the shape is not compiled).
 bool launch_a(const SpecArgs& a, cudaStream_t st);
 bool launch_b(const SpecArgs& a, cudaStream_t st);
 bool launch_c(const SpecArgs& a, cudaStream_t st);
 
-// Stage twiddle table of 1023 rows x 16 complex FP32 values (see above).
-constexpr int TWT_ROWS = 1023;
-void fill_stage_twiddles(float2* twt_dev, cudaStream_t st);
+// Words (16 bytes) of the tables that fill_tables writes: forward twiddles,
+// inverse twiddles, post factors (two per word).
+constexpr int TABLE_WORDS = TWF_WORDS + TWI_WORDS + POST_WORDS / 2;
+void fill_tables(float4* tab_dev, cudaStream_t st);
 
 }  // namespace kspec
 
 namespace kspec {
 
-// Calls f.template run<B, NT>() for a runtime (B, NT) with 6 <= B <= 13,
-// NT in {1, 2, 4, 8} and at most 1024 threads per block; false otherwise.
+// Calls f.template run<B, TH>() for a runtime (B, TH); false otherwise.
+template <int B, int TH, class F>
+bool dispatch_one(const F& f) {
+    if constexpr (lt_of(B) <= TH && TH <= max_threads(B)) return f.template run<B, TH>();
+    return false;
+}
+
 template <int B, class F>
-bool dispatch_nt(int nt, const F& f) {
-    switch (nt) {
-        case 1: return f.template run<B, 1>();
-        case 2: return f.template run<B, 2>();
-        case 4:
-            if constexpr (tpb(B, 4) <= 1024) return f.template run<B, 4>();
-            return false;
-        case 8:
-            if constexpr (tpb(B, 8) <= 1024) return f.template run<B, 8>();
-            return false;
+bool dispatch_th(int th, const F& f) {
+    switch (th) {
+        case 32: return dispatch_one<B, 32>(f);
+        case 64: return dispatch_one<B, 64>(f);
+        case 128: return dispatch_one<B, 128>(f);
+        case 256: return dispatch_one<B, 256>(f);
+        case 512: return dispatch_one<B, 512>(f);
         default: return false;
     }
 }
 
 template <class F>
-bool dispatch(int b, int nt, const F& f) {
+bool dispatch(int b, int th, const F& f) {
     switch (b) {
-        case 6: return dispatch_nt<6>(nt, f);
-        case 7: return dispatch_nt<7>(nt, f);
-        case 8: return dispatch_nt<8>(nt, f);
-        case 9: return dispatch_nt<9>(nt, f);
-        case 10: return dispatch_nt<10>(nt, f);
-        case 11: return dispatch_nt<11>(nt, f);
-        case 12: return dispatch_nt<12>(nt, f);
-        case 13: return dispatch_nt<13>(nt, f);
+        case 6: return dispatch_th<6>(th, f);
+        case 7: return dispatch_th<7>(th, f);
+        case 8: return dispatch_th<8>(th, f);
+        case 9: return dispatch_th<9>(th, f);
+        case 10: return dispatch_th<10>(th, f);
+        case 11: return dispatch_th<11>(th, f);
+        case 12: return dispatch_th<12>(th, f);
+        case 13: return dispatch_th<13>(th, f);
         default: return false;
     }
 }

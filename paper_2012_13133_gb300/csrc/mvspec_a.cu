@@ -1,30 +1,63 @@
 // Pass A of the specialised FP32 matvec (mvspec.cuh) for every supported
-// (log2 M2, rows per block), the shape check and the stage twiddle table.
+// (log2 M2, threads per block), the block sizes and the twiddle tables.
 #include "kry_internal.cuh"
 #include "mvspec.cuh"
 
 namespace kspec {
 
-bool supported(int M1, int M2, int G, int C) {
-    auto pow2 = [](int x) { return x > 0 && (x & (x - 1)) == 0; };
-    if (!pow2(M1) || !pow2(M2) || M1 < 64 || M2 < 64 || M1 > 8192 || M2 > 8192) return false;
-    if (!pow2(G) || !pow2(C) || G > 8 || C > 8 || C > (M2 >> 4)) return false;
-    return G * (M2 >> 4) <= 1024 && C * (M1 >> 4) <= 1024;
+int transform_threads(int M) { return lt_of(ilog2i(M)); }
+
+int block_threads(int M, int nt, int most) {
+    const int lt = transform_threads(M), cap = max_threads(ilog2i(M));
+    int th = lt;
+    while (th < lt * nt && 2 * th <= cap && 2 * (th / lt) <= most) th *= 2;
+    while (th < 32) th *= 2;
+    return th;
 }
 
-__global__ void k_stage_twiddles(float2* __restrict__ twt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= TWT_ROWS * 16) return;
-    const int row = i >> 4, m = i & 15;
-    const int ns = 1 << (31 - __clz(row + 1));   // row = ns - 1 + k, k < ns
-    const int k = row + 1 - ns;
+// cos of the twiddle angle with its zero replaced by +-2^-27 (fftspec.cuh) and the tangent that goes with it.
+__device__ __forceinline__ float2 cos_tan(double turns) {
     double s, c;
-    sincospi(-2.0 * (double)(k * m) / (16.0 * (double)ns), &s, &c);
-    twt[i] = make_float2((float)c, (float)s);
+    sincospi(2.0 * turns, &s, &c);
+    float cf = (float)c;
+    if (fabsf(cf) < 7.450580596923828e-9f) cf = c < 0.0 ? -7.450580596923828e-9f : 7.450580596923828e-9f;
+    return make_float2(cf, (float)(s / (double)cf));
 }
 
-void fill_stage_twiddles(float2* twt_dev, cudaStream_t st) {
-    k_stage_twiddles<<<(TWT_ROWS * 16 + 255) / 256, 256, 0, st>>>(twt_dev);
+// Angle (in turns) of entry e = s + 2^{l-2} of level l at stride ns, frequency k.
+__device__ __forceinline__ double entry_turns(int e, int ns, double k) {
+    const int l = e == 0 ? 1 : 2 + (31 - __clz(e));
+    return (k / ns + (e - tw_base(l))) / (double)(1 << l);
+}
+
+__global__ void k_tables(float4* __restrict__ tab) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < TWF_WORDS) {
+        const int ns = 1 << (31 - __clz(i / 8 + 2));   // sections of 8 ns words from 8 (ns - 2)
+        const int r = i - 8 * (ns - 2), e = r / ns, k = r - e * ns;
+        const float2 a = cos_tan(entry_turns(e, ns, k)), b = cos_tan(entry_turns(e, ns, k + 0.5));
+        tab[i] = make_float4(a.x, b.x, a.y, b.y);
+    } else if (i < TWF_WORDS + TWI_WORDS) {
+        const int w = i - TWF_WORDS;
+        const int ns = 1 << (31 - __clz(w / 4 + 2));
+        const int r = w - 4 * (ns - 2), e = r / ns, k = r - e * ns;
+        const float2 a = cos_tan(entry_turns(2 * e, ns, k)), b = cos_tan(entry_turns(2 * e + 1, ns, k));
+        tab[i] = make_float4(a.x, a.y, b.x, b.y);
+    } else if (i < TABLE_WORDS) {
+        float2 f[2];
+        for (int q = 0; q < 2; ++q) {
+            const int w = 2 * (i - TWF_WORDS - TWI_WORDS) + q;   // sections of h words from h - 32
+            const int h = 1 << (31 - __clz(w + 32));
+            double s, c;
+            sincospi((double)(w + 32 - h) / (double)h, &s, &c);
+            f[q] = make_float2((float)c, (float)s);
+        }
+        tab[i] = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+    }
+}
+
+void fill_tables(float4* tab_dev, cudaStream_t st) {
+    k_tables<<<(TABLE_WORDS + 255) / 256, 256, 0, st>>>(tab_dev);
     KRY_CHECK_LAUNCH();
 }
 
@@ -32,18 +65,19 @@ namespace {
 struct RunA {
     const SpecArgs& a;
     cudaStream_t st;
-    template <int B, int NT>
+    template <int B, int TH>
     bool run() const {
-        auto k = ks_pass_a<B, NT>;
+        constexpr int NT = nt_of(B, TH);
+        auto k = ks_pass_a<B, TH>;
         KRY_ALLOW_MAX_SMEM(k);
         dim3 grid((a.n1 + NT - 1) / NT, a.np);
-        launch_pdl(k, grid, dim3(tpb(B, NT)), smem_bytes(B, NT), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0,
-                   a.rowptr, a.colidx, a.n1, a.n2, a.C, a.logC, a.slab, a.twt, a.skip);
+        launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0, a.bits, a.wpr,
+                   a.n1, a.n2, a.logCs, reinterpret_cast<float4*>(a.slab), a.twf, a.skip);
         return true;
     }
 };
 }  // namespace
 
-bool launch_a(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M2), a.G, RunA{a, st}); }
+bool launch_a(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M2), a.G * transform_threads(a.M2), RunA{a, st}); }
 
 }  // namespace kspec

@@ -1,5 +1,5 @@
 // Pass B of the specialised FP32 matvec (mvspec.cuh) for every supported
-// (log2 M1, columns per block).
+// (log2 M1, threads per block).
 #include "kry_internal.cuh"
 #include "mvspec.cuh"
 
@@ -9,18 +9,18 @@ namespace {
 struct RunB {
     const SpecArgs& a;
     cudaStream_t st;
-    template <int B, int NT>
+    template <int B, int TH>
     bool run() const {
-        auto k = ks_pass_b<B, NT>;
+        auto k = ks_pass_b<B, TH>;
         KRY_ALLOW_MAX_SMEM(k);
-        dim3 grid(a.M2 / NT, a.np);
-        launch_pdl(k, grid, dim3(tpb(B, NT)), smem_bytes(B, NT), st, a.slab, a.lamP, a.n1, a.M2, a.twt, a.pair0, a.lam_stride,
-                                                       a.vpt, a.skip, a.nvec);
+        dim3 grid(a.M2 / nt_of(B, TH), a.np);
+        launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, a.slab, a.lamP, a.n1, a.M2, a.logCs, a.twf, a.twi, a.post,
+                   a.pair0, a.lam_stride, a.vpt, a.skip, a.nvec);
         return true;
     }
 };
 }  // namespace
 
-bool launch_b(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M1), a.C, RunB{a, st}); }
+bool launch_b(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M1), a.C * transform_threads(a.M1), RunB{a, st}); }
 
 }  // namespace kspec

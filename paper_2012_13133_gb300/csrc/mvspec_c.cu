@@ -1,5 +1,5 @@
 // Pass C of the specialised FP32 matvec (mvspec.cuh) for every supported
-// (log2 M2, rows per block).
+// (log2 M2, threads per block).
 #include "kry_internal.cuh"
 #include "mvspec.cuh"
 
@@ -9,19 +9,20 @@ namespace {
 struct RunC {
     const SpecArgs& a;
     cudaStream_t st;
-    template <int B, int NT>
+    template <int B, int TH>
     bool run() const {
-        auto k = ks_pass_c<B, NT>;
+        constexpr int NT = nt_of(B, TH);
+        auto k = ks_pass_c<B, TH>;
         KRY_ALLOW_MAX_SMEM(k);
         dim3 grid((a.n1 + NT - 1) / NT, a.np);
-        launch_pdl(k, grid, dim3(tpb(B, NT)), smem_bytes(B, NT), st, a.slab, a.vin, a.ld_in, a.scale, a.vout, a.ld_out, a.nvec,
-                                                       a.pair0, a.rowptr, a.colidx, a.n1, a.n2, a.C, a.logC, a.tau2,
-                                                       a.dots, a.nds, a.twt, a.tau2v, a.vpt, a.skip);
+        launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, reinterpret_cast<const float4*>(a.slab), a.vin, a.ld_in,
+                   a.scale, a.vout, a.ld_out, a.nvec, a.pair0, a.bits, a.wpr, a.n1, a.n2, a.logCs, a.tau2, a.dots,
+                   a.nds, a.twi, a.post, a.tau2v, a.vpt, a.skip);
         return true;
     }
 };
 }  // namespace
 
-bool launch_c(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M2), a.G, RunC{a, st}); }
+bool launch_c(const SpecArgs& a, cudaStream_t st) { return dispatch(ilog2i(a.M2), a.G * transform_threads(a.M2), RunC{a, st}); }
 
 }  // namespace kspec

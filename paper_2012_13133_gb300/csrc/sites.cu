@@ -172,15 +172,6 @@ __global__ void k_cell_sort(const int* __restrict__ cellptr, int64_t N, int* __r
     }
 }
 
-__global__ void k_full_lists(int* __restrict__ rowptr, int* __restrict__ colidx, int n1, int n2) {
-    const int64_t N = (int64_t)n1 * n2;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        colidx[i] = (int)(i % n2);
-        if (i % n2 == 0) rowptr[i / n2] = (int)i;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) rowptr[n1] = (int)N;
-}
-
 // Step 1: grid[v][c] = scale[v] * sum over the entries of cell c of w * vin[v][site].
 template <typename T>
 __global__ void k_site_scatter(const int* __restrict__ cellptr, const int* __restrict__ ent_site,
@@ -327,12 +318,7 @@ bool build_sites(kry_ctx* ctx, int n1, int n2, double dx1, double dx2, const dou
                                              S.ent_w32.as<float>());
     KRY_CHECK_LAUNCH();
     // whole-grid index lists of the FFT passes (step 2)
-    ctx->rowptr_full.ensure((size_t)(n1 + 1) * sizeof(int));
-    ctx->colidx_full.ensure((size_t)N * sizeof(int));
-    k_full_lists<<<grid_for(N), 256, 0, st>>>(ctx->rowptr_full.as<int>(), ctx->colidx_full.as<int>(), n1, n2);
-    KRY_CHECK_LAUNCH();
-    ctx->full_n1 = n1;
-    ctx->full_n2 = n2;
+    build_full_lists(ctx, n1, n2);
     KRY_CUDA(cudaStreamSynchronize(st));
     return true;
 }
