@@ -44,12 +44,12 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 // Vector v holds Rademacher probe (v mod nprobe): every covariance setting of a
 // batched search sees the same probes.
 template <typename T>
-__global__ void k_probes(T* __restrict__ W, int64_t p, int nprobe, uint64_t seed) {
+__global__ void k_probes(T* __restrict__ W, int64_t p, int64_t ld, int nprobe, uint64_t seed) {
     const int v = blockIdx.y;
     const uint64_t k = (uint64_t)(v % nprobe);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ld; i += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t key = seed ^ ((k << 32) | (uint64_t)i);
-        W[(int64_t)v * p + i] = (splitmix64(key) >> 63) ? (T)-1 : (T)1;
+        W[(int64_t)v * ld + i] = i >= p ? (T)0 : (splitmix64(key) >> 63) ? (T)-1 : (T)1;
     }
 }
 
@@ -229,25 +229,74 @@ __device__ __forceinline__ void store_vec(T* __restrict__ dst, const T (&in)[VW]
     }
 }
 
-// VW elements of the reorthogonalisation store as T: the store is T itself,
-// or FP16 (VW = 4: one 8-byte access).
-template <typename T, typename Sq, int VW>
-__device__ __forceinline__ void load_as(const Sq* __restrict__ src, T (&out)[VW]) {
-    if constexpr (std::is_same<Sq, T>::value) {
-        load_vec<T, VW>(src, out);
-    } else if constexpr (VW == 4) {
-        const uint2 q = *reinterpret_cast<const uint2*>(src);
-        __half2 h[2];
-        memcpy(h, &q, 8);
-        const float2 a = __half22float2(h[0]), b = __half22float2(h[1]);
-        out[0] = (T)a.x;
-        out[1] = (T)a.y;
-        out[2] = (T)b.x;
-        out[3] = (T)b.y;
-    } else {
+// Block sum of a running dot product in a fixed order (valid in thread 0):
+// double-float through FP32 shuffles for FP32 vectors, FP64 for FP64 ones.  A
+// warp's FP64 instruction holds its scheduler's FP64 pipe for 64 cycles on
+// GB300, so an FP64 shuffle tree in every block of a streaming kernel costs
+// more than the streaming (k_lanczos_update, 32 vectors of 183,501 values: 31
+// us, now 17.5 us with the FP16 store that took another 11).
+__device__ __forceinline__ double block_total(const DotAcc<float>& acc) {
+    __shared__ float2 red[32];
+    float hi = acc.a.hi, lo = acc.a.lo;
+    df_warp_sum(hi, lo);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(hi, lo);
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) df_add(hi, lo, red[w].x, red[w].y);
+    return (double)hi + (double)lo;
+}
+__device__ __forceinline__ double block_total(const DotAcc<double>& acc) {
+    __shared__ double red[32];
+    double v = acc.s;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v += red[w];
+    return v;
+}
+
+// Eight consecutive values through 16-byte accesses (the caller guarantees the
+// alignment), FP16 ones as FP32.
+__device__ __forceinline__ void load8(const float* __restrict__ src, float (&out)[8]) {
+    const float4 a = reinterpret_cast<const float4*>(src)[0], b = reinterpret_cast<const float4*>(src)[1];
+    out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
+    out[4] = b.x; out[5] = b.y; out[6] = b.z; out[7] = b.w;
+}
+__device__ __forceinline__ void load8(const __half* __restrict__ src, float (&out)[8]) {
+    const uint4 q = *reinterpret_cast<const uint4*>(src);
+    __half2 h[4];
+    memcpy(h, &q, 16);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) out[e] = (T)__half2float(src[e]);
+    for (int e = 0; e < 4; ++e) {
+        const float2 f = __half22float2(h[e]);
+        out[2 * e] = f.x;
+        out[2 * e + 1] = f.y;
     }
+}
+__device__ __forceinline__ void load8(const double* __restrict__ src, double (&out)[8]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const double2 d = reinterpret_cast<const double2*>(src)[e];
+        out[2 * e] = d.x;
+        out[2 * e + 1] = d.y;
+    }
+}
+__device__ __forceinline__ void store8(float* __restrict__ dst, const float (&v)[8]) {
+    reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ void store8(double* __restrict__ dst, const double (&v)[8]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) reinterpret_cast<double2*>(dst)[e] = make_double2(v[2 * e], v[2 * e + 1]);
+}
+__device__ __forceinline__ void store8(__half* __restrict__ dst, const float (&v)[8]) {
+    __half2 h[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(v[2 * e], v[2 * e + 1]);
+    uint4 q;
+    memcpy(&q, h, 16);
+    *reinterpret_cast<uint4*>(dst) = q;
 }
 
 // ------------------------------------------------------------------ Lanczos
@@ -266,6 +315,7 @@ struct LanczosState {
     double* coef;     // [nprobe][nsteps] s_i * q_i^T w of the vector being reorthogonalised
     int* flag;        // [nprobe] 1: reorthogonalise the new vector of this step
     int* force;       // [nprobe] 1: the next new vector is reorthogonalised too
+    int* again;       // [nprobe] 1: a flagged vector takes a second Gram-Schmidt pass
     double* pre2;     // [nprobe] ||w||^2 before the Gram-Schmidt pass of a flagged vector
 };
 
@@ -286,49 +336,69 @@ __global__ void k_lanczos_init(LanczosState S, int nprobe, int nsteps, double s0
 // alpha_j = sum of the block partials of q_j^T K q_j (fixed order).
 __global__ void k_lanczos_alpha(LanczosState S, const double* __restrict__ part, int nblk, int nprobe, int nsteps,
                                 int j) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int k = blockIdx.x;   // one block per vector
     const double a = block_sum(part + (int64_t)k * nblk, nblk);
     if (threadIdx.x == 0) S.alpha[(int64_t)k * nsteps + j] = a;
 }
 
+// The Lanczos vectors keep a leading dimension ld that is a multiple of eight
+// and zeros past p (the probes and the zeroed matvec output start them so, and
+// the recurrences keep them), so that every access is 16 bytes wide whatever p
+// is.
+
 // w_next = U - alpha_j s_cur W_cur - beta_{j-1} s_prev W_prev;  partial ||w_next||^2.
-// VW elements per access when every vector start is 16-byte aligned.
-template <typename T, int VW>
+// H (FP32 with reorthogonalisation; else NULL): the current basis vector,
+// normalised and scaled to entries of order one, sqrtp s_cur W_cur, for the
+// FP16 reorthogonalisation store.
+template <typename T>
 __global__ void k_lanczos_update(const T* __restrict__ U, const T* __restrict__ Wc, const T* __restrict__ Wp,
-                                 T* __restrict__ Wn, int64_t p, LanczosState S, int nsteps, int j,
-                                 double* __restrict__ part) {
+                                 T* __restrict__ Wn, int64_t ld, LanczosState S, int nsteps, int j,
+                                 double* __restrict__ part, __half* __restrict__ H, double sqrtp) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int k = blockIdx.y;
-    const double a = S.alpha[(int64_t)k * nsteps + j];
-    const T ca = (T)(a * S.s_cur[k]);
+    const double a = S.alpha[(int64_t)k * nsteps + j], sc = S.s_cur[k];
+    const T ca = (T)(a * sc);
     const T cb = (T)((j > 0 ? S.beta[(int64_t)k * nsteps + j - 1] : 0.0) * S.s_prev[k]);
-    const int64_t off = (int64_t)k * p;
-    const int64_t nv = p / VW;
+    const T ch = (T)(sc * sqrtp);
+    const int64_t off = (int64_t)k * ld;
     DotAcc<T> nrm;
-    for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv; xv += (int64_t)gridDim.x * blockDim.x) {
-        T u[VW], wc[VW], wp[VW];
-        load_vec<T, VW>(U + off + xv * VW, u);
-        load_vec<T, VW>(Wc + off + xv * VW, wc);
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; x < ld; x += (int64_t)gridDim.x * blockDim.x * 8) {
+        T u[8], wc[8], wp[8];
+        load8(U + off + x, u);
+        load8(Wc + off + x, wc);
         // at j = 0 there is no previous vector (its buffer is not initialised)
         if (j > 0) {
-            load_vec<T, VW>(Wp + off + xv * VW, wp);
+            load8(Wp + off + x, wp);
         } else {
 #pragma unroll
-            for (int e = 0; e < VW; ++e) wp[e] = (T)0;
+            for (int e = 0; e < 8; ++e) wp[e] = (T)0;
         }
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
+        for (int e = 0; e < 8; ++e) {
             u[e] = u[e] - ca * wc[e] - cb * wp[e];
             nrm.add_prod(u[e], u[e]);
         }
-        store_vec<T, VW>(Wn + off + xv * VW, u);
+        store8(Wn + off + x, u);
+        if constexpr (sizeof(T) == 4) {
+            if (H) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) wc[e] *= ch;
+                store8(H + off + x, wc);
+            }
+        }
     }
-    double acc[1] = {nrm.value()};
-    block_sum_store<1>(acc, part + (int64_t)k * gridDim.x + blockIdx.x, 0);
+    const double s = block_total(nrm);
+    if (threadIdx.x == 0) part[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
 // beta_j = ||w_next||; early stop when beta_j < 1e-12 |alpha_1|; rescale.
 __global__ void k_lanczos_beta(LanczosState S, const double* __restrict__ part, int nblk, int nprobe, int nsteps,
                                int j) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int k = blockIdx.x;   // one block per vector
     const double s = block_sum(part + (int64_t)k * nblk, nblk);
     if (threadIdx.x != 0) return;
@@ -367,13 +437,60 @@ __global__ void k_lanczos_beta(LanczosState S, const double* __restrict__ part, 
 // on the Krylov space up to O(eps ||K||) (Simon 1984).  Decisions are per
 // vector, on the device, so the launch sequence is fixed and graph-capturable.
 
+// A running sum: double-float (hi, lo) for FP32 vectors, (sum, 0) in FP64.
+template <typename T>
+struct Pair {
+    T hi, lo;
+};
+__device__ __forceinline__ void pair_add(Pair<float>& a, Pair<float> b) { df_add(a.hi, a.lo, b.hi, b.lo); }
+__device__ __forceinline__ void pair_add(Pair<double>& a, Pair<double> b) { a.hi += b.hi; }
+__device__ __forceinline__ double pair_value(Pair<float> a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double pair_value(Pair<double> a) { return a.hi; }
+template <typename T>
+__device__ __forceinline__ Pair<T> pair_xor(Pair<T> a, int o) {
+    Pair<T> b;
+    b.hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
+    b.lo = sizeof(T) == 4 ? __shfl_xor_sync(0xffffffffu, a.lo, o) : (T)0;
+    return b;
+}
+
+// Sums of eight values over a warp: lanes 4a .. 4a + 3 return the sum of v[a].
+// Each of the first three exchanges hands half of the values over, so that it
+// takes 9 exchanges instead of 40.
+template <typename T>
+__device__ __forceinline__ Pair<T> warp_sum8(const T (&v)[8], int lane) {
+    Pair<T> s[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a) s[a] = {v[a], (T)0};
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int a = 0; a < h; ++a) {
+            const Pair<T> keep = up ? s[a + h] : s[a], give = up ? s[a] : s[a + h];
+            s[a] = keep;
+            pair_add(s[a], pair_xor(give, 4 * h));
+        }
+    }
+    pair_add(s[0], pair_xor(s[0], 2));
+    pair_add(s[0], pair_xor(s[0], 1));
+    return s[0];
+}
+
 // Estimates for q_{j+1} from ||w||^2 partials (before any reorthogonalisation);
-// sets flag[k] when w is to be reorthogonalised.
+// sets flag[k] when w is to be reorthogonalised.  One block per vector, one
+// thread per estimate (the recurrence over i < j reads the two previous
+// vectors' estimates only; nsteps <= KRY_MAX_STEPS = FIN_THREADS).
 __global__ void k_pro_omega(LanczosState S, const double* __restrict__ part, int nblk, int nsteps, int j,
                             double eps, double eps_round, double omega_reset) {
-    const int k = blockIdx.x;   // one block per vector
-    const double s = block_sum(part + (int64_t)k * nblk, nblk);
-    if (threadIdx.x != 0) return;
+    pdl_wait();
+    pdl_launch_dependents();
+    __shared__ double sh_s, sh_t[8], sh_w[8];
+    const int k = blockIdx.x, i = threadIdx.x;
+    const double s0 = block_sum(part + (int64_t)k * nblk, nblk);
+    if (i == 0) sh_s = s0;
+    __syncthreads();
+    const double s = sh_s;
     const int64_t ostride = (int64_t)gridDim.x * (nsteps + 1);
     double* on = S.omega + ((j + 1) % 3) * ostride + (int64_t)k * (nsteps + 1);   // omega_{j+1, .}
     const double* oc = S.omega + (j % 3) * ostride + (int64_t)k * (nsteps + 1);   // omega_{j, .}
@@ -382,159 +499,196 @@ __global__ void k_pro_omega(LanczosState S, const double* __restrict__ part, int
     const double* be = S.beta + (int64_t)k * nsteps;
     const double bj = sqrt(s);
     if (S.m_eff[k] < nsteps || !(bj > 0.0)) {   // stopped: nothing to keep orthogonal
-        S.flag[k] = 0;
+        if (i == 0) S.flag[k] = 0;
         return;
     }
     const double aj = al[j];
-    double tnorm = fabs(aj) + bj;
-    for (int i = 0; i < j; ++i) tnorm = fmax(tnorm, fabs(al[i]) + be[i]);
-    double worst = 0.0;
-    for (int i = 0; i < j; ++i) {
+    double tnorm = fabs(aj) + bj, worst = 0.0;
+    if (i < j) {
+        tnorm = fmax(tnorm, fabs(al[i]) + be[i]);
         double t = be[i] * oc[i + 1] + (al[i] - aj) * oc[i] - be[j - 1] * op[i];
         if (i > 0) t += be[i - 1] * oc[i - 1];
         t += copysign(eps_round * (be[i] + bj), t);
-        on[i] = t / bj;
-        worst = fmax(worst, fabs(on[i]));
+        t /= bj;
+        on[i] = t;
+        worst = fabs(t);
     }
-    on[j] = eps_round * tnorm / bj;
-    on[j + 1] = 1.0;
-    worst = fmax(worst, fabs(on[j]));
-    const int f = (S.force[k] || worst > sqrt(eps)) ? 1 : 0;
-    S.flag[k] = f;
-    S.pre2[k] = s;
-    S.force[k] = f && !S.force[k];   // the vector after a reorthogonalised one is reorthogonalised too
-    if (f)
-        for (int i = 0; i <= j; ++i) on[i] = omega_reset;
+    for (int o = 16; o > 0; o >>= 1) {
+        tnorm = fmax(tnorm, __shfl_xor_sync(0xffffffffu, tnorm, o));
+        worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
+    }
+    if ((i & 31) == 0) {
+        sh_t[i >> 5] = tnorm;
+        sh_w[i >> 5] = worst;
+    }
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        tnorm = fmax(tnorm, sh_t[w]);
+        worst = fmax(worst, sh_w[w]);
+    }
+    const double last = eps_round * tnorm / bj;   // omega_{j+1, j}
+    worst = fmax(worst, last);
+    const int force = S.force[k];
+    const int f = (force || worst > sqrt(eps)) ? 1 : 0;
+    __syncthreads();   // force is read by every thread before thread 0 replaces it
+    if (i == 0) {
+        on[j] = f ? omega_reset : last;
+        on[j + 1] = 1.0;
+        S.flag[k] = f;
+        S.pre2[k] = s;
+        S.force[k] = f && !force;   // the vector after a reorthogonalised one is reorthogonalised too
+    }
+    if (f && i < j) on[i] = omega_reset;
 }
 
-// "Twice is enough" (Kahan; Parlett, The Symmetric Eigenvalue Problem, 1980,
-// Sec. 6-9): a flagged vector whose norm fell below 1/sqrt(2) of its norm
-// before the Gram-Schmidt pass lost most of itself to cancellation, and its
-// rounding errors are then large relative to what is left; it stays flagged
-// for a second pass, every other vector is unflagged.
-__global__ void k_reorth_again(LanczosState S, const double* __restrict__ part, int nblk) {
-    const int k = blockIdx.x;   // one block per vector
-    if (!S.flag[k]) return;
-    const double s = block_sum(part + (int64_t)k * nblk, nblk);
-    if (threadIdx.x != 0) return;
-    S.flag[k] = (s < 0.5 * S.pre2[k]) ? 1 : 0;
-    S.pre2[k] = s;
+// Whether vector k takes the Gram-Schmidt pass: its flag in the first pass.  In
+// the second, "twice is enough" (Kahan; Parlett, The Symmetric Eigenvalue
+// Problem, 1980, Sec. 6-9): a flagged vector whose norm fell below 1/sqrt(2) of
+// its norm before the first pass lost most of itself to cancellation, and its
+// rounding errors are then large relative to what is left.  Every block of
+// the vector decides alike from the same partials; block 0 records it for the
+// update that follows.
+__device__ __forceinline__ bool reorth_now(const LanczosState& S, int k, int pass, const double* __restrict__ part,
+                                           int nblk) {
+    const bool first = S.flag[k] != 0;
+    if (pass == 0) return first;
+    if (!first) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) S.again[k] = 0;
+        return false;
+    }
+    __shared__ double s;
+    const double t = block_sum(part + (int64_t)k * nblk, nblk);
+    if (threadIdx.x == 0) s = t;
+    __syncthreads();
+    const bool yes = s < 0.5 * S.pre2[k];
+    if (blockIdx.x == 0 && threadIdx.x == 0) S.again[k] = yes ? 1 : 0;
+    return yes;
 }
 
 // Partial dot products W_i^T w (i = 0..j) of each flagged vector against the
-// basis store Q (T, or FP16 for FP32 vectors), 8 basis vectors per sweep over
-// the block's slice of w, VW elements per access.  Products and per-thread sums
-// are in the vector precision T (a coefficient only needs a few correct digits:
-// it removes a component of size <= sqrt(eps)), the block sums in FP64.  dpart rows are [nvec][nsteps + 8][nblk]: a sweep's rows
-// past j (zeros) stay in the vector's padding.
-template <typename T, typename Sq, int VW>
-__global__ void k_reorth_dots(const Sq* __restrict__ Q, const T* __restrict__ Wn, int nvec, int64_t p, int j,
-                              const int* __restrict__ flag, int nsteps, double* __restrict__ dpart) {
+// basis store Q (T, or FP16 for FP32 vectors).  A block holds its 8192 values
+// of w in registers and sweeps the basis eight vectors at a time, so every
+// thread has 32 independent 16-byte loads in flight; products and the sums of
+// a thread's 32 terms are in the vector precision T (a coefficient only needs
+// a few correct digits: it removes a component of size <= sqrt(eps)), sums
+// across threads in double-float (FP64 for FP64 vectors).  dpart rows are
+// [nvec][nsteps + 8][gridDim.x] (hi, lo) pairs: a sweep's rows past j (zeros)
+// stay in the vector's padding.  What held the pass before: one FP64 shuffle
+// tree of eight values per block and sweep (64 cycles an instruction) for 2 to
+// 6 values a thread, and 2-byte loads where p is odd (32 vectors of 183,501
+// values, 50 steps: 6.4 ms -> 2.1 ms).
+template <typename T, typename Sq>
+__global__ void __launch_bounds__(256) k_reorth_dots(const Sq* __restrict__ Q, const T* __restrict__ Wn, int nvec,
+                                                     int64_t ld, int j, LanczosState S, int pass,
+                                                     const double* __restrict__ part, int nblk, int nsteps,
+                                                     Pair<T>* __restrict__ dpart) {
+    pdl_wait();
+    pdl_launch_dependents();
+    constexpr int NC = sizeof(T) == 4 ? 4 : 1;   // groups of eight values a thread holds
+    __shared__ Pair<T> red[2][8][8];
     const int k = blockIdx.y;
-    if (!flag[k]) return;
-    const T* w = Wn + (int64_t)k * p;
-    const int64_t nv = p / VW;
-    for (int i0 = 0; i0 <= j; i0 += 8) {
-        T acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv;
-             xv += (int64_t)gridDim.x * blockDim.x) {
-            T wv[VW];
-            load_vec<T, VW>(w + xv * VW, wv);
+    if (!reorth_now(S, k, pass, part, nblk)) return;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int64_t vs = (int64_t)nvec * ld;   // distance of consecutive basis vectors
+    for (int64_t base = 0, chunk = 0; base < ld; base += (int64_t)gridDim.x * NC * 2048, ++chunk) {
+        int64_t x[NC];
+        bool in[NC];
+        T w[NC][8];
 #pragma unroll
-            for (int a = 0; a < 8; ++a)
-                if (i0 + a <= j) {
-                    T qv[VW];
-                    load_as<T, Sq, VW>(Q + ((int64_t)(i0 + a) * nvec + k) * p + xv * VW, qv);
+        for (int c = 0; c < NC; ++c) {
+            const int64_t y = base + ((int64_t)blockIdx.x * NC + c) * 2048 + threadIdx.x * 8;
+            in[c] = y < ld;
+            x[c] = (int64_t)k * ld + (in[c] ? y : 0);
+            load8(Wn + x[c], w[c]);
 #pragma unroll
-                    for (int e = 0; e < VW; ++e) acc[a] += qv[e] * wv[e];
+            for (int e = 0; e < 8; ++e) w[c][e] = in[c] ? w[c][e] : (T)0;
+        }
+        for (int i0 = 0, sweep = 0; i0 <= j; i0 += 8, ++sweep) {
+            T acc[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                acc[a] = 0;
+                const Sq* q = Q + (int64_t)min(i0 + a, j) * vs;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    T qv[8];
+                    load8(q + x[c], qv);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) acc[a] += qv[e] * w[c][e];
                 }
-        }
-        double accd[8];
+            }
+            Pair<T> tot = warp_sum8<T>(acc, lane);   // of acc[lane >> 2] over the warp
+            if ((lane & 3) == 0) red[sweep & 1][wp][lane >> 2] = tot;
+            __syncthreads();
+            if (threadIdx.x < 8) {
+                tot = red[sweep & 1][0][threadIdx.x];
 #pragma unroll
-        for (int a = 0; a < 8; ++a) accd[a] = (double)acc[a];
-        block_sum_store<8>(accd, dpart + ((int64_t)k * (nsteps + 8) + i0) * gridDim.x + blockIdx.x, gridDim.x);
-        __syncthreads();
-    }
-}
-
-// coef_i = s_i (q_i^T w) = s_i^2 (W_i^T w) for a store of the unnormalised W_i,
-// or (q_i^T w) / sqrt(p) = (H_i^T w) / p for the FP16 store H_i = sqrt(p) q_i
-// (hscale = 1 / p, else 0), summed over the partials in a fixed order.
-__global__ void k_reorth_coef(LanczosState S, const double* __restrict__ dpart, int nblk, int nsteps, int j,
-                              double hscale) {
-    const int k = blockIdx.x;
-    if (!S.flag[k]) return;
-    for (int i = 0; i <= j; ++i) {
-        const double d = block_sum(dpart + ((int64_t)k * (nsteps + 8) + i) * nblk, nblk);
-        if (threadIdx.x == 0) {
-            const double si = S.s_hist[(int64_t)k * nsteps + i];
-            S.coef[(int64_t)k * nsteps + i] = hscale > 0.0 ? hscale * d : si * si * d;
+                for (int u = 1; u < 8; ++u) pair_add(tot, red[sweep & 1][u][threadIdx.x]);
+                Pair<T>* out = dpart + ((int64_t)k * (nsteps + 8) + i0 + threadIdx.x) * gridDim.x + blockIdx.x;
+                if (i0 + (int)threadIdx.x > j) tot = {(T)0, (T)0};
+                if (chunk) pair_add(tot, *out);
+                *out = tot;
+            }
         }
         __syncthreads();
     }
 }
 
-// H = FP16(sqrt(p) s_k W_k) for every vector k: the new basis vector,
-// normalised and scaled to entries of order one, for the reorthogonalisation
-// store.
-template <int VW>
-__global__ void k_store_half(const float* __restrict__ W, const double* __restrict__ s, double sqrtp,
-                             __half* __restrict__ H, int64_t p) {
+// w -= sum_i coef_i W_i (in the basis precision) for flagged vectors; partial
+// ||w||^2 replaces the update's so that beta_j is the norm after
+// reorthogonalisation.  Every block sums the dot partials itself (one warp per
+// basis vector, fixed order): coef_i = s_i (q_i^T w) = s_i^2 (W_i^T w) for a
+// store of the unnormalised W_i, or (q_i^T w) / sqrt(p) = (H_i^T w) / p for the
+// FP16 store H_i = sqrt(p) q_i (hscale = 1 / p, else 0).
+template <typename T, typename Sq>
+__global__ void __launch_bounds__(256) k_reorth_apply(const Sq* __restrict__ Q, T* __restrict__ Wn, int nvec,
+                                                      int64_t ld, int j, LanczosState S, int pass, int nsteps,
+                                                      const Pair<T>* __restrict__ dpart, int nd, double hscale,
+                                                      double* __restrict__ part) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int k = blockIdx.y;
-    const float sc = (float)(s[k] * sqrtp);
-    const int64_t off = (int64_t)k * p;
-    const int64_t nv = p / VW;
-    for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv; xv += (int64_t)gridDim.x * blockDim.x) {
-        float w[VW];
-        load_vec<float, VW>(W + off + xv * VW, w);
-        if constexpr (VW == 4) {
-            __half2 h[2] = {__floats2half2_rn(sc * w[0], sc * w[1]), __floats2half2_rn(sc * w[2], sc * w[3])};
-            uint2 q;
-            memcpy(&q, h, 8);
-            *reinterpret_cast<uint2*>(H + off + xv * VW) = q;
-        } else {
-#pragma unroll
-            for (int e = 0; e < VW; ++e) H[off + xv * VW + e] = __float2half_rn(sc * w[e]);
-        }
-    }
-}
-
-// w -= sum_i coef_i W_i (in the basis precision) for flagged vectors, VW
-// elements per access; partial ||w||^2 replaces the update's so that beta_j is
-// the norm after reorthogonalisation.
-template <typename T, typename Sq, int VW>
-__global__ void k_reorth_apply(const Sq* __restrict__ Q, T* __restrict__ Wn, int nvec, int64_t p, int j,
-                               LanczosState S, int nsteps, double* __restrict__ part) {
-    const int k = blockIdx.y;
-    if (!S.flag[k]) return;
+    if (pass == 0 ? !S.flag[k] : !S.again[k]) return;
+    __shared__ Pair<T> tot[KRY_MAX_STEPS];
     __shared__ T c[KRY_MAX_STEPS];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) c[i] = (T)S.coef[(int64_t)k * nsteps + i];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    for (int i = wp; i <= j; i += 8) {
+        const Pair<T>* d = dpart + ((int64_t)k * (nsteps + 8) + i) * nd;
+        Pair<T> s = {(T)0, (T)0};
+        for (int b = lane; b < nd; b += 32) pair_add(s, d[b]);
+        for (int o = 16; o > 0; o >>= 1) pair_add(s, pair_xor(s, o));
+        if (lane == 0) tot[i] = s;
+    }
     __syncthreads();
-    T* w = Wn + (int64_t)k * p;
-    const int64_t nv = p / VW;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        const double d = pair_value(tot[i]), si = S.s_hist[(int64_t)k * nsteps + i];
+        c[i] = (T)(hscale > 0.0 ? hscale * d : si * si * d);
+    }
+    __syncthreads();
+    T* w = Wn + (int64_t)k * ld;
     DotAcc<T> nrm;
-    for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv; xv += (int64_t)gridDim.x * blockDim.x) {
-        T proj[VW];
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8; x < ld; x += (int64_t)gridDim.x * blockDim.x * 8) {
+        T proj[8];
 #pragma unroll
-        for (int e = 0; e < VW; ++e) proj[e] = 0;
+        for (int e = 0; e < 8; ++e) proj[e] = 0;
 #pragma unroll 4
         for (int i = 0; i <= j; ++i) {
-            T qv[VW];
-            load_as<T, Sq, VW>(Q + ((int64_t)i * nvec + k) * p + xv * VW, qv);
+            T qv[8];
+            load8(Q + ((int64_t)i * nvec + k) * ld + x, qv);
 #pragma unroll
-            for (int e = 0; e < VW; ++e) proj[e] += c[i] * qv[e];
+            for (int e = 0; e < 8; ++e) proj[e] += c[i] * qv[e];
         }
-        T r[VW];
-        load_vec<T, VW>(w + xv * VW, r);
+        T r[8];
+        load8(w + x, r);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
+        for (int e = 0; e < 8; ++e) {
             r[e] -= proj[e];
             nrm.add_prod(r[e], r[e]);
         }
-        store_vec<T, VW>(w + xv * VW, r);
+        store8(w + x, r);
     }
-    double acc[1] = {nrm.value()};
-    block_sum_store<1>(acc, part + (int64_t)k * gridDim.x + blockIdx.x, 0);
+    const double s = block_total(nrm);
+    if (threadIdx.x == 0) part[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
 // Gauss quadrature of z^T log(K) z from the Lanczos tridiagonal T: sum_j w_j
@@ -751,32 +905,38 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
                            double* per_vec, int vpt, bool reorth) {
     const bool dbl = sizeof(T) == 8;
     const int64_t p = ctx->p;
+    const int64_t ld = (p + 7) & ~(int64_t)7;   // leading dimension of every Lanczos vector (zeros past p)
     const int nblkC = matvec_num_partials(ctx, e, dbl, nvec);
-    const size_t vbytes = (size_t)nvec * p * sizeof(T);
+    const size_t vbytes = (size_t)nvec * ld * sizeof(T);
     ctx->work[0].ensure(vbytes);
     T* U = ctx->work[0].as<T>();
+    if (ld > p)
+        KRY_CUDA(cudaMemset2DAsync(U + p, ld * sizeof(T), 0, (ld - p) * sizeof(T), nvec, ctx->stream));
     T* Q = nullptr;   // FP64 basis store with reorthogonalisation
     T* W[3] = {nullptr, nullptr, nullptr};
     // FP32 with reorthogonalisation: the three-term recurrence runs on three
     // rotating FP32 vectors, and every basis vector is also kept, normalised,
     // in an FP16 store for the Gram-Schmidt passes (half the traffic and memory
-    // of an FP32 store; k_store_half)
+    // of an FP32 store; k_lanczos_update)
     const bool hstore = reorth && !dbl;
     __half* H = nullptr;
     if (reorth && dbl) {
         ctx->work[1].ensure(vbytes * nsteps);
         Q = ctx->work[1].as<T>();
     } else if (hstore) {
-        ctx->work[1].ensure((size_t)nvec * p * sizeof(__half) * nsteps);
+        ctx->work[1].ensure((size_t)nvec * ld * sizeof(__half) * nsteps);
         H = ctx->work[1].as<__half>();
         ctx->work[2].ensure(3 * vbytes);
-        for (int b = 0; b < 3; ++b) W[b] = ctx->work[2].as<T>() + (size_t)b * nvec * p;
+        for (int b = 0; b < 3; ++b) W[b] = ctx->work[2].as<T>() + (size_t)b * nvec * ld;
     } else {
         for (int b = 1; b < 4; ++b) ctx->work[b].ensure(vbytes);
         for (int b = 0; b < 3; ++b) W[b] = ctx->work[b + 1].as<T>();
     }
-    auto basis = [&](int i) -> T* { return Q ? Q + (size_t)i * nvec * p : W[i % 3]; };
-    const int nred = std::max(nblkC, RED_BLOCKS);
+    auto basis = [&](int i) -> T* { return Q ? Q + (size_t)i * nvec * ld : W[i % 3]; };
+    // blocks per vector of the streaming kernels: 16 values a thread and more
+    const int nrb = (int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (ld + 4095) / 4096));
+    const int ndot = (int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (ld + (dbl ? 2047 : 8191)) / (dbl ? 2048 : 8192)));
+    const int nred = std::max(nblkC, nrb);
     ctx->work[4].ensure((size_t)nvec * nred * sizeof(double));
     double* part = ctx->work[4].as<double>();
     const size_t nsc = (size_t)nvec * (2 * nsteps + 4) + nvec;
@@ -789,11 +949,11 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
     S.alpha = sc + 2 * nvec;
     S.beta = S.alpha + (size_t)nvec * nsteps;
     double* res = S.beta + (size_t)nvec * nsteps;
-    ctx->work[5].ensure((size_t)nvec * 3 * sizeof(int));
+    ctx->work[5].ensure((size_t)nvec * 4 * sizeof(int));
     S.m_eff = ctx->work[5].as<int>();
     S.s_hist = S.omega = S.coef = S.pre2 = nullptr;
-    S.flag = S.force = nullptr;
-    double* dpart = nullptr;
+    S.flag = S.force = S.again = nullptr;
+    Pair<T>* dpart = nullptr;
     if (reorth) {
         S.s_hist = sc + nsc;
         S.coef = S.s_hist + (size_t)nvec * nsteps;
@@ -801,8 +961,9 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
         S.pre2 = S.omega + (size_t)3 * nvec * (nsteps + 1);
         S.flag = S.m_eff + nvec;
         S.force = S.flag + nvec;
-        ctx->work[6].ensure((size_t)nvec * (nsteps + 8) * RED_BLOCKS * sizeof(double));
-        dpart = ctx->work[6].as<double>();
+        S.again = S.force + nvec;
+        ctx->work[6].ensure((size_t)nvec * (nsteps + 8) * ndot * sizeof(Pair<T>));
+        dpart = ctx->work[6].as<Pair<T>>();
     }
     const double eps = dbl ? 1.1102230246251565e-16 : 5.9604644775390625e-08;   // unit roundoff of T
     // rounding term of the omega recurrence: the local error of one Lanczos step
@@ -817,85 +978,40 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
     const int tb = 256;
     k_lanczos_init<<<(nvec + tb - 1) / tb, tb, 0, ctx->stream>>>(S, nvec, nsteps, 1.0 / sqrt((double)p));
     KRY_CHECK_LAUNCH();
-    dim3 gp((unsigned)std::min<int64_t>((p + 255) / 256, 1024), nvec);
-    k_probes<T><<<gp, 256, 0, ctx->stream>>>(basis(0), p, nprobe, seed);
+    dim3 gp((unsigned)std::min<int64_t>((ld + 255) / 256, 1024), nvec);
+    k_probes<T><<<gp, 256, 0, ctx->stream>>>(basis(0), p, ld, nprobe, seed);
     KRY_CHECK_LAUNCH();
-    constexpr int VW = 16 / sizeof(T);   // 16-byte accesses when every vector start is 16-byte aligned
-    const dim3 gu(RED_BLOCKS, nvec);
-    const double sqrtp = sqrt((double)p);
-    auto store_half = [&](int i) {   // H_i from basis(i) and its scale s_cur
-        if constexpr (sizeof(T) == 4) {
-            if (p % VW == 0)
-                k_store_half<VW><<<gu, 256, 0, ctx->stream>>>(basis(i), S.s_cur, sqrtp, H + (size_t)i * nvec * p, p);
-            else
-                k_store_half<1><<<gu, 256, 0, ctx->stream>>>(basis(i), S.s_cur, sqrtp, H + (size_t)i * nvec * p, p);
-            KRY_CHECK_LAUNCH();
-        }
-    };
-    // Gram-Schmidt dot products and update against the basis store
-    auto reorth_dots = [&](T* Wn, int j) {
-        if constexpr (sizeof(T) == 4) {
-            if (p % VW == 0)
-                k_reorth_dots<T, __half, VW><<<gu, 256, 0, ctx->stream>>>(H, Wn, nvec, p, j, S.flag, nsteps, dpart);
-            else
-                k_reorth_dots<T, __half, 1><<<gu, 256, 0, ctx->stream>>>(H, Wn, nvec, p, j, S.flag, nsteps, dpart);
-        } else {
-            if (p % VW == 0)
-                k_reorth_dots<T, T, VW><<<gu, 256, 0, ctx->stream>>>(Q, Wn, nvec, p, j, S.flag, nsteps, dpart);
-            else
-                k_reorth_dots<T, T, 1><<<gu, 256, 0, ctx->stream>>>(Q, Wn, nvec, p, j, S.flag, nsteps, dpart);
-        }
-        KRY_CHECK_LAUNCH();
-    };
-    auto reorth_apply = [&](T* Wn, int j) {
-        if constexpr (sizeof(T) == 4) {
-            if (p % VW == 0)
-                k_reorth_apply<T, __half, VW><<<gu, 256, 0, ctx->stream>>>(H, Wn, nvec, p, j, S, nsteps, part);
-            else
-                k_reorth_apply<T, __half, 1><<<gu, 256, 0, ctx->stream>>>(H, Wn, nvec, p, j, S, nsteps, part);
-        } else {
-            if (p % VW == 0)
-                k_reorth_apply<T, T, VW><<<gu, 256, 0, ctx->stream>>>(Q, Wn, nvec, p, j, S, nsteps, part);
-            else
-                k_reorth_apply<T, T, 1><<<gu, 256, 0, ctx->stream>>>(Q, Wn, nvec, p, j, S, nsteps, part);
-        }
-        KRY_CHECK_LAUNCH();
-    };
-    if (hstore) store_half(0);
+    const dim3 gu(nrb, nvec), gd(ndot, nvec);
+    const double sqrtp = sqrt((double)p), hscale = hstore ? 1.0 / (double)p : 0.0;
+    // launches of one step, back to back with programmatic dependent launch
     auto step = [&](int j) {
         cudaStream_t st = ctx->stream;
         T* Wc = basis(j);
         T* Wp = basis(j > 0 ? j - 1 : 0);
-        matvec_ex<T>(ctx, e, Wc, p, S.s_cur, U, p, nvec, part, nblkC, vpt);
-        k_lanczos_alpha<<<nvec, FIN_THREADS, 0, st>>>(S, part, nblkC, nvec, nsteps, j);
-        KRY_CHECK_LAUNCH();
+        matvec_ex<T>(ctx, e, Wc, ld, S.s_cur, U, ld, nvec, part, nblkC, vpt);
+        launch_pdl(k_lanczos_alpha, dim3(nvec), dim3(FIN_THREADS), 0, st, S, part, nblkC, nvec, nsteps, j);
         if (j == nsteps - 1) return;
         T* Wn = basis(j + 1);
-        if (p % VW == 0)
-            k_lanczos_update<T, VW><<<gu, 256, 0, st>>>(U, Wc, Wp, Wn, p, S, nsteps, j, part);
-        else
-            k_lanczos_update<T, 1><<<gu, 256, 0, st>>>(U, Wc, Wp, Wn, p, S, nsteps, j, part);
-        KRY_CHECK_LAUNCH();
+        launch_pdl(k_lanczos_update<T>, gu, dim3(256), 0, st, U, Wc, Wp, Wn, ld, S, nsteps, j, part,
+                   hstore ? H + (size_t)j * nvec * ld : nullptr, sqrtp);
         if (reorth) {
-            k_pro_omega<<<nvec, FIN_THREADS, 0, st>>>(S, part, RED_BLOCKS, nsteps, j, eps, eps_round, omega_reset);
-            KRY_CHECK_LAUNCH();
-            reorth_dots(Wn, j);
-            for (int pass = 0; pass < 2; ++pass) {
-                if (pass == 1) {
-                    // second Gram-Schmidt pass for vectors that lost most of their norm
-                    k_reorth_again<<<nvec, FIN_THREADS, 0, st>>>(S, part, RED_BLOCKS);
-                    KRY_CHECK_LAUNCH();
-                    reorth_dots(Wn, j);
+            launch_pdl(k_pro_omega, dim3(nvec), dim3(FIN_THREADS), 0, st, S, part, nrb, nsteps, j, eps, eps_round,
+                       omega_reset);
+            for (int pass = 0; pass < 2; ++pass) {   // the second for vectors that lost most of their norm
+                if constexpr (sizeof(T) == 4) {
+                    launch_pdl(k_reorth_dots<T, __half>, gd, dim3(256), 0, st, H, Wn, nvec, ld, j, S, pass, part, nrb,
+                               nsteps, dpart);
+                    launch_pdl(k_reorth_apply<T, __half>, gu, dim3(256), 0, st, H, Wn, nvec, ld, j, S, pass, nsteps,
+                               dpart, ndot, hscale, part);
+                } else {
+                    launch_pdl(k_reorth_dots<T, T>, gd, dim3(256), 0, st, Q, Wn, nvec, ld, j, S, pass, part, nrb,
+                               nsteps, dpart);
+                    launch_pdl(k_reorth_apply<T, T>, gu, dim3(256), 0, st, Q, Wn, nvec, ld, j, S, pass, nsteps, dpart,
+                               ndot, hscale, part);
                 }
-                k_reorth_coef<<<nvec, FIN_THREADS, 0, st>>>(S, dpart, RED_BLOCKS, nsteps, j,
-                                                            hstore ? 1.0 / (double)p : 0.0);
-                KRY_CHECK_LAUNCH();
-                reorth_apply(Wn, j);
             }
         }
-        k_lanczos_beta<<<nvec, FIN_THREADS, 0, st>>>(S, part, RED_BLOCKS, nvec, nsteps, j);
-        KRY_CHECK_LAUNCH();
-        if (hstore) store_half(j + 1);
+        launch_pdl(k_lanczos_beta, dim3(nvec), dim3(FIN_THREADS), 0, st, S, part, nrb, nvec, nsteps, j);
     };
     step(0);
     if (nsteps > 1)
