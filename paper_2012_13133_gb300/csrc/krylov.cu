@@ -1080,10 +1080,9 @@ __global__ void k_cg_start(const double* __restrict__ B, int64_t ldb, T* __restr
 
 __global__ void k_cg_init_scalars(CgState S, const double* __restrict__ part, int nblk, int nrhs,
                                   const double* __restrict__ tol) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nrhs) return;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(int64_t)k * nblk + b];
+    const int k = blockIdx.x;   // one block per right-hand side
+    const double s = block_sum(part + (int64_t)k * nblk, nblk);
+    if (threadIdx.x != 0) return;
     S.rr[k] = s;
     S.thr2[k] = tol[k] * tol[k] * s;
     S.done[k] = (s == 0.0 || s <= S.thr2[k]) ? 1 : 0;
@@ -1182,10 +1181,9 @@ static int cg_inner(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t l
     S.ndone = S.iters + nrhs;
 
     dim3 gv(RED_BLOCKS, nrhs);
-    const int tb = 128;
     k_cg_start<T><<<gv, 256, 0, st>>>(B, ldb, X, R, P, p, part);
     KRY_CHECK_LAUNCH();
-    k_cg_init_scalars<<<(nrhs + tb - 1) / tb, tb, 0, st>>>(S, part, RED_BLOCKS, nrhs, tol_dev);
+    k_cg_init_scalars<<<nrhs, FIN_THREADS, 0, st>>>(S, part, RED_BLOCKS, nrhs, tol_dev);
     KRY_CHECK_LAUNCH();
     int* hdone = reinterpret_cast<int*>(ctx->host_pinned);
     int it = 0;
@@ -1232,16 +1230,22 @@ __global__ void k_residual(const double* __restrict__ B, int64_t ldb, const doub
     block_sum_store<2>(acc, part + ((int64_t)k * gridDim.x + blockIdx.x) * 2, 1);
 }
 
+// Lane sums of part[0], part[stride], ... (n values) over a warp in a fixed
+// order; valid in every lane.  (One warp per sum: a single thread's 128
+// dependent FP64 adds took 15 us.)
+__device__ __forceinline__ double warp_sum(const double* __restrict__ part, int n, int stride) {
+    double v = 0.0;
+    for (int b = threadIdx.x & 31; b < n; b += 32) v += part[(int64_t)b * stride];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Column norms from the residual kernel's partials: one warp per sum.
 __global__ void k_norms_final(const double* __restrict__ part, int nblk, int nrhs, double* __restrict__ out) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nrhs) return;
-    double a = 0.0, b = 0.0;
-    for (int j = 0; j < nblk; ++j) {
-        a += part[((int64_t)k * nblk + j) * 2];
-        b += part[((int64_t)k * nblk + j) * 2 + 1];
-    }
-    out[2 * k] = sqrt(a);
-    out[2 * k + 1] = sqrt(b);
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // 2 k + (0: ||r||, 1: ||b||)
+    if (i >= 2 * nrhs) return;
+    const double s = warp_sum(part + (int64_t)(i >> 1) * nblk * 2 + (i & 1), nblk, 2);
+    if ((threadIdx.x & 31) == 0) out[i] = sqrt(s);
 }
 
 __global__ void k_set(double* x, int64_t n, double v) {
@@ -1264,7 +1268,7 @@ static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int
     dim3 gv(RED_BLOCKS, nrhs);
     k_residual<<<gv, 256, 0, st>>>(B, ldb, KX, R, p, part);
     KRY_CHECK_LAUNCH();
-    k_norms_final<<<(nrhs + 127) / 128, 128, 0, st>>>(part, RED_BLOCKS, nrhs, fin);
+    k_norms_final<<<(2 * nrhs + 7) / 8, 256, 0, st>>>(part, RED_BLOCKS, nrhs, fin);
     KRY_CHECK_LAUNCH();
     nrm.resize(2 * nrhs);
     KRY_CUDA(cudaMemcpyAsync(nrm.data(), fin, 2 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1322,15 +1326,19 @@ struct RcgState {
 // blocks.
 static int cg_blocks(int nrhs) { return std::max(8, std::min(304, 1216 / std::max(1, nrhs))); }
 
+// The FP32 vectors of the loop keep a leading dimension ld that is a multiple of
+// eight, with zeros past p, so that every access is 16 bytes wide whatever p is.
+
 // X = 0 (a double-float pair Xh + Xl), R = P = (float) B; partials of ||B||^2
 // (FP64) per column, one per block.
 __global__ void k_rcg_start(const double* __restrict__ B, int64_t ldb, float* __restrict__ Xh, float* __restrict__ Xl,
-                            float* __restrict__ R, float* __restrict__ P, int64_t p, double* __restrict__ part_rr) {
+                            float* __restrict__ R, float* __restrict__ P, int64_t p, int64_t ld,
+                            double* __restrict__ part_rr) {
     const int k = blockIdx.y;
     double acc[1] = {0.0};
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x) {
-        const double b = B[(int64_t)k * ldb + i];
-        const int64_t o = (int64_t)k * p + i;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ld; i += (int64_t)gridDim.x * blockDim.x) {
+        const double b = i < p ? B[(int64_t)k * ldb + i] : 0.0;
+        const int64_t o = (int64_t)k * ld + i;
         Xh[o] = 0.f;
         Xl[o] = 0.f;
         R[o] = (float)b;
@@ -1345,15 +1353,14 @@ __global__ void k_rcg_start(const double* __restrict__ B, int64_t ldb, float* __
 __global__ void k_rcg_init_scalars(RcgState S, const double* __restrict__ part_rr, int nblk,
                                    const double* __restrict__ part_rz, int nrz, int nrhs,
                                    const double* __restrict__ tol) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < nrhs) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += part_rr[(int64_t)k * nblk + b];
-        double g = s;
-        if (part_rz) {
-            g = 0.0;
-            for (int b = 0; b < nrz; ++b) g += part_rz[(int64_t)k * nrz + b];
-        }
+    const int k = blockIdx.x;   // one block per right-hand side
+    const double s = block_sum(part_rr + (int64_t)k * nblk, nblk);
+    double g = s;
+    if (part_rz) {
+        __syncthreads();   // block_sum's shared slots are reused
+        g = block_sum(part_rz + (int64_t)k * nrz, nrz);
+    }
+    if (threadIdx.x == 0) {
         S.gam[k] = g;
         S.rr[k] = s;
         S.rr_ref[k] = s;
@@ -1378,12 +1385,14 @@ __global__ void k_rcg_alpha(RcgState S, const double* __restrict__ part_pq, int 
 }
 
 // X += alpha P in double-float (Xh + Xl, FP32 instructions only), R -= alpha Q
-// (FP32); partials of ||R||^2 in double-float.  VW elements per 16-byte access
-// (the internal vectors are 16-byte aligned when p % 4 == 0).
-template <int VW>
-__global__ void k_rcg_update(float* __restrict__ Xh, float* __restrict__ Xl, float* __restrict__ R,
-                             const float* __restrict__ P, const float* __restrict__ Q, int64_t p, RcgState S,
-                             double* __restrict__ part_rr) {
+// (FP32); partials of ||R||^2 in double-float.  Streaming: five vectors read,
+// three written, from L2 where they fit (4 columns of 524,288 or
+// 152,950 values: 15.8 and 11.6 us with FP64 shuffle trees and, for odd p,
+// scalar accesses; 9 us on average now).
+__global__ void __launch_bounds__(256) k_rcg_update(float* __restrict__ Xh, float* __restrict__ Xl,
+                                                    float* __restrict__ R, const float* __restrict__ P,
+                                                    const float* __restrict__ Q, int64_t ld, RcgState S,
+                                                    double* __restrict__ part_rr) {
     pdl_wait();
     pdl_launch_dependents();
     const int k = blockIdx.y;
@@ -1392,29 +1401,28 @@ __global__ void k_rcg_update(float* __restrict__ Xh, float* __restrict__ Xl, flo
     const float af = (float)a;
     float ahi, alo;
     df_split(a, ahi, alo);
-    const int64_t off = (int64_t)k * p;
-    const int64_t nv = p / VW;
-    DFAcc nrm;
-    for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv; xv += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t o = off + xv * VW;
-        float r[VW], pv[VW], qv[VW], xh[VW], xl[VW];
-        load_vec<float, VW>(R + o, r);
-        load_vec<float, VW>(P + o, pv);
-        load_vec<float, VW>(Q + o, qv);
-        load_vec<float, VW>(Xh + o, xh);
-        load_vec<float, VW>(Xl + o, xl);
+    const int64_t off = (int64_t)k * ld;
+    DotAcc<float> nrm;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; x < ld; x += (int64_t)gridDim.x * blockDim.x * 4) {
+        const int64_t o = off + x;
+        float r[4], pv[4], qv[4], xh[4], xl[4];
+        load_vec<float, 4>(R + o, r);
+        load_vec<float, 4>(P + o, pv);
+        load_vec<float, 4>(Q + o, qv);
+        load_vec<float, 4>(Xh + o, xh);
+        load_vec<float, 4>(Xl + o, xl);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
+        for (int e = 0; e < 4; ++e) {
             df_axpy(xh[e], xl[e], ahi, alo, pv[e]);
             r[e] -= af * qv[e];
             nrm.add_prod(r[e], r[e]);
         }
-        store_vec<float, VW>(Xh + o, xh);
-        store_vec<float, VW>(Xl + o, xl);
-        store_vec<float, VW>(R + o, r);
+        store_vec<float, 4>(Xh + o, xh);
+        store_vec<float, 4>(Xl + o, xl);
+        store_vec<float, 4>(R + o, r);
     }
-    double acc[1] = {nrm.value()};
-    block_sum_store<1>(acc, part_rr + (int64_t)k * gridDim.x + blockIdx.x, 0);
+    const double s = block_total(nrm);
+    if (threadIdx.x == 0) part_rr[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
 // rr' = r^T r from the update's partials and gamma' = r^T z from part_rz (nrz
@@ -1446,45 +1454,44 @@ __global__ void k_rcg_beta(RcgState S, const double* __restrict__ part_rr, int n
 }
 
 // P = Z + beta P (FP32); Z = R without a preconditioner.
-template <int VW>
-__global__ void k_rcg_pupdate(float* __restrict__ P, const float* __restrict__ Z, int64_t p, RcgState S) {
+__global__ void __launch_bounds__(256) k_rcg_pupdate(float* __restrict__ P, const float* __restrict__ Z, int64_t ld,
+                                                     RcgState S) {
     pdl_wait();
     pdl_launch_dependents();
     const int k = blockIdx.y;
     if (S.done[k]) return;
     const float b = (float)S.beta[k];
-    float* Pk = P + (int64_t)k * p;
-    const float* Zk = Z + (int64_t)k * p;
-    const int64_t nv = p / VW;
-    for (int64_t xv = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; xv < nv; xv += (int64_t)gridDim.x * blockDim.x) {
-        float z[VW], pv[VW];
-        load_vec<float, VW>(Zk + xv * VW, z);
-        load_vec<float, VW>(Pk + xv * VW, pv);
+    float* Pk = P + (int64_t)k * ld;
+    const float* Zk = Z + (int64_t)k * ld;
+    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; x < ld; x += (int64_t)gridDim.x * blockDim.x * 4) {
+        float z[4], pv[4];
+        load_vec<float, 4>(Zk + x, z);
+        load_vec<float, 4>(Pk + x, pv);
 #pragma unroll
-        for (int e = 0; e < VW; ++e) pv[e] = z[e] + b * pv[e];
-        store_vec<float, VW>(Pk + xv * VW, pv);
+        for (int e = 0; e < 4; ++e) pv[e] = z[e] + b * pv[e];
+        store_vec<float, 4>(Pk + x, pv);
     }
 }
 
 // X = Xh + Xl in FP64 (the caller's layout, leading dimension ldx).
-__global__ void k_df_to_f64(const float* __restrict__ Xh, const float* __restrict__ Xl, int64_t p,
+__global__ void k_df_to_f64(const float* __restrict__ Xh, const float* __restrict__ Xl, int64_t p, int64_t ld,
                             double* __restrict__ X, int64_t ldx) {
     const int k = blockIdx.y;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x)
-        X[(int64_t)k * ldx + i] = (double)Xh[(int64_t)k * p + i] + (double)Xl[(int64_t)k * p + i];
+        X[(int64_t)k * ldx + i] = (double)Xh[(int64_t)k * ld + i] + (double)Xl[(int64_t)k * ld + i];
 }
 
 // Residual replacement of the running columns of the round: R = (float) R64,
 // rr = rr_ref = ||R64||^2 and, without a preconditioner, gamma = rr (P is
 // kept); done when ||R64|| <= rtol ||B|| or the iteration budget is spent (a
 // non-finite residual also ends the column; the caller reports it).
-__global__ void k_rcg_replace(const double* __restrict__ R64, float* __restrict__ R, int64_t p,
+__global__ void k_rcg_replace(const double* __restrict__ R64, float* __restrict__ R, int64_t p, int64_t ld,
                               const double* __restrict__ norms, RcgState S, int maxit, int precond,
                               const int* __restrict__ sel) {
     const int k = blockIdx.y;
     if (S.done[k] || sel[k]) return;   // only the columns of the round (the others' norms are stale)
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x)
-        R[(int64_t)k * p + i] = (float)R64[(int64_t)k * p + i];
+        R[(int64_t)k * ld + i] = (float)R64[(int64_t)k * p + i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {   // (want is cleared by k_count_done, after every block)
         const double rn = norms[2 * k];
         if (!precond) S.gam[k] = rn * rn;
@@ -1532,7 +1539,8 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
                        const kry_embed* pre) {
     const int64_t p = ctx->p;
     cudaStream_t st = ctx->stream;
-    const size_t vb = (size_t)nrhs * p * sizeof(float);
+    const int64_t ld = (p + 7) & ~(int64_t)7;   // leading dimension of the FP32 vectors (zeros past p)
+    const size_t vb = (size_t)nrhs * ld * sizeof(float);
     ctx->work[7].ensure(vb);
     ctx->work[8].ensure(vb);
     ctx->work[9].ensure(vb);
@@ -1572,23 +1580,26 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     ctx->kxbuf.ensure((size_t)nrhs * p * sizeof(double));
     ctx->work[12].ensure(2 * vb);
     float* Xh = ctx->work[12].as<float>();   // the solution as a double-float pair
-    float* Xl = Xh + (size_t)nrhs * p;
+    float* Xl = Xh + (size_t)nrhs * ld;
 
     dim3 gv(RED_BLOCKS, nrhs);
     dim3 gc(nbc, nrhs);
     const int tbeta = std::max(32, ((nrhs + 31) / 32) * 32);
-    const bool vec = p % 4 == 0;   // 16-byte accesses: every column start is 16-byte aligned
+    if (ld > p) {   // the matvec writes the first p values of Q and Z only
+        KRY_CUDA(cudaMemset2DAsync(Q + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
+        if (pre) KRY_CUDA(cudaMemset2DAsync(Z + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
+    }
     auto to_f64 = [&]() {
-        k_df_to_f64<<<gv, 256, 0, st>>>(Xh, Xl, p, X, ldx);
+        k_df_to_f64<<<gv, 256, 0, st>>>(Xh, Xl, p, ld, X, ldx);
         KRY_CHECK_LAUNCH();
     };
-    k_rcg_start<<<gc, 256, 0, st>>>(B, ldb, Xh, Xl, R, P, p, part_rr);
+    k_rcg_start<<<gc, 256, 0, st>>>(B, ldb, Xh, Xl, R, P, p, ld, part_rr);
     KRY_CHECK_LAUNCH();
-    if (pre) matvec_ex<float>(ctx, pre, R, p, nullptr, Z, p, nrhs, part_rz, nblkC, vpt, nullptr);   // z = M^-1 r
-    k_rcg_init_scalars<<<1, tbeta, 0, st>>>(S, part_rr, nbc, part_rz, nblkC, nrhs, ctx->tolbuf.as<double>());
+    if (pre) matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, nullptr);   // z = M^-1 r
+    k_rcg_init_scalars<<<nrhs, FIN_THREADS, 0, st>>>(S, part_rr, nbc, part_rz, nblkC, nrhs, ctx->tolbuf.as<double>());
     KRY_CHECK_LAUNCH();
     if (pre) {   // p = z (beta = 0)
-        launch_pdl(vec ? k_rcg_pupdate<4> : k_rcg_pupdate<1>, gc, dim3(256), 0, st, P, (const float*)Z, p, S);
+        launch_pdl(k_rcg_pupdate, gc, dim3(256), 0, st, P, (const float*)Z, ld, S);
     }
     int* hflag = reinterpret_cast<int*>(ctx->host_pinned);
     const int poll = 8;
@@ -1601,13 +1612,13 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
         // waits for its predecessor's completion before touching its outputs;
         // columns that have converged are not transformed (pairs of finished
         // columns skip every pass)
-        matvec_ex<float>(ctx, e, P, p, nullptr, Q, p, nrhs, part_pq, nblkC, vpt, S.done);
+        matvec_ex<float>(ctx, e, P, ld, nullptr, Q, ld, nrhs, part_pq, nblkC, vpt, S.done);
         launch_pdl(k_rcg_alpha, dim3(nrhs), dim3(FIN_THREADS), 0, s2, S, part_pq, nblkC);
-        launch_pdl(vec ? k_rcg_update<4> : k_rcg_update<1>, gc, dim3(256), 0, s2, Xh, Xl, R, P, Q, p, S, part_rr);
-        if (pre) matvec_ex<float>(ctx, pre, R, p, nullptr, Z, p, nrhs, part_rz, nblkC, vpt, S.done);
+        launch_pdl(k_rcg_update, gc, dim3(256), 0, s2, Xh, Xl, R, P, Q, ld, S, part_rr);
+        if (pre) matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, S.done);
         launch_pdl(k_rcg_beta, dim3(nrhs), dim3(FIN_THREADS), 0, s2, S, part_rr, nbc, (const double*)part_rz, nblkC,
                    maxit);
-        launch_pdl(vec ? k_rcg_pupdate<4> : k_rcg_pupdate<1>, gc, dim3(256), 0, s2, P, (const float*)Z, p, S);
+        launch_pdl(k_rcg_pupdate, gc, dim3(256), 0, s2, P, (const float*)Z, ld, S);
     };
     // Iterations run in blocks of `poll`.  The first block runs directly (it
     // sizes every buffer); later blocks replay one captured graph.
@@ -1638,10 +1649,10 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
             to_f64();
             true_residual(ctx, e, B, ldb, X, ldx, nrhs, R64, ctx->kxbuf.as<double>(), nrm, vpt, sel);
             double* dn = ctx->red.as<double>() + (size_t)nrhs * RED_BLOCKS * 2;   // device norms
-            k_rcg_replace<<<gc, 256, 0, st>>>(R64, R, p, dn, S, maxit, pre ? 1 : 0, sel);
+            k_rcg_replace<<<gc, 256, 0, st>>>(R64, R, p, ld, dn, S, maxit, pre ? 1 : 0, sel);
             KRY_CHECK_LAUNCH();
             if (pre) {   // z = M^-1 r and gamma = r^T z for the replaced r
-                matvec_ex<float>(ctx, pre, R, p, nullptr, Z, p, nrhs, part_rz, nblkC, vpt, sel);
+                matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, sel);
                 k_rcg_regamma<<<nrhs, FIN_THREADS, 0, st>>>(S, part_rz, nblkC, sel);
                 KRY_CHECK_LAUNCH();
             }
@@ -1722,15 +1733,14 @@ __global__ void k_gram(const double* __restrict__ V, int64_t ldv, const double* 
 // quad = y^T K^-1 y - beta^T X^T K^-1 y; loglik = -1/2 (logdet + quad + p log 2 pi).
 __global__ void k_gls(const double* __restrict__ part, int nblk, int ncov, int64_t p, double logdet,
                       double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int nc = ncov + 1;
-    double G[KRY_MAX_COV + 1][KRY_MAX_COV + 1];
-    for (int a = 0; a < nc; ++a)
-        for (int b = 0; b < nc; ++b) {
-            double s = 0.0;
-            for (int j = 0; j < nblk; ++j) s += part[(int64_t)(a * nc + b) * nblk + j];
-            G[a][b] = s;
-        }
+    __shared__ double G[KRY_MAX_COV + 1][KRY_MAX_COV + 1];
+    for (int i = threadIdx.x >> 5; i < nc * nc; i += blockDim.x >> 5) {   // one warp per entry
+        const double s = warp_sum(part + (int64_t)i * nblk, nblk, 1);
+        if ((threadIdx.x & 31) == 0) G[i / nc][i % nc] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     // symmetrise (V^T K^-1 V is symmetric in exact arithmetic)
     double A[KRY_MAX_COV][KRY_MAX_COV], g[KRY_MAX_COV], L[KRY_MAX_COV][KRY_MAX_COV];
     for (int a = 0; a < ncov; ++a) {
@@ -1783,7 +1793,7 @@ GlsResult gls(kry_ctx* ctx, const double* V, const double* Z, int ncov, double l
     dim3 g(RED_BLOCKS, nc * nc);
     k_gram<<<g, 256, 0, st>>>(V, p, Z, p, p, nc, part);
     KRY_CHECK_LAUNCH();
-    k_gls<<<1, 32, 0, st>>>(part, RED_BLOCKS, ncov, p, logdet, out);
+    k_gls<<<1, 256, 0, st>>>(part, RED_BLOCKS, ncov, p, logdet, out);
     KRY_CHECK_LAUNCH();
     KRY_CUDA(cudaMemcpyAsync(ctx->host_pinned, out, (3 + ncov) * sizeof(double), cudaMemcpyDeviceToHost, st));
     KRY_CUDA(cudaStreamSynchronize(st));
