@@ -448,7 +448,7 @@ kry_status kry_create(kry_ctx** out, int device, void* cuda_stream) {
         KRY_CUDA(cudaDeviceGetAttribute(&ctx->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
         // every scratch buffer is stream-ordered on the context stream; keep freed
         // pool memory cached in this process instead of returning it at each sync
-        DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->tw64, &ctx->spec_tab, &ctx->slab32,
+        DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->spec_tab, &ctx->tab64, &ctx->slab32,
                           &ctx->slab64, &ctx->scal, &ctx->eig_c, &ctx->eig_z, &ctx->eig_d, &ctx->red, &ctx->tolbuf,
                           &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full, &ctx->cellbits_full,
                       &ctx->sites.corner, &ctx->sites.w64, &ctx->sites.w32, &ctx->sites.cellptr, &ctx->sites.ent_site,
@@ -478,7 +478,7 @@ void kry_destroy(kry_ctx* ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     else cudaDeviceSynchronize();
-    DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->tw64, &ctx->spec_tab, &ctx->slab32,
+    DevBuf* bufs[] = {&ctx->rowptr, &ctx->colidx, &ctx->cellidx, &ctx->cellbits, &ctx->tw32, &ctx->spec_tab, &ctx->tab64, &ctx->slab32,
                       &ctx->slab64, &ctx->scal, &ctx->eig_c, &ctx->eig_z, &ctx->eig_d, &ctx->red, &ctx->tolbuf,
                       &ctx->kxbuf, &ctx->cbuf, &ctx->sbuf, &ctx->zbuf, &ctx->gbuf, &ctx->boot, &ctx->gk, &ctx->rowptr_full, &ctx->colidx_full, &ctx->cellbits_full,
                       &ctx->sites.corner, &ctx->sites.w64, &ctx->sites.w32, &ctx->sites.cellptr, &ctx->sites.ent_site,

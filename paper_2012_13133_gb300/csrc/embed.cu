@@ -12,276 +12,398 @@
 #include <algorithm>
 #include <cfloat>
 
-#include "fft.cuh"
+#include "fft64.cuh"
 #include "kry_internal.cuh"
 #include "matern.cuh"
+#include "mv64.cuh"
 #include "mvspec.cuh"
 
 namespace kry {
 
 // ------------------------------------------------------------------ twiddles
 
-__global__ void k_twiddles(double2* tw64, float2* tw32) {
+__global__ void k_twiddles(float2* tw32) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= KRY_TWN) return;
     double s, c;
     sincospi(-2.0 * (double)k / (double)KRY_TWN, &s, &c);
-    tw64[k] = make_double2(c, s);
     tw32[k] = make_float2((float)c, (float)s);
 }
 
 void init_twiddles(kry_ctx* ctx) {
-    ctx->tw64.ensure(KRY_TWN * sizeof(double2));
     ctx->tw32.ensure(KRY_TWN * sizeof(float2));
-    k_twiddles<<<(KRY_TWN + 255) / 256, 256, 0, ctx->stream>>>(ctx->tw64.as<double2>(), ctx->tw32.as<float2>());
+    k_twiddles<<<(KRY_TWN + 255) / 256, 256, 0, ctx->stream>>>(ctx->tw32.as<float2>());
     KRY_CHECK_LAUNCH();
+    ctx->tab64.ensure((size_t)kf64::TW_WORDS * sizeof(double2));
+    kf64::fill_table(ctx->tab64.as<double2>(), ctx->stream);
     ctx->spec_tab.ensure((size_t)kspec::TABLE_WORDS * sizeof(float4));
     kspec::fill_tables(ctx->spec_tab.as<float4>(), ctx->stream);
 }
 
 // ------------------------------------------------------------------ lag covariance
 
+// Covariance parameters of one evaluation, scaled for it: x = s d with s =
+// sqrt(2 nu) / range.
 struct CovDev {
-    double sigma2, inv_range, nu, ca, sa, ratio, dx1, dx2;
+    double sigma2, inv_range, nu, s, ca, sa, ratio, dx1, dx2;
+    int kind;   // 0, 1, 2: nu = 1/2, 3/2, 5/2 (closed forms); 3: any other nu
+    bool even;  // d is even in each lag coordinate by itself
 };
 
-__device__ __forceinline__ double cov_at(const CovDev& p, double l1, double l2) {
-    const double r = kry_scaled_dist(l1 * p.dx1, l2 * p.dx2, p.ca, p.sa, p.ratio, p.inv_range);
-    return p.sigma2 * kry_matern(r, p.nu);
+// Any other nu (Bessel functions), at distance d.
+__device__ __noinline__ double lag_general(const CovDev& p, double d, bool drange) {
+    const double r = d * p.inv_range;
+    if (!drange) return p.sigma2 * kry_matern(r, p.nu);
+    return r <= 0.0 ? 0.0 : p.sigma2 * kry_matern_dr(r, p.nu) * (-r * p.inv_range);
 }
 
-// d/d(range) of sigma^2 rho(d / range): with r = d / range, dr / d(range) = -r / range.
-__device__ __forceinline__ double cov_drange_at(const CovDev& p, double l1, double l2) {
-    const double r = kry_scaled_dist(l1 * p.dx1, l2 * p.dx2, p.ca, p.sa, p.ratio, p.inv_range);
-    if (r <= 0.0) return 0.0;
-    return p.sigma2 * kry_matern_dr(r, p.nu) * (-r * p.inv_range);
+// sigma^2 rho_nu at lag (l1, l2) grid steps (drange: its derivative with respect
+// to the range; with r = d / range, dr / d(range) = -r / range).
+__device__ __forceinline__ double lag_entry(const CovDev& p, double l1, double l2, bool drange) {
+    const double h1 = l1 * p.dx1, h2 = l2 * p.dx2;
+    const double u = p.ca * h1 + p.sa * h2, v = p.ratio * (p.ca * h2 - p.sa * h1);
+    const double d = sqrt(u * u + v * v);
+    if (p.kind == 3) return lag_general(p, d, drange);
+    const double x = d * p.s, e = exp(-x);
+    double f;
+    if (!drange) f = p.kind == 0 ? 1.0 : p.kind == 1 ? 1.0 + x : 1.0 + x + x * x * (1.0 / 3.0);
+    else f = p.inv_range * (p.kind == 0 ? x : p.kind == 1 ? x * x : x * x * (1.0 + x) * (1.0 / 3.0));
+    return p.sigma2 * f * e;
 }
 
-template <bool DRANGE>
-__device__ __forceinline__ double lag_entry(const CovDev& p, double l1, double l2) {
-    return DRANGE ? cov_drange_at(p, l1, l2) : cov_at(p, l1, l2);
-}
-
-// First row of the block-circulant extension of the covariance (DRANGE: of
-// its range derivative) on the M1 x M2 torus.
-template <bool DRANGE = false>
-__global__ void k_lag_cov(double* __restrict__ c, int M1, int M2, CovDev p) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)M1 * M2) return;
-    const int j1 = (int)(idx / M2);
-    const int j2 = (int)(idx - (int64_t)j1 * M2);
-    const int a1 = (2 * j1 <= M1) ? j1 : j1 - M1;
-    const int b1 = (2 * j1 < M1) ? j1 : j1 - M1;
-    const int a2 = (2 * j2 <= M2) ? j2 : j2 - M2;
-    const int b2 = (2 * j2 < M2) ? j2 : j2 - M2;
-    double v;
-    if (a1 == b1 && a2 == b2) {
-        v = lag_entry<DRANGE>(p, a1, a2);
-    } else if (a1 == b1) {
-        v = 0.5 * (lag_entry<DRANGE>(p, a1, a2) + lag_entry<DRANGE>(p, a1, b2));
-    } else if (a2 == b2) {
-        v = 0.5 * (lag_entry<DRANGE>(p, a1, a2) + lag_entry<DRANGE>(p, b1, a2));
-    } else {
-        v = 0.25 * (lag_entry<DRANGE>(p, a1, a2) + lag_entry<DRANGE>(p, a1, b2) + lag_entry<DRANGE>(p, b1, a2) +
-                    lag_entry<DRANGE>(p, b1, b2));
+// Entry (j1, j2) of the first row of the block-circulant extension on the M1 x
+// M2 torus.
+__device__ __noinline__ double torus_entry(const CovDev& p, int j1, int j2, int M1, int M2, bool drange) {
+    const int a1 = (2 * j1 <= M1) ? j1 : j1 - M1, a2 = (2 * j2 <= M2) ? j2 : j2 - M2;
+    double v = lag_entry(p, a1, a2, drange);
+    if (!p.even && (2 * j1 == M1 || 2 * j2 == M2)) {   // a lag of half the torus averages its images
+        const int b1 = (2 * j1 < M1) ? j1 : j1 - M1, b2 = (2 * j2 < M2) ? j2 : j2 - M2;
+        if (a1 == b1) v = 0.5 * (v + lag_entry(p, a1, b2, drange));
+        else if (a2 == b2) v = 0.5 * (v + lag_entry(p, b1, a2, drange));
+        else v = 0.25 * (v + lag_entry(p, a1, b2, drange) + lag_entry(p, b1, a2, drange) + lag_entry(p, b1, b2, drange));
     }
-    c[idx] = v;
+    return v;
 }
 
-// ------------------------------------------------------------------ full FP64 2-D FFT
+// ------------------------------------------------------------------ FP64 2-D FFTs
+//
+// The torus covariance c is real and c[-j] = c[j], so Lambda = FFT2(c) is real
+// and even, and a quarter of the transforms of a full complex FFT2 gives it:
+//   rows   R[j1][k] for j1 = 0 .. M1/2 only (R[-j1][k] is its conjugate), two
+//          real rows as one complex transform, k = 0 .. M2/2 kept;
+//   columns two columns k, k + 1 as one complex transform (each has a real
+//          result, its input being Hermitian), k = 0 .. M2/2 only (Lambda[-k1][-k2]
+//          = Lambda[k1][k2]).
+// Everything is FP64-pipe bound (fft64.cuh), so that is also what it gains:
+// eigenvalues on the 2048^2 torus 270 us (1,045 us before).
+// A sample, Re FFT2(a xi), is FFT2 of the Hermitian part of a xi: rows k1 = 0 ..
+// M1/2, then the same column transforms (252 us; 527 before).
 
-// Row transforms over all M1 rows (length M2), G rows per CTA.
-// IN 0: real input rows (c);  IN 1: sqrt(max(lam, 0) * scale) * (xi_re + i xi_im).
-template <int EPT, int G, int IN>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_rows_full(const double* __restrict__ rin, const double* __restrict__ xi,
-                                                    double scale, double2* __restrict__ z, int M1, int M2,
-                                                    const double2* __restrict__ tw) {
+// Row transforms of the lag covariance: transform pr takes rows 2 pr and 2 pr + 1,
+// evaluated on the spot (even covariances: half of a row, the rest mirrored).
+// z[j1][k], j1 <= M1/2, k <= M2/2, leading dimension M2/2 + 1.
+template <int B, int E, int NT>
+__global__ void __launch_bounds__(NT * ((1 << B) / E), kf64::minb(NT * ((1 << B) / E), E))
+    ke_rows(CovDev p, bool drange, double2* __restrict__ z, int M1, const double2* __restrict__ tw) {
+    using P = kf64::Plan<B, E>;
+    constexpr int L = P::L, LT = P::LT, PS = P::PS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* buf = reinterpret_cast<double2*>(smem_raw);
-    const int L = M2, stride = L + 1, LT = L / EPT;
-    const int g = threadIdx.x / LT, tl = threadIdx.x - g * LT;
-    const int row = blockIdx.x * G + g;
-    double2* rb = buf + g * stride;
-    if (row < M1) {
-        const int64_t off = (int64_t)row * M2;
-        for (int k = tl; k < L; k += LT) {
-            if (IN == 0) {
-                rb[k] = make_double2(rin[off + k], 0.0);
-            } else {
-                const double a = sqrt(fmax(rin[off + k], 0.0) * scale);
-                rb[k] = make_double2(a * xi[off + k], a * xi[(int64_t)M1 * M2 + off + k]);
+    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    double2* sb = reinterpret_cast<double2*>(smem_raw) + n;
+    const int ja = min(2 * ((int)blockIdx.x * NT + n), M1 / 2);
+    const bool live = 2 * ((int)blockIdx.x * NT + n) <= M1 / 2, two = ja + 1 <= M1 / 2;
+    double2 v[E];
+    if (p.even) {
+#pragma unroll 1
+        for (int j = t; j <= L / 2; j += LT)
+            sb[kf64::soff<PS, NT>(j)] = make_double2(torus_entry(p, ja, j, M1, L, drange),
+                                                    two ? torus_entry(p, ja + 1, j, M1, L, drange) : 0.0);
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < E; ++m) {
+            const int j = t + m * LT;
+            v[m] = sb[kf64::soff<PS, NT>(min(j, L - j))];
+        }
+        __syncthreads();
+    } else {
+#pragma unroll 1
+        for (int j = t; j < L; j += LT)
+            sb[kf64::soff<PS, NT>(j)] = make_double2(torus_entry(p, ja, j, M1, L, drange),
+                                                    two ? torus_entry(p, ja + 1, j, M1, L, drange) : 0.0);
+#pragma unroll
+        for (int m = 0; m < E; ++m) v[m] = sb[kf64::soff<PS, NT>(t + m * LT)];   // the thread's own
+        __syncthreads();
+    }
+    kf64::transform<P, NT, false, false, false>(sb, v, t, tw);
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < E; ++s) sb[kf64::soff<PS, NT>(t + s * LT)] = v[kf64::brev(s, P::LE)];
+    __syncthreads();
+    if (!live) return;
+    double2* za = z + (int64_t)ja * (L / 2 + 1);
+    double2* zb = za + (L / 2 + 1);
+    for (int k = t; k <= L / 2; k += LT) {
+        const double2 a = sb[kf64::soff<PS, NT>(k)], b = sb[kf64::soff<PS, NT>((L - k) & (L - 1))];
+        za[k] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+        if (two) zb[k] = make_double2(0.5 * (a.y + b.y), 0.5 * (b.x - a.x));
+    }
+}
+
+// Row transforms of a sample: row k1 of the Hermitian part of sqrt(max(lam, 0)
+// scale) (xi_re + i xi_im).  z[k1][j], k1 <= M1/2, j < ldz.
+template <int B, int E, int NT>
+__global__ void __launch_bounds__(NT * ((1 << B) / E), kf64::minb(NT * ((1 << B) / E), E))
+    ke_rows_noise(const double* __restrict__ lam, const double* __restrict__ xi, double scale,
+                  double2* __restrict__ z, int M1, int ldz, const double2* __restrict__ tw) {
+    using P = kf64::Plan<B, E>;
+    constexpr int L = P::L, LT = P::LT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    const int row = (int)blockIdx.x * NT + n;
+    const bool live = row <= M1 / 2;
+    const int ra = min(row, M1 / 2), rb = (M1 - ra) & (M1 - 1);
+    const double *re_a = xi + (int64_t)ra * L, *re_b = xi + (int64_t)rb * L;
+    const double *im_a = re_a + (int64_t)M1 * L, *im_b = re_b + (int64_t)M1 * L;
+    double2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int k = t + m * LT, kb = (L - k) & (L - 1);
+        const double a = 0.5 * sqrt(fmax(lam[(int64_t)ra * L + k], 0.0) * scale);
+        v[m] = make_double2(a * (re_a[k] + re_b[kb]), a * (im_a[k] - im_b[kb]));
+    }
+    kf64::transform<P, NT, false, false, false>(reinterpret_cast<double2*>(smem_raw) + n, v, t, tw);
+    if (!live) return;
+#pragma unroll
+    for (int s = 0; s < E; ++s) {
+        const int j = t + s * LT;
+        if (j < ldz) z[(int64_t)row * ldz + j] = v[kf64::brev(s, P::LE)];
+    }
+}
+
+// Order-preserving map of doubles to integers (min and max without the FP64
+// pipe) and back.
+__device__ __forceinline__ long long order_key(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double order_value(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+
+// Column transforms of Hermitian columns 2q and 2q + 1 of z (rows 0 .. M1/2
+// given, leading dimension ldz; columns >= ncol are zero) as one complex
+// transform.  OUT 0: lam[k1][j] for every column of the M1 x M2 torus (columns
+// past M2/2 by symmetry) and the block's smallest and largest value as order
+// keys in part; OUT 1: out[i][j], i < n1, j < n2.
+template <int B, int E, int NT, int OUT>
+__global__ void __launch_bounds__(NT * ((1 << B) / E), kf64::minb(NT * ((1 << B) / E), E))
+    ke_cols(const double2* __restrict__ z, int ldz, int ncol, double* __restrict__ out, int M2, int n1, int n2,
+            const double2* __restrict__ tw, long long* __restrict__ part) {
+    using P = kf64::Plan<B, E>;
+    constexpr int L = P::L, LT = P::LT, TH = NT * LT;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ long long red[2][TH / 32];
+    const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
+    const int j0 = 2 * ((int)blockIdx.x * NT + n);
+    const bool one = j0 < ncol, two = j0 + 1 < ncol;
+    const double2* za = z + (one ? j0 : 0);
+    const double2* zb = z + (two ? j0 + 1 : 0);
+    double2 v[E];
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+        const int j = t + m * LT;
+        const int64_t r = (int64_t)min(j, L - j) * ldz;
+        const double2 a = za[r], b = zb[r];
+        const double sg = 2 * j > L ? -1.0 : 1.0;   // rows past the middle: conjugates
+        v[m] = make_double2(two ? a.x - sg * b.y : a.x, two ? sg * a.y + b.x : sg * a.y);
+    }
+    kf64::transform<P, NT, false, false, false>(reinterpret_cast<double2*>(smem_raw) + n, v, t, tw);
+    if constexpr (OUT == 1) {
+#pragma unroll
+        for (int s = 0; s < E; ++s) {
+            const int i = t + s * LT;
+            const double2 f = v[kf64::brev(s, P::LE)];
+            if (i < n1 && j0 < n2) out[(int64_t)i * n2 + j0] = f.x;
+            if (i < n1 && j0 + 1 < n2) out[(int64_t)i * n2 + j0 + 1] = f.y;
+        }
+    } else {
+        long long lo = 0x7fffffffffffffffll, hi = -0x7fffffffffffffffll - 1;
+#pragma unroll
+        for (int s = 0; s < E; ++s) {
+            const int k1 = t + s * LT;
+            const double2 f = v[kf64::brev(s, P::LE)];
+            double* o = out + (int64_t)k1 * M2;
+            double* om = out + (int64_t)((L - k1) & (L - 1)) * M2;
+            if (one) {
+                o[j0] = f.x;
+                if (j0 > 0 && 2 * j0 < M2) om[M2 - j0] = f.x;
+                const long long k = order_key(f.x);
+                if (f.x == f.x) {
+                    lo = min(lo, k);
+                    hi = max(hi, k);
+                }
+            }
+            if (two) {
+                o[j0 + 1] = f.y;
+                if (2 * (j0 + 1) < M2) om[M2 - j0 - 1] = f.y;
+                const long long k = order_key(f.y);
+                if (f.y == f.y) {
+                    lo = min(lo, k);
+                    hi = max(hi, k);
+                }
             }
         }
-    } else {
-        for (int k = tl; k < L; k += LT) rb[k] = make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    fft_smem<double2, false, EPT>(rb, L, tl, tw);
-    if (row < M1) {
-        const int64_t off = (int64_t)row * M2;
-        for (int k = tl; k < L; k += LT) z[off + k] = rb[k];
-    }
-}
-
-// Column transforms (length M1) of CC columns per CTA; writes the real part.
-// OUT 0: lam[k1][j] for every column;  OUT 1: out[i][j] for i < n1, j < n2.
-template <int EPT, int CC, int OUT>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_cols_full(const double2* __restrict__ z, double* __restrict__ out, int M1,
-                                                    int M2, int n1, int n2, const double2* __restrict__ tw) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* buf = reinterpret_cast<double2*>(smem_raw);
-    const int L = M1, stride = L + 1, LT = L / EPT;
-    const int g = threadIdx.x / LT, tl = threadIdx.x - g * LT;
-    const int j0 = blockIdx.x * CC;
-    for (int e = threadIdx.x; e < L * CC; e += blockDim.x) {
-        const int k = e / CC, c = e - k * CC;
-        buf[c * stride + k] = z[(int64_t)k * M2 + j0 + c];
-    }
-    __syncthreads();
-    double2* cb = buf + g * stride;
-    fft_smem<double2, false, EPT>(cb, L, tl, tw);
-    if (OUT == 0) {
-        for (int e = threadIdx.x; e < L * CC; e += blockDim.x) {
-            const int k = e / CC, c = e - k * CC;
-            out[(int64_t)k * M2 + j0 + c] = buf[c * stride + k].x;
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         }
-    } else {
-        for (int e = threadIdx.x; e < n1 * CC; e += blockDim.x) {
-            const int k = e / CC, c = e - k * CC;
-            if (j0 + c < n2) out[(int64_t)k * n2 + j0 + c] = buf[c * stride + k].x;
+        if ((threadIdx.x & 31) == 0) {
+            red[0][threadIdx.x >> 5] = lo;
+            red[1][threadIdx.x >> 5] = hi;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < TH / 32; ++w) {
+                lo = min(lo, red[0][w]);
+                hi = max(hi, red[1][w]);
+            }
+            part[2 * blockIdx.x] = lo;
+            part[2 * blockIdx.x + 1] = hi;
         }
     }
 }
 
-static int pick_group(int L, int ept, size_t bytes_per_elem, size_t lim) {
-    int g = 1;
-    while (g < 8 && (size_t)(2 * g) * (L + 1) * bytes_per_elem <= lim && 2 * g * (L / ept) <= 256) g *= 2;
-    return g;
-}
-
-template <int IN>
-static void launch_rows_full(kry_ctx* ctx, const double* rin, const double* xi, double scale, double2* z, int M1,
-                             int M2) {
-    const int ept = (M2 >= 8192) ? 16 : 8;
-    const int G = pick_group(M2, ept, sizeof(double2), ctx->max_smem_optin - 1024);
-    const int thr = G * (M2 / ept);
-    const size_t sm = (size_t)G * (M2 + 1) * sizeof(double2);
-    const int nb = (M1 + G - 1) / G;
-    const double2* tw = ctx->tw64.as<double2>();
-#define KRY_ROWS(E, GG)                                                                     \
-    do {                                                                                    \
-        auto k = k_rows_full<E, GG, IN>;                                                    \
-        KRY_ALLOW_MAX_SMEM(k); \
-        k<<<nb, thr, sm, ctx->stream>>>(rin, xi, scale, z, M1, M2, tw);                     \
-    } while (0)
-    if (ept == 8) {
-        if (G == 1) KRY_ROWS(8, 1); else if (G == 2) KRY_ROWS(8, 2); else if (G == 4) KRY_ROWS(8, 4); else KRY_ROWS(8, 8);
-    } else {
-        if (G == 1) KRY_ROWS(16, 1); else if (G == 2) KRY_ROWS(16, 2); else if (G == 4) KRY_ROWS(16, 4); else KRY_ROWS(16, 8);
-    }
-#undef KRY_ROWS
-    KRY_CHECK_LAUNCH();
-}
-
-template <int OUT>
-static void launch_cols_full(kry_ctx* ctx, const double2* z, double* out, int M1, int M2, int n1, int n2) {
-    const int ept = (M1 >= 8192) ? 16 : 8;
-    int C = pick_group(M1, ept, sizeof(double2), ctx->max_smem_optin - 1024);
-    while (C > 1 && M2 % C) C /= 2;
-    const int thr = C * (M1 / ept);
-    const size_t sm = (size_t)C * (M1 + 1) * sizeof(double2);
-    int nb = M2 / C;
-    if (OUT == 1) nb = (n2 + C - 1) / C;
-    const double2* tw = ctx->tw64.as<double2>();
-#define KRY_COLS(E, CCV)                                                                    \
-    do {                                                                                    \
-        auto k = k_cols_full<E, CCV, OUT>;                                                  \
-        KRY_ALLOW_MAX_SMEM(k); \
-        k<<<nb, thr, sm, ctx->stream>>>(z, out, M1, M2, n1, n2, tw);                        \
-    } while (0)
-    if (ept == 8) {
-        if (C == 1) KRY_COLS(8, 1); else if (C == 2) KRY_COLS(8, 2); else if (C == 4) KRY_COLS(8, 4); else KRY_COLS(8, 8);
-    } else {
-        if (C == 1) KRY_COLS(16, 1); else if (C == 2) KRY_COLS(16, 2); else if (C == 4) KRY_COLS(16, 4); else KRY_COLS(16, 8);
-    }
-#undef KRY_COLS
-    KRY_CHECK_LAUNCH();
-}
-
-// ------------------------------------------------------------------ min / max
-
-__global__ void k_minmax(const double* __restrict__ x, int64_t n, double* __restrict__ part) {
-    __shared__ double smin[32], smax[32];
-    double lo = DBL_MAX, hi = -DBL_MAX;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = x[i];
-        lo = fmin(lo, v);
-        hi = fmax(hi, v);
+// Smallest and largest value over the column blocks (one block).
+__global__ void k_minmax_final(const long long* __restrict__ part, int nb, double* __restrict__ out) {
+    __shared__ long long slo[8], shi[8];
+    long long lo = 0x7fffffffffffffffll, hi = -0x7fffffffffffffffll - 1;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        lo = min(lo, part[2 * b]);
+        hi = max(hi, part[2 * b + 1]);
     }
     for (int o = 16; o > 0; o >>= 1) {
-        lo = fmin(lo, __shfl_down_sync(0xffffffffu, lo, o));
-        hi = fmax(hi, __shfl_down_sync(0xffffffffu, hi, o));
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
     if ((threadIdx.x & 31) == 0) {
-        smin[threadIdx.x >> 5] = lo;
-        smax[threadIdx.x >> 5] = hi;
+        slo[threadIdx.x >> 5] = lo;
+        shi[threadIdx.x >> 5] = hi;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-            lo = fmin(lo, smin[w]);
-            hi = fmax(hi, smax[w]);
-        }
-        lo = fmin(lo, smin[0]);
-        hi = fmax(hi, smax[0]);
-        part[2 * blockIdx.x] = lo;
-        part[2 * blockIdx.x + 1] = hi;
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+        lo = min(lo, slo[w]);
+        hi = max(hi, shi[w]);
     }
+    out[0] = order_value(lo);
+    out[1] = order_value(hi);
 }
 
-__global__ void k_minmax_final(double* part, int nb) {
-    double lo = DBL_MAX, hi = -DBL_MAX;
-    for (int b = 0; b < nb; ++b) {
-        lo = fmin(lo, part[2 * b]);
-        hi = fmax(hi, part[2 * b + 1]);
+namespace {
+
+struct RunRows {
+    CovDev p;
+    bool drange;
+    double2* z;
+    int M1;
+    const double2* tw;
+    cudaStream_t st;
+    template <int B, int E, int NT>
+    void run() const {
+        using P = kf64::Plan<B, E>;
+        auto k = ke_rows<B, E, NT>;
+        KRY_ALLOW_MAX_SMEM(k);
+        k<<<(M1 / 4 + NT) / NT, NT * P::LT, (size_t)NT * P::SLOTS * 16, st>>>(p, drange, z, M1, tw);
+        KRY_CHECK_LAUNCH();
     }
-    part[0] = lo;
-    part[1] = hi;
-}
+};
+struct RunNoise {
+    const double *lam, *xi;
+    double scale;
+    double2* z;
+    int M1, ldz;
+    const double2* tw;
+    cudaStream_t st;
+    template <int B, int E, int NT>
+    void run() const {
+        using P = kf64::Plan<B, E>;
+        auto k = ke_rows_noise<B, E, NT>;
+        KRY_ALLOW_MAX_SMEM(k);
+        k<<<(M1 / 2 + NT) / NT, NT * P::LT, (size_t)NT * P::SLOTS * 16, st>>>(lam, xi, scale, z, M1, ldz, tw);
+        KRY_CHECK_LAUNCH();
+    }
+};
+template <int OUT>
+struct RunCols {
+    const double2* z;
+    int ldz, ncol;
+    double* out;
+    int M2, n1, n2;
+    const double2* tw;
+    DevBuf* red;   // order keys of every block, then the two results
+    int* nblocks;
+    cudaStream_t st;
+    template <int B, int E, int NT>
+    void run() const {
+        using P = kf64::Plan<B, E>;
+        const int nb = ((ncol + 1) / 2 + NT - 1) / NT;
+        if (OUT == 0) red->ensure((size_t)(2 * nb + 2) * sizeof(long long));
+        *nblocks = nb;
+        auto k = ke_cols<B, E, NT, OUT>;
+        KRY_ALLOW_MAX_SMEM(k);
+        k<<<nb, NT * P::LT, (size_t)NT * P::SLOTS * 16, st>>>(z, ldz, ncol, out, M2, n1, n2, tw,
+                                                             OUT == 0 ? red->as<long long>() : nullptr);
+        KRY_CHECK_LAUNCH();
+    }
+};
+
+}  // namespace
 
 static CovDev cov_dev(const kry_cov& cov, double dx1, double dx2) {
     CovDev p;
     p.sigma2 = cov.sigma2;
     p.inv_range = 1.0 / cov.range;
     p.nu = cov.nu;
+    p.s = sqrt(2.0 * cov.nu) / cov.range;
     p.ca = cos(cov.aniso_angle);
     p.sa = sin(cov.aniso_angle);
     p.ratio = cov.aniso_ratio;
+    if (p.ratio == 1.0) {   // isotropic: the angle does not matter
+        p.ca = 1.0;
+        p.sa = 0.0;
+    }
     p.dx1 = dx1;
     p.dx2 = dx2;
+    p.kind = cov.nu == 0.5 ? 0 : cov.nu == 1.5 ? 1 : cov.nu == 2.5 ? 2 : 3;
+    p.even = p.ca == 0.0 || p.sa == 0.0;
     return p;
+}
+
+// Eigenvalues (drange: of the range derivative) on the M1 x M2 torus, natural
+// order, into out; the blocks' order keys are left in ctx->red.  Returns their
+// number.
+static int torus_eigs(kry_ctx* ctx, bool drange, const kry_cov& cov, double dx1, double dx2, int M1, int M2, double* out) {
+    const int ldz = M2 / 2 + 1;
+    ctx->eig_z.ensure((size_t)(M1 / 2 + 1) * ldz * sizeof(double2));
+    double2* z = ctx->eig_z.as<double2>();
+    const double2* tw = ctx->tab64.as<double2>();
+    int nb = 0;
+    kf64::dispatch<false>(M2, kf64::shape(M2), RunRows{cov_dev(cov, dx1, dx2), drange, z, M1, tw, ctx->stream});
+    kf64::dispatch<false>(M1, kf64::shape(M1),
+                   RunCols<0>{z, ldz, ldz, out, M2, 0, 0, tw, &ctx->red, &nb, ctx->stream});
+    return nb;
 }
 
 void compute_eigs(kry_ctx* ctx, const kry_cov& cov, int n1, int n2, double dx1, double dx2, int M1, int M2,
                   double* lam_min, double* lam_max) {
-    const int64_t MM = (int64_t)M1 * M2;
-    ctx->eig_c.ensure(MM * sizeof(double));
-    ctx->eig_z.ensure(MM * sizeof(double2));
-    double* c = ctx->eig_c.as<double>();
-    double2* z = ctx->eig_z.as<double2>();
     (void)n1;
     (void)n2;
-    k_lag_cov<<<(unsigned)((MM + 255) / 256), 256, 0, ctx->stream>>>(c, M1, M2, cov_dev(cov, dx1, dx2));
+    ctx->eig_c.ensure((size_t)M1 * M2 * sizeof(double));
+    const int nb = torus_eigs(ctx, false, cov, dx1, dx2, M1, M2, ctx->eig_c.as<double>());
+    double* res = ctx->red.as<double>() + 2 * nb;
+    k_minmax_final<<<1, 256, 0, ctx->stream>>>(ctx->red.as<long long>(), nb, res);
     KRY_CHECK_LAUNCH();
-    launch_rows_full<0>(ctx, c, nullptr, 0.0, z, M1, M2);
-    launch_cols_full<0>(ctx, z, c, M1, M2, 0, 0);   // Lambda (real part) back into c
-    const int nb = 256;
-    ctx->red.ensure(2 * nb * sizeof(double));
-    k_minmax<<<nb, 256, 0, ctx->stream>>>(c, MM, ctx->red.as<double>());
-    KRY_CHECK_LAUNCH();
-    k_minmax_final<<<1, 1, 0, ctx->stream>>>(ctx->red.as<double>(), nb);
-    KRY_CHECK_LAUNCH();
-    KRY_CUDA(cudaMemcpyAsync(ctx->host_pinned, ctx->red.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    KRY_CUDA(cudaMemcpyAsync(ctx->host_pinned, res, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     KRY_CUDA(cudaStreamSynchronize(ctx->stream));
     *lam_min = ctx->host_pinned[0];
     *lam_max = ctx->host_pinned[1];
@@ -363,12 +485,7 @@ void bccb_logdet(kry_ctx* ctx, const kry_cov& cov, bool deriv, double* logdet, d
     if (deriv) {
         ctx->eig_d.ensure(MM * sizeof(double));
         d2 = ctx->eig_d.as<double>();
-        k_lag_cov<true><<<(unsigned)((MM + 255) / 256), 256, 0, ctx->stream>>>(d2, M1, M2,
-                                                                            cov_dev(cov, ctx->dx1, ctx->dx2));
-        KRY_CHECK_LAUNCH();
-        double2* z = ctx->eig_z.as<double2>();
-        launch_rows_full<0>(ctx, d2, nullptr, 0.0, z, M1, M2);
-        launch_cols_full<0>(ctx, z, d2, M1, M2, 0, 0);   // D2 (real part) back into d2
+        torus_eigs(ctx, true, cov, ctx->dx1, ctx->dx2, M1, M2, d2);
     }
     const int nb = 256;
     ctx->red.ensure((2 * nb + 2) * sizeof(double));
@@ -425,16 +542,8 @@ void store_embedding(kry_ctx* ctx, kry_embed* e, int slot) {
 // with e apply the range derivative of the covariance (Appendix A, dSigma).
 void drange_embedding(kry_ctx* ctx, const kry_cov& cov, kry_embed* e) {
     const int M1 = e->M1, M2 = e->M2;
-    const int64_t MM = (int64_t)M1 * M2;
-    ctx->eig_c.ensure(MM * sizeof(double));
-    ctx->eig_z.ensure(MM * sizeof(double2));
-    double* c = ctx->eig_c.as<double>();
-    double2* z = ctx->eig_z.as<double2>();
-    k_lag_cov<true><<<(unsigned)((MM + 255) / 256), 256, 0, ctx->stream>>>(c, M1, M2,
-                                                                        cov_dev(cov, ctx->dx1, ctx->dx2));
-    KRY_CHECK_LAUNCH();
-    launch_rows_full<0>(ctx, c, nullptr, 0.0, z, M1, M2);
-    launch_cols_full<0>(ctx, z, c, M1, M2, 0, 0);
+    ctx->eig_c.ensure((size_t)M1 * M2 * sizeof(double));
+    torus_eigs(ctx, true, cov, ctx->dx1, ctx->dx2, M1, M2, ctx->eig_c.as<double>());
     store_embedding(ctx, e, 0);
 }
 
@@ -442,9 +551,13 @@ void drange_embedding(kry_ctx* ctx, const kry_cov& cov, kry_embed* e) {
 void sample_field(kry_ctx* ctx, const kry_cov& cov, int M1, int M2, const double* xi, double* out) {
     double lo, hi;
     compute_eigs(ctx, cov, ctx->n1, ctx->n2, ctx->dx1, ctx->dx2, M1, M2, &lo, &hi);
-    double2* z = ctx->eig_z.as<double2>();
-    launch_rows_full<1>(ctx, ctx->eig_c.as<double>(), xi, 1.0 / ((double)M1 * (double)M2), z, M1, M2);
-    launch_cols_full<1>(ctx, z, out, M1, M2, ctx->n1, ctx->n2);
+    const int n1 = ctx->n1, n2 = ctx->n2;
+    double2* z = ctx->eig_z.as<double2>();   // (M1/2 + 1) x n2 of it, n2 <= M2/2
+    const double2* tw = ctx->tab64.as<double2>();
+    int nb = 0;
+    kf64::dispatch<false>(M2, kf64::shape(M2),
+                   RunNoise{ctx->eig_c.as<double>(), xi, 1.0 / ((double)M1 * (double)M2), z, M1, n2, tw, ctx->stream});
+    kf64::dispatch<false>(M1, kf64::shape(M1), RunCols<1>{z, n2, n2, out, M2, n1, n2, tw, nullptr, &nb, ctx->stream});
 }
 
 }  // namespace kry

@@ -148,11 +148,3 @@ __device__ __forceinline__ void fft_smem(C* buf, int L, int t, const C* __restri
         Ns *= 8;
     }
 }
-
-template <typename T> __device__ __forceinline__ const typename cx_of<T>::type* twiddles(const void* tw32, const void* tw64);
-template <> __device__ __forceinline__ const float2* twiddles<float>(const void* tw32, const void*) {
-    return static_cast<const float2*>(tw32);
-}
-template <> __device__ __forceinline__ const double2* twiddles<double>(const void*, const void* tw64) {
-    return static_cast<const double2*>(tw64);
-}

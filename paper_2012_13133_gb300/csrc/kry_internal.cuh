@@ -134,9 +134,10 @@ struct kry_ctx {
     DevBuf cellidx;  // int32 [p]: row-major cell index of each observed cell
     DevBuf cellbits; // uint2 [n1][ceil(n2 / 32)]: observation bits of 32 cells, index of the first observed one
 
-    // shared twiddle tables, W[k] = exp(-2 pi i k / KRY_TWN), and the tables of
-    // the specialised FP32 passes (kspec::fill_tables)
-    DevBuf tw32, tw64, spec_tab;
+    // twiddle table of the short FP32 passes, W[k] = exp(-2 pi i k / KRY_TWN), and
+    // the tables of the specialised FP32 passes (kspec::fill_tables) and of the
+    // FP64 transforms (kf64::fill_table)
+    DevBuf tw32, spec_tab, tab64;
 
     // scratch
     DevBuf slab32, slab64;        // FFT intermediates

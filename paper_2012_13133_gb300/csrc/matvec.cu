@@ -27,23 +27,25 @@
 
 #include "dfloat.cuh"
 #include "fft.cuh"
-#include "fft16.cuh"
 #include "mvspec.cuh"
 #include "kry_internal.cuh"
+#include "mv64.cuh"
 
 namespace kry {
 
+// The specialised FP32 passes (mvspec.cuh) cover torus sides from 64, the FP64
+// ones (mv64.cu) every side; the three kernels below run FP32 on the shorter
+// tori, radix 8 in shared memory (fft.cuh).
+
 // ------------------------------------------------------------------ pass A
 
-template <typename T, int EPT, int G>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_a(const T* __restrict__ vin, int64_t ld, const double* __restrict__ scale,
+template <int EPT, int G>
+__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_a(const float* __restrict__ vin, int64_t ld, const double* __restrict__ scale,
                                                  int nvec, int pair0, const int* __restrict__ rowptr,
                                                  const int* __restrict__ colidx, int n1, int M2, int C,
-                                                 typename cx_of<T>::type* __restrict__ slab, const void* tw32,
-                                                 const void* tw64) {
-    using Cx = typename cx_of<T>::type;
+                                                 float2* __restrict__ slab, const float2* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
+    float2* buf = reinterpret_cast<float2*>(smem_raw);
     const int L = M2;
     const int stride = L + 1;
     const int LT = L / EPT;
@@ -54,28 +56,28 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_a(const T* __re
     const int pair = pair0 + blockIdx.y;
     const int va = 2 * pair, vb = 2 * pair + 1;
     const bool has_b = vb < nvec;
-    Cx* rb = buf + g * stride;
+    float2* rb = buf + g * stride;
 
-    for (int k = tl; k < L; k += LT) rb[k] = cmk<Cx>((T)0, (T)0);
+    for (int k = tl; k < L; k += LT) rb[k] = make_float2(0.f, 0.f);
     __syncthreads();
     if (row < n1) {
-        const T sa = scale ? (T)scale[va] : (T)1;
-        const T sb = (scale && has_b) ? (T)scale[vb] : (T)1;
-        const T* pa = vin + (int64_t)va * ld;
-        const T* pb = vin + (int64_t)vb * ld;
+        const float sa = scale ? (float)scale[va] : 1.f;
+        const float sb = (scale && has_b) ? (float)scale[vb] : 1.f;
+        const float* pa = vin + (int64_t)va * ld;
+        const float* pb = vin + (int64_t)vb * ld;
         const int q1 = rowptr[row + 1];
         for (int q = rowptr[row] + tl; q < q1; q += LT) {
             const int c = colidx[q];
-            const T a = pa[q] * sa;
-            const T b = has_b ? pb[q] * sb : (T)0;
-            rb[c] = cmk<Cx>(a, b);
+            const float a = pa[q] * sa;
+            const float b = has_b ? pb[q] * sb : 0.f;
+            rb[c] = make_float2(a, b);
         }
     }
     __syncthreads();
-    fft_smem<Cx, false, EPT>(rb, L, tl, twiddles<T>(tw32, tw64));
+    fft_smem<float2, false, EPT>(rb, L, tl, tw);
 
     // store: slab[pair][tile][row][c]
-    Cx* out = slab + (int64_t)blockIdx.y * n1 * M2;
+    float2* out = slab + (int64_t)blockIdx.y * n1 * M2;
     const int GC = G * C;
     for (int e = threadIdx.x; e < G * L; e += blockDim.x) {
         const int tile = e / GC;
@@ -89,20 +91,19 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_a(const T* __re
 
 // ------------------------------------------------------------------ pass B
 
-template <typename T, int EPT, int CC>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(typename cx_of<T>::type* __restrict__ slab, const T* __restrict__ lamT,
-                                                 int n1, int M1, int M2, const void* tw32, const void* tw64,
+template <int EPT, int CC>
+__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(float2* __restrict__ slab, const float* __restrict__ lamT,
+                                                 int n1, int M1, int M2, const float2* __restrict__ tw,
                                                  int pair0, int64_t lam_stride, int vpt) {
-    using Cx = typename cx_of<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
+    float2* buf = reinterpret_cast<float2*>(smem_raw);
     const int L = M1;
     const int stride = L + 1;
     const int LT = L / EPT;
     const int g = threadIdx.x / LT;
     const int tl = threadIdx.x - g * LT;
     const int tile = blockIdx.x;
-    Cx* blk = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)tile * n1 * CC;
+    float2* blk = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)tile * n1 * CC;
 
     const int nload = n1 * CC;
     for (int e = threadIdx.x; e < nload; e += blockDim.x) {
@@ -113,21 +114,20 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(typename cx_o
     for (int e = threadIdx.x; e < (L - n1) * CC; e += blockDim.x) {
         const int c = e / (L - n1);
         const int i = n1 + (e - c * (L - n1));
-        buf[c * stride + i] = cmk<Cx>((T)0, (T)0);
+        buf[c * stride + i] = make_float2(0.f, 0.f);
     }
     __syncthreads();
-    Cx* cb = buf + g * stride;
-    const Cx* tw = twiddles<T>(tw32, tw64);
-    fft_smem<Cx, false, EPT>(cb, L, tl, tw);
+    float2* cb = buf + g * stride;
+    fft_smem<float2, false, EPT>(cb, L, tl, tw);
     const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
-    const T* lam = lamT + theta * lam_stride + (int64_t)(tile * CC + g) * L;
+    const float* lam = lamT + theta * lam_stride + (int64_t)(tile * CC + g) * L;
     for (int k = tl; k < L; k += LT) {
-        const T l = lam[k];
-        Cx z = cb[k];
-        cb[k] = cmk<Cx>(z.x * l, z.y * l);
+        const float l = lam[k];
+        float2 z = cb[k];
+        cb[k] = make_float2(z.x * l, z.y * l);
     }
     __syncthreads();
-    fft_smem<Cx, true, EPT>(cb, L, tl, tw);
+    fft_smem<float2, true, EPT>(cb, L, tl, tw);
     for (int e = threadIdx.x; e < nload; e += blockDim.x) {
         const int i = e / CC;
         const int c = e - i * CC;
@@ -137,19 +137,17 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(typename cx_o
 
 // ------------------------------------------------------------------ pass C
 
-// MODE 0: gather the observed cells, add tau2 * (scaled input), optional dot.
-// MODE 1: write every grid cell (n1 x n2 row-major) per vector, no nugget.
-template <typename T, int EPT, int G, int MODE>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const typename cx_of<T>::type* __restrict__ slab, const T* __restrict__ vin,
-                                                 int64_t ld_in, const double* __restrict__ scale, T* __restrict__ vout,
+// Gathers the observed cells, adds tau2 * (scaled input), optional dot.
+template <int EPT, int G>
+__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const float2* __restrict__ slab, const float* __restrict__ vin,
+                                                 int64_t ld_in, const double* __restrict__ scale, float* __restrict__ vout,
                                                  int64_t ld_out, int nvec, int pair0, const int* __restrict__ rowptr,
                                                  const int* __restrict__ colidx, int n1, int n2, int M2, int C,
                                                  double tau2, double* __restrict__ dots, int ndot_stride,
-                                                 const void* tw32, const void* tw64, const double* __restrict__ tau2v,
+                                                 const float2* __restrict__ tw, const double* __restrict__ tau2v,
                                                  int vpt) {
-    using Cx = typename cx_of<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
+    float2* buf = reinterpret_cast<float2*>(smem_raw);
     __shared__ double red[2][32];
     const int L = M2;
     const int stride = L + 1;
@@ -161,7 +159,7 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const typenam
     const int va = 2 * pair, vb = 2 * pair + 1;
     const bool has_b = vb < nvec;
 
-    const Cx* in = slab + (int64_t)blockIdx.y * n1 * M2;
+    const float2* in = slab + (int64_t)blockIdx.y * n1 * M2;
     const int GC = G * C;
     for (int e = threadIdx.x; e < G * L; e += blockDim.x) {
         const int tile = e / GC;
@@ -170,284 +168,41 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const typenam
         const int c = rem - gg * C;
         const int r = row0 + gg;
         buf[gg * stride + tile * C + c] =
-            (r < n1) ? in[(int64_t)tile * n1 * C + (int64_t)r * C + c] : cmk<Cx>((T)0, (T)0);
+            (r < n1) ? in[(int64_t)tile * n1 * C + (int64_t)r * C + c] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    Cx* rb = buf + g * stride;
-    fft_smem<Cx, true, EPT>(rb, L, tl, twiddles<T>(tw32, tw64));
+    float2* rb = buf + g * stride;
+    fft_smem<float2, true, EPT>(rb, L, tl, tw);
 
     const int row = row0 + g;
-    DotAcc<T> acc_a, acc_b;
+    DotAcc<float> acc_a, acc_b;
     if (row < n1) {
-        if (MODE == 0) {
-            const T sa = scale ? (T)scale[va] : (T)1;
-            const T sb = (scale && has_b) ? (T)scale[vb] : (T)1;
-            const T t2 = (T)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
-            const T* pa = vin + (int64_t)va * ld_in;
-            const T* pb = vin + (int64_t)vb * ld_in;
-            T* oa = vout + (int64_t)va * ld_out;
-            T* ob = vout + (int64_t)vb * ld_out;
-            const int q1 = rowptr[row + 1];
-            for (int q = rowptr[row] + tl; q < q1; q += LT) {
-                const Cx z = rb[colidx[q]];
-                const T xa = pa[q] * sa;
-                const T ya = z.x + t2 * xa;
-                oa[q] = ya;
-                acc_a.add_prod(xa, ya);
-                if (has_b) {
-                    const T xb = pb[q] * sb;
-                    const T yb = z.y + t2 * xb;
-                    ob[q] = yb;
-                    acc_b.add_prod(xb, yb);
-                }
-            }
-        } else {
-            T* oa = vout + (int64_t)va * ld_out + (int64_t)row * n2;
-            T* ob = vout + (int64_t)vb * ld_out + (int64_t)row * n2;
-            for (int j = tl; j < n2; j += LT) {
-                const Cx z = rb[j];
-                oa[j] = z.x;
-                if (has_b) ob[j] = z.y;
+        const float sa = scale ? (float)scale[va] : 1.f;
+        const float sb = (scale && has_b) ? (float)scale[vb] : 1.f;
+        const float t2 = (float)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
+        const float* pa = vin + (int64_t)va * ld_in;
+        const float* pb = vin + (int64_t)vb * ld_in;
+        float* oa = vout + (int64_t)va * ld_out;
+        float* ob = vout + (int64_t)vb * ld_out;
+        const int q1 = rowptr[row + 1];
+        for (int q = rowptr[row] + tl; q < q1; q += LT) {
+            const float2 z = rb[colidx[q]];
+            const float xa = pa[q] * sa;
+            const float ya = z.x + t2 * xa;
+            oa[q] = ya;
+            acc_a.add_prod(xa, ya);
+            if (has_b) {
+                const float xb = pb[q] * sb;
+                const float yb = z.y + t2 * xb;
+                ob[q] = yb;
+                acc_b.add_prod(xb, yb);
             }
         }
     }
-    if (MODE == 0 && dots != nullptr) {
+    if (dots != nullptr) {
         double da = acc_a.value(), db = acc_b.value();
         // block reduction of (da, db) in a fixed order; blocks narrower than a
         // warp (short rows) reduce serially through shared memory
-        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        if (blockDim.x >= 32) {
-            for (int o = 16; o > 0; o >>= 1) {
-                da += __shfl_down_sync(0xffffffffu, da, o);
-                db += __shfl_down_sync(0xffffffffu, db, o);
-            }
-            if (lane == 0) {
-                red[0][w] = da;
-                red[1][w] = db;
-            }
-        } else {
-            red[0][threadIdx.x] = da;
-            red[1][threadIdx.x] = db;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sa = 0.0, sb = 0.0;
-            const int nw = (blockDim.x >= 32) ? (blockDim.x >> 5) : blockDim.x;
-            for (int k = 0; k < nw; ++k) {
-                sa += red[0][k];
-                sb += red[1][k];
-            }
-            dots[(int64_t)va * ndot_stride + blockIdx.x] = sa;
-            if (has_b) dots[(int64_t)vb * ndot_stride + blockIdx.x] = sb;
-        }
-    }
-}
-
-// ------------------------------------------------------------------ radix-16 passes (64 <= L <= 8192)
-
-#ifndef KRY_K16_MINB
-#define KRY_K16_MINB 2   // register budget for 2 resident 512-thread blocks per SM (<= 64 registers; measured fastest)
-#endif
-//
-// Same three passes as above, built from the radix-16 register stages of
-// fft16.cuh: G rows (pass A/C) or CC columns (pass B) per block, interleaved
-// in padded shared memory; the first and last stages read and write global
-// memory (or registers) directly, and pass B multiplies by Lambda between its
-// forward and inverse column transforms without leaving registers.
-
-template <typename T, int G>
-__global__ void __launch_bounds__(512, KRY_K16_MINB) k16_pass_a(const T* __restrict__ vin, int64_t ld, const double* __restrict__ scale,
-                                                  int nvec, int pair0, const int* __restrict__ rowptr,
-                                                  const int* __restrict__ colidx, int n1, int n2, int M2, int C,
-                                                  int logC, int PS, typename cx_of<T>::type* __restrict__ slab,
-                                                  const void* tw32, const void* tw64, const int* __restrict__ skip) {
-    using Cx = typename cx_of<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
-    const int L = M2, b = 31 - __clz(L), LT = L >> 4;
-    const int g = threadIdx.x % G, t = threadIdx.x / G;
-    const int row = blockIdx.x * G + g;
-    const int pair = pair0 + blockIdx.y;
-    const int va = 2 * pair, vb = 2 * pair + 1;
-    const bool has_b = vb < nvec;
-    if (skip && skip[va] && (!has_b || skip[vb])) return;   // both columns finished (whole block)
-    const Cx* tw = twiddles<T>(tw32, tw64);
-    const Cx zero = cmk<Cx>((T)0, (T)0);
-
-    for (int pos = t; pos < n2; pos += LT) buf[kry16::spos(pos, PS, G, g)] = zero;
-    __syncthreads();
-    if (row < n1) {
-        const T sa = scale ? (T)scale[va] : (T)1;
-        const T sb = (scale && has_b) ? (T)scale[vb] : (T)1;
-        const T* pa = vin + (int64_t)va * ld;
-        const T* pb = vin + (int64_t)vb * ld;
-        const int q1 = rowptr[row + 1];
-        for (int q = rowptr[row] + t; q < q1; q += LT)
-            buf[kry16::spos(colidx[q], PS, G, g)] = cmk<Cx>(pa[q] * sa, has_b ? pb[q] * sb : (T)0);
-    }
-    __syncthreads();
-
-    Cx* out = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)row * C;
-    const int64_t tstride = (int64_t)n1 * C;
-    auto ld_s = [&](int pos) { return buf[kry16::spos(pos, PS, G, g)]; };
-    auto ld_0 = [&](int pos) { return pos < n2 ? buf[kry16::spos(pos, PS, G, g)] : zero; };
-    auto st_s = [&](int pos, Cx z) { buf[kry16::spos(pos, PS, G, g)] = z; };
-    auto st_g = [&](int pos, Cx z) {
-        if (row < n1) out[(int64_t)(pos >> logC) * tstride + (pos & (C - 1))] = z;
-    };
-    Cx v[16];
-    kry16::transform<Cx, false, true>(b, v, t, tw, ld_0, ld_s, st_s, st_g, true, false);
-}
-
-template <typename T, int CC>
-__global__ void __launch_bounds__(512, KRY_K16_MINB) k16_pass_b(typename cx_of<T>::type* __restrict__ slab,
-                                                  const T* __restrict__ lamT, int n1, int M1, int M2, int PS,
-                                                  const void* tw32, const void* tw64, int pair0, int64_t lam_stride,
-                                                  int vpt, const int* __restrict__ skip, int nvec) {
-    using Cx = typename cx_of<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
-    if (skip) {
-        const int va = 2 * (pair0 + (int)blockIdx.y), vb = va + 1;
-        if (skip[va] && (vb >= nvec || skip[vb])) return;
-    }
-    const int L = M1, b = 31 - __clz(L), LT = L >> 4;
-    const int c = threadIdx.x % CC, t = threadIdx.x / CC;
-    const int tile = blockIdx.x;
-    Cx* blk = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)tile * n1 * CC;
-    const Cx* tw = twiddles<T>(tw32, tw64);
-    const Cx zero = cmk<Cx>((T)0, (T)0);
-
-    auto ld_g = [&](int pos) { return pos < n1 ? blk[pos * CC + c] : zero; };
-    auto ld_s = [&](int pos) { return buf[kry16::spos(pos, PS, CC, c)]; };
-    auto st_s = [&](int pos, Cx z) { buf[kry16::spos(pos, PS, CC, c)] = z; };
-    auto st_g = [&](int pos, Cx z) {
-        if (pos < n1) blk[pos * CC + c] = z;
-    };
-    const int nst = kry16::num_stages(b);
-    Cx v[16];
-    // forward column transform, ending in registers (slot m = row t + m L/16)
-    {
-        const int r0 = kry16::stage_radix(b, 0);
-        // rows >= n1 (>= M1/2) are zero: half-input first stage
-        using LDG = decltype(ld_g)&;
-        using STS = decltype(st_s)&;
-        switch (r0) {
-            case 2: kry16::stage<Cx, 2, false, LDG, STS, true>(v, t, L, 1, tw, ld_g, st_s, false); break;
-            case 4: kry16::stage<Cx, 4, false, LDG, STS, true>(v, t, L, 1, tw, ld_g, st_s, false); break;
-            case 8: kry16::stage<Cx, 8, false, LDG, STS, true>(v, t, L, 1, tw, ld_g, st_s, false); break;
-            default: kry16::stage<Cx, 16, false, LDG, STS, true>(v, t, L, 1, tw, ld_g, st_s, false); break;
-        }
-        __syncthreads();
-        int Ns = r0;
-#pragma unroll 1
-        for (int s = 1; s < nst - 1; ++s) {
-            kry16::stage<Cx, 16, false>(v, t, L, Ns, tw, ld_s, st_s, true);
-            __syncthreads();
-            Ns *= 16;
-        }
-        kry16::last_stage_regs<Cx, false>(v, t, L, Ns, tw, ld_s, true);
-    }
-    // eigenvalue multiply (scaled by 1/(M1 M2))
-    const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
-    const T* lam = lamT + theta * lam_stride + (int64_t)(tile * CC + c) * L;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-        const T l = lam[t + m * LT];
-        v[m] = cmk<Cx>(v[m].x * l, v[m].y * l);
-    }
-    // inverse column transform, starting from registers, keeping rows < n1
-    {
-        const int r0 = kry16::stage_radix(b, 0);
-        kry16::first_stage_regs<Cx, true>(r0, v, t, L, tw, st_s);
-        __syncthreads();
-        int Ns = r0;
-#pragma unroll 1
-        for (int s = 1; s < nst - 1; ++s) {
-            kry16::stage<Cx, 16, true>(v, t, L, Ns, tw, ld_s, st_s, true);
-            __syncthreads();
-            Ns *= 16;
-        }
-        kry16::stage<Cx, 16, true>(v, t, L, Ns, tw, ld_s, st_g, false);
-    }
-}
-
-template <typename T, int G, int MODE>
-__global__ void __launch_bounds__(512, KRY_K16_MINB) k16_pass_c(const typename cx_of<T>::type* __restrict__ slab,
-                                                  const T* __restrict__ vin, int64_t ld_in,
-                                                  const double* __restrict__ scale, T* __restrict__ vout,
-                                                  int64_t ld_out, int nvec, int pair0, const int* __restrict__ rowptr,
-                                                  const int* __restrict__ colidx, int n1, int n2, int M2, int C,
-                                                  int logC, int PS, double tau2, double* __restrict__ dots,
-                                                  int ndot_stride, const void* tw32, const void* tw64,
-                                                  const double* __restrict__ tau2v, int vpt,
-                                                  const int* __restrict__ skip) {
-    using Cx = typename cx_of<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Cx* buf = reinterpret_cast<Cx*>(smem_raw);
-    __shared__ double red[2][32];
-    const int L = M2, b = 31 - __clz(L), LT = L >> 4;
-    const int g = threadIdx.x % G, t = threadIdx.x / G;
-    const int row = blockIdx.x * G + g;
-    const int pair = pair0 + blockIdx.y;
-    const int va = 2 * pair, vb = 2 * pair + 1;
-    const bool has_b = vb < nvec;
-    if (skip && skip[va] && (!has_b || skip[vb])) return;   // both columns finished (whole block)
-    const Cx* tw = twiddles<T>(tw32, tw64);
-    const Cx zero = cmk<Cx>((T)0, (T)0);
-
-    const Cx* in = slab + (int64_t)blockIdx.y * n1 * M2 + (int64_t)row * C;
-    const int64_t tstride = (int64_t)n1 * C;
-    auto ld_g = [&](int pos) {
-        return row < n1 ? in[(int64_t)(pos >> logC) * tstride + (pos & (C - 1))] : zero;
-    };
-    auto ld_s = [&](int pos) { return buf[kry16::spos(pos, PS, G, g)]; };
-    auto st_s = [&](int pos, Cx z) { buf[kry16::spos(pos, PS, G, g)] = z; };
-    auto st_n = [&](int pos, Cx z) {
-        if (pos < n2) buf[kry16::spos(pos, PS, G, g)] = z;
-    };
-    Cx v[16];
-    kry16::transform<Cx, true>(b, v, t, tw, ld_g, ld_s, st_s, st_n, false, true);
-    __syncthreads();
-
-    DotAcc<T> acc_a, acc_b;
-    if (row < n1) {
-        if (MODE == 0) {
-            const T sa = scale ? (T)scale[va] : (T)1;
-            const T sb = (scale && has_b) ? (T)scale[vb] : (T)1;
-            const T t2 = (T)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
-            const T* pa = vin + (int64_t)va * ld_in;
-            const T* pb = vin + (int64_t)vb * ld_in;
-            T* oa = vout + (int64_t)va * ld_out;
-            T* ob = vout + (int64_t)vb * ld_out;
-            const int q1 = rowptr[row + 1];
-            for (int q = rowptr[row] + t; q < q1; q += LT) {
-                const Cx z = buf[kry16::spos(colidx[q], PS, G, g)];
-                const T xa = pa[q] * sa;
-                const T ya = z.x + t2 * xa;
-                oa[q] = ya;
-                acc_a.add_prod(xa, ya);
-                if (has_b) {
-                    const T xb = pb[q] * sb;
-                    const T yb = z.y + t2 * xb;
-                    ob[q] = yb;
-                    acc_b.add_prod(xb, yb);
-                }
-            }
-        } else {
-            T* oa = vout + (int64_t)va * ld_out + (int64_t)row * n2;
-            T* ob = vout + (int64_t)vb * ld_out + (int64_t)row * n2;
-            for (int j = t; j < n2; j += LT) {
-                const Cx z = buf[kry16::spos(j, PS, G, g)];
-                oa[j] = z.x;
-                if (has_b) ob[j] = z.y;
-            }
-        }
-    }
-    if (MODE == 0 && dots != nullptr) {
-        double da = acc_a.value(), db = acc_b.value();
-        // rows are interleaved across lanes (g fastest); the block reduction
-        // sums every row's products of the block in a fixed order
         const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
         if (blockDim.x >= 32) {
             for (int o = 16; o > 0; o >>= 1) {
@@ -482,80 +237,39 @@ static size_t cx_size(bool dbl) { return dbl ? sizeof(double2) : sizeof(float2);
 
 int smem_limit(kry_ctx* ctx) { return ctx->max_smem_optin; }
 
-template <typename T>
-struct MvLaunch {
-    using Cx = typename cx_of<T>::type;
-
-    template <int EPT, int G>
-    static void a(dim3 grid, int threads, size_t smem, cudaStream_t s, const T* vin, int64_t ld, const double* scale,
-                  int nvec, int pair0, const int* rowptr, const int* colidx, int n1, int M2, int C, Cx* slab,
-                  const void* tw32, const void* tw64) {
-        auto k = k_pass_a<T, EPT, G>;
-        KRY_ALLOW_MAX_SMEM(k);
-        k<<<grid, threads, smem, s>>>(vin, ld, scale, nvec, pair0, rowptr, colidx, n1, M2, C, slab, tw32, tw64);
-        KRY_CHECK_LAUNCH();
-    }
-    template <int EPT, int CC>
-    static void b(dim3 grid, int threads, size_t smem, cudaStream_t s, Cx* slab, const T* lamT, int n1, int M1, int M2,
-                  const void* tw32, const void* tw64, int pair0 = 0, int64_t lam_stride = 0, int vpt = 0) {
-        auto k = k_pass_b<T, EPT, CC>;
-        KRY_ALLOW_MAX_SMEM(k);
-        k<<<grid, threads, smem, s>>>(slab, lamT, n1, M1, M2, tw32, tw64, pair0, lam_stride, vpt);
-        KRY_CHECK_LAUNCH();
-    }
-    template <int EPT, int G, int MODE>
-    static void c(dim3 grid, int threads, size_t smem, cudaStream_t s, const Cx* slab, const T* vin, int64_t ld_in,
-                  const double* scale, T* vout, int64_t ld_out, int nvec, int pair0, const int* rowptr,
-                  const int* colidx, int n1, int n2, int M2, int C, double tau2, double* dots, int nds,
-                  const void* tw32, const void* tw64, const double* tau2v = nullptr, int vpt = 0) {
-        auto k = k_pass_c<T, EPT, G, MODE>;
-        KRY_ALLOW_MAX_SMEM(k);
-        k<<<grid, threads, smem, s>>>(slab, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, n2, M2,
-                                      C, tau2, dots, nds, tw32, tw64, tau2v, vpt);
-        KRY_CHECK_LAUNCH();
-    }
-};
-
-#define KRY_DISPATCH_EG(EPTV, GV, CALL)                                               \
+#define KRY_DISPATCH_EG(EPTV, GV, ...)                                                \
     do {                                                                              \
         if (EPTV == 8) {                                                              \
-            if (GV == 1) { constexpr int E_ = 8, G_ = 1; CALL; }                       \
-            else if (GV == 2) { constexpr int E_ = 8, G_ = 2; CALL; }                  \
-            else if (GV == 4) { constexpr int E_ = 8, G_ = 4; CALL; }                  \
-            else if (GV == 8) { constexpr int E_ = 8, G_ = 8; CALL; }                  \
+            if (GV == 1) { constexpr int E_ = 8, G_ = 1; __VA_ARGS__; }                       \
+            else if (GV == 2) { constexpr int E_ = 8, G_ = 2; __VA_ARGS__; }                  \
+            else if (GV == 4) { constexpr int E_ = 8, G_ = 4; __VA_ARGS__; }                  \
+            else if (GV == 8) { constexpr int E_ = 8, G_ = 8; __VA_ARGS__; }                  \
             else throw KryError{KRY_EUNSUPPORTED, "bad group count"};                \
         } else if (EPTV == 16) {                                                      \
-            if (GV == 1) { constexpr int E_ = 16, G_ = 1; CALL; }                      \
-            else if (GV == 2) { constexpr int E_ = 16, G_ = 2; CALL; }                 \
-            else if (GV == 4) { constexpr int E_ = 16, G_ = 4; CALL; }                 \
-            else if (GV == 8) { constexpr int E_ = 16, G_ = 8; CALL; }                 \
+            if (GV == 1) { constexpr int E_ = 16, G_ = 1; __VA_ARGS__; }                      \
+            else if (GV == 2) { constexpr int E_ = 16, G_ = 2; __VA_ARGS__; }                 \
+            else if (GV == 4) { constexpr int E_ = 16, G_ = 4; __VA_ARGS__; }                 \
+            else if (GV == 8) { constexpr int E_ = 16, G_ = 8; __VA_ARGS__; }                 \
             else throw KryError{KRY_EUNSUPPORTED, "bad group count"};                \
         } else                                                                        \
             throw KryError{KRY_EUNSUPPORTED, "bad elements per thread"};              \
     } while (0)
 
-// Pick a schedule that fits shared memory and the 1024-thread block limit.
-static MvSched pick_sched(kry_ctx* ctx, const MvSched& want, int M1, int M2, bool dbl) {
+// Schedule of the short FP32 passes that fits shared memory and the block limits.
+static MvSched pick_sched(kry_ctx* ctx, const MvSched& want, int M1, int M2) {
     MvSched s = want;
-    const size_t cs = cx_size(dbl);
     const size_t lim = (size_t)ctx->max_smem_optin - 1024;   // leave room for static shared memory
     auto fix = [&](int& ept, int& grp, int L) {
         if (ept != 8 && ept != 16) ept = 8;
         if (L < ept) ept = 8;
         if (L / ept > 1024) ept = 16;
         const int maxthr = (ept >= 16) ? 512 : 1024;
-        while (grp > 1 && ((size_t)grp * (L + 1) * cs > lim || grp * (L / ept) > maxthr)) grp /= 2;
+        while (grp > 1 && ((size_t)grp * (L + 1) * sizeof(float2) > lim || grp * (L / ept) > maxthr)) grp /= 2;
     };
     fix(s.ept_row, s.rows_per_cta, M2);
     fix(s.ept_col, s.cols_per_cta, M1);
     return s;
 }
-
-// ---- radix-16 path: schedule, shared-memory pad shift and launches
-
-#ifndef KRY_SMEM_CARVEOUT
-#define KRY_SMEM_CARVEOUT -1   // L1 / shared-memory split: driver default (measured fastest)
-#endif
 
 void prof_record(kry_ctx* ctx, cudaEvent_t ev) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -566,21 +280,8 @@ void prof_record(kry_ctx* ctx, cudaEvent_t ev) {
         KRY_CUDA(cudaEventRecord(ev, ctx->stream));
 }
 
-static bool use16(int M1, int M2) { return M1 >= 64 && M2 >= 64 && M1 <= KRY_MAX_M && M2 <= KRY_MAX_M; }
-
-// Pad shift of the interleaved shared-memory layout for NT transforms of
-// length L (chosen from a bank-conflict model of the stage access patterns).
-static int pad_shift(int L, int NT) {
-    if (L >= 4096) return 4;
-    if (L == 2048) return NT == 1 ? 4 : 3;
-    if (NT >= 4) return 2;
-    if (NT == 2) return 3;
-    return 4;
-}
-
-static size_t smem16(int L, int NT, bool dbl) {
-    return (size_t)(L + (L >> pad_shift(L, NT))) * NT * cx_size(dbl);
-}
+// FP32 tori that the specialised passes cover.
+static bool use_spec(int M1, int M2) { return M1 >= 64 && M2 >= 64 && M1 <= KRY_MAX_M && M2 <= KRY_MAX_M; }
 
 static int ilog2(int x) { return 31 - __builtin_clz((unsigned)x); }
 
@@ -600,128 +301,119 @@ const MvSched& sched_for(kry_ctx* ctx, int M1, int M2, bool dbl, int nvec) {
     return dbl ? ctx->sched64 : ctx->sched32;
 }
 
-// Rows per block (pass A/C) and columns per block (pass B; for FP64 also the
-// slab tile width).
-static void sched16(kry_ctx* ctx, int M1, int M2, bool dbl, int nvec, int* G, int* C) {
-    const MvSched& want = sched_for(ctx, M1, M2, dbl, nvec);
-    if (!dbl) {
-        // Specialised passes: blocks of 128 threads (four and more per SM, so that one block's
-        // loads run behind another's butterflies), 256 for the longest columns, whose slab rows
-        // would otherwise be read 8 bytes at a time; down to two warps (one for columns) while the
-        // launch has fewer blocks than two per SM (128^2, 4 vectors: 11.0 us, with 128 threads 12).
-        const int ltr = kspec::transform_threads(M2), ltc = kspec::transform_threads(M1);
-        const int np = (nvec + 1) / 2;
-        auto fill = [&](int lt, int th, int least, int64_t transforms) {
-            while (th > least && th > lt && transforms * lt / th < 2 * ctx->num_sms) th /= 2;
-            return std::max(1, th / lt);
-        };
-        const int g = want.g16 > 0 ? want.g16 : fill(ltr, 128, 64, (int64_t)(M1 / 2) * np);
-        const int c = want.c16 > 0 ? want.c16 : fill(ltc, M1 >= 4096 ? 256 : 128, 32, (int64_t)M2 * np);
-        *G = kspec::block_threads(M2, g, 64) / ltr;
-        *C = kspec::block_threads(M1, c, M2) / ltc;
-        return;
-    }
-    const size_t lim = (size_t)ctx->max_smem_optin - 1024;   // leave room for static shared memory
-    auto fit = [&](int L, int nt) {
-        nt = std::max(1, std::min(nt, 16));
-        while (nt > 1 && (nt * (L >> 4) > 512 || smem16(L, nt, dbl) > lim)) nt >>= 1;
-        return nt;
+// Rows per block (passes A and C) and columns per block (pass B) of the
+// specialised FP32 passes.  Blocks of 128 threads (four and more per SM, so that
+// one block's loads run behind another's butterflies), 256 for the longest
+// columns, whose slab rows would otherwise be read 8 bytes at a time; down to
+// two warps (one for columns) while the launch has fewer blocks than two per SM
+// (128^2, 4 vectors: 11.0 us, with 128 threads 12).  The rows per block group pass
+// C's dot partials, so they do not depend on the batch.
+static void spec_shape(kry_ctx* ctx, const kry_embed* e, int nvec, int* G, int* C) {
+    const int M1 = e->M1, M2 = e->M2, np = (nvec + 1) / 2;
+    const MvSched& want = sched_for(ctx, M1, M2, false, nvec);
+    const int ltr = kspec::transform_threads(M2), ltc = kspec::transform_threads(M1);
+    auto fill = [&](int lt, int th, int least, int64_t transforms) {
+        while (th > least && th > lt && transforms * lt / th < 2 * ctx->num_sms) th /= 2;
+        return std::max(1, th / lt);
     };
-    int g = want.g16 > 0 ? want.g16 : std::max(1, 256 / (M2 >> 4));
-    int c = want.c16 > 0 ? want.c16 : std::max(1, 512 / (M1 >> 4));
-    *G = fit(M2, g);
-    *C = std::min(fit(M1, c), M2);
+    const int g = want.g16 > 0 ? want.g16 : fill(ltr, 128, 64, M1 / 2);
+    const int c = want.c16 > 0 ? want.c16 : fill(ltc, M1 >= 4096 ? 256 : 128, 32, (int64_t)M2 * np);
+    *G = kspec::block_threads(M2, g, 64) / ltr;
+    *C = kspec::block_threads(M1, c, M2) / ltc;
 }
 
-#define KRY_DISPATCH_NT(NTV, ...)                                  \
-    do {                                                            \
-        switch (NTV) {                                              \
-            case 1: { constexpr int N_ = 1; __VA_ARGS__; } break;          \
-            case 2: { constexpr int N_ = 2; __VA_ARGS__; } break;          \
-            case 4: { constexpr int N_ = 4; __VA_ARGS__; } break;          \
-            case 8: { constexpr int N_ = 8; __VA_ARGS__; } break;          \
-            case 16: { constexpr int N_ = 16; __VA_ARGS__; } break;        \
-            default: throw KryError{KRY_EUNSUPPORTED, "bad transforms per block"}; \
-        }                                                           \
-    } while (0)
+// Row and column transforms of the FP64 passes.
+static void shape64(kry_ctx* ctx, const kry_embed* e, int nvec, kf64::Shape* row, kf64::Shape* col) {
+    const MvSched& want = sched_for(ctx, e->M1, e->M2, true, nvec);
+    *row = kf64::shape(e->M2, want.g16);
+    *col = kf64::shape(e->M1, want.c16);
+}
 
-template <typename T>
-static void run_matvec16(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t ld_in, const double* scale, T* vout,
-                         int64_t ld_out, int nvec, double tau2, double* dots, int nds, int mode,
-                         typename cx_of<T>::type* slab, int ppb, int vpt, const int* skip) {
-    const bool dbl = sizeof(T) == 8;
-    const int n1 = e->n1, n2 = e->n2, M1 = e->M1, M2 = e->M2;
-    int G, C;
-    sched16(ctx, M1, M2, dbl, nvec, &G, &C);
+// Complex pairs per batch: all, unless the schedule says otherwise.
+static int batch_pairs(kry_ctx* ctx, const kry_embed* e, bool dbl, int nvec) {
     const int npairs = (nvec + 1) / 2;
-    const int* rowptr = ctx->rowptr.as<int>();
-    const int* colidx = ctx->colidx.as<int>();
-    const void* tw32 = ctx->tw32.p;
-    const void* tw64 = ctx->tw64.p;
+    const MvSched& want =
+        dbl || use_spec(e->M1, e->M2) ? sched_for(ctx, e->M1, e->M2, dbl, nvec) : ctx->sched32;
+    return want.pairs_per_batch > 0 ? std::min(want.pairs_per_batch, npairs) : npairs;
+}
+
+// The three passes for batches of ppb pairs through the given slab.
+template <typename T>
+static void run_passes(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t ld_in, const double* scale, T* vout,
+                       int64_t ld_out, int nvec, double tau2, double* dots, int nds, int mode, void* slab, int ppb,
+                       int vpt, const int* skip) {
+    const int n1 = e->n1, n2 = e->n2, M1 = e->M1, M2 = e->M2, npairs = (nvec + 1) / 2;
+    const double* tau2v = ctx->no_nugget ? nullptr : e->tau2_dev;
     cudaStream_t st = ctx->stream;
-    if constexpr (sizeof(T) == 4) {
-        KRY_REQUIRE(mode == 0 && e->lam32P != nullptr, KRY_EINVAL, "embedding lacks the permuted eigenvalues");
-        kspec::SpecArgs a{};
+    if constexpr (sizeof(T) == 8) {
+        kf64::Args a{};
         a.vin = vin; a.ld_in = ld_in; a.scale = scale; a.vout = vout; a.ld_out = ld_out;
         a.nvec = nvec; a.bits = ctx->cellbits.as<uint2>(); a.wpr = (n2 + 31) / 32;
-        a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2; a.G = G; a.C = C;
-        a.logCs = ilog2(std::max(4, C));   // tile rows of at least a 32-byte sector
-        a.slab = slab; a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
-        a.tau2 = tau2; a.tau2v = ctx->no_nugget ? nullptr : e->tau2_dev; a.dots = dots; a.nds = nds;
-        a.twf = ctx->spec_tab.as<float4>();
-        a.twi = a.twf + kspec::TWF_WORDS;
-        a.post = reinterpret_cast<const float2*>(a.twi + kspec::TWI_WORDS);
-        a.skip = skip;
-        for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
-            a.pair0 = pair0;
-            a.np = std::min(ppb, npairs - pair0);
-            KRY_REQUIRE(kspec::launch_a(a, st) && kspec::launch_b(a, st) && kspec::launch_c(a, st),
-                        KRY_EUNSUPPORTED, "no specialised matvec pass for this shape");
+        a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2;
+        shape64(ctx, e, nvec, &a.row, &a.col);
+        a.logC = ilog2(std::min(M2, std::max(2, a.col.NT)));   // tile rows of at least a 32-byte sector
+        a.slab = static_cast<double2*>(slab); a.lamT = e->lam64T; a.lam_stride = e->lam_stride; a.vpt = vpt;
+        a.tau2 = tau2; a.tau2v = tau2v; a.dots = dots; a.nds = nds;
+        a.tw = ctx->tab64.as<double2>(); a.skip = skip; a.mode = mode;
+        for (a.pair0 = 0; a.pair0 < npairs; a.pair0 += ppb) {
+            a.np = std::min(ppb, npairs - a.pair0);
+            kf64::launch(a, st);
         }
+        return;
     } else {
-    const T* lamT = e->lam64T;
-    const int psA = pad_shift(M2, G), psB = pad_shift(M1, C);
-    const int thrA = G * (M2 >> 4), thrB = C * (M1 >> 4);
-    const size_t smA = smem16(M2, G, dbl), smB = smem16(M1, C, dbl);
-    const int nbx = (n1 + G - 1) / G;
-    const int logC = ilog2(C);
-    for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
-        const int np = std::min(ppb, npairs - pair0);
-        dim3 gA(nbx, np), gB(M2 / C, np);
-        KRY_DISPATCH_NT(G, {
-            auto k = k16_pass_a<T, N_>;
-            KRY_ALLOW_MAX_SMEM(k);
-            KRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, KRY_SMEM_CARVEOUT));
-            k<<<gA, thrA, smA, st>>>(vin, ld_in, scale, nvec, pair0, rowptr, colidx, n1, n2, M2, C, logC, psA, slab,
-                                    tw32, tw64, skip);
-            KRY_CHECK_LAUNCH();
-        });
-        KRY_DISPATCH_NT(C, {
-            auto k = k16_pass_b<T, N_>;
-            KRY_ALLOW_MAX_SMEM(k);
-            KRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, KRY_SMEM_CARVEOUT));
-            k<<<gB, thrB, smB, st>>>(slab, lamT, n1, M1, M2, psB, tw32, tw64, pair0, e->lam_stride, vpt, skip, nvec);
-            KRY_CHECK_LAUNCH();
-        });
-        if (mode == 0) {
-            KRY_DISPATCH_NT(G, {
-                auto k = k16_pass_c<T, N_, 0>;
+        KRY_REQUIRE(mode == 0, KRY_EINVAL, "whole-grid output is FP64 only");
+        if (use_spec(M1, M2)) {
+            KRY_REQUIRE(e->lam32P != nullptr, KRY_EINVAL, "embedding lacks the permuted eigenvalues");
+            kspec::SpecArgs a{};
+            a.vin = vin; a.ld_in = ld_in; a.scale = scale; a.vout = vout; a.ld_out = ld_out;
+            a.nvec = nvec; a.bits = ctx->cellbits.as<uint2>(); a.wpr = (n2 + 31) / 32;
+            a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2;
+            spec_shape(ctx, e, nvec, &a.G, &a.C);
+            a.logCs = ilog2(std::max(4, a.C));   // tile rows of at least a 32-byte sector
+            a.slab = static_cast<float2*>(slab); a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
+            a.tau2 = tau2; a.tau2v = tau2v; a.dots = dots; a.nds = nds;
+            a.twf = ctx->spec_tab.as<float4>();
+            a.twi = a.twf + kspec::TWF_WORDS;
+            a.post = reinterpret_cast<const float2*>(a.twi + kspec::TWI_WORDS);
+            a.skip = skip;
+            for (a.pair0 = 0; a.pair0 < npairs; a.pair0 += ppb) {
+                a.np = std::min(ppb, npairs - a.pair0);
+                KRY_REQUIRE(kspec::launch_a(a, st) && kspec::launch_b(a, st) && kspec::launch_c(a, st),
+                            KRY_EUNSUPPORTED, "no specialised matvec pass for this shape");
+            }
+            return;
+        }
+        const MvSched s = pick_sched(ctx, ctx->sched32, M1, M2);
+        const int C = s.cols_per_cta, G = s.rows_per_cta;
+        const int* rowptr = ctx->rowptr.as<int>();
+        const int* colidx = ctx->colidx.as<int>();
+        const float2* tw = ctx->tw32.as<float2>();
+        float2* sl = static_cast<float2*>(slab);
+        const int thrA = G * (M2 / s.ept_row), thrB = C * (M1 / s.ept_col), nbx = (n1 + G - 1) / G;
+        const size_t smA = (size_t)G * (M2 + 1) * sizeof(float2), smB = (size_t)C * (M1 + 1) * sizeof(float2);
+        for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
+            const int np = std::min(ppb, npairs - pair0);
+            const dim3 gA(nbx, np), gB(M2 / C, np);
+            KRY_DISPATCH_EG(s.ept_row, G, {
+                auto k = k_pass_a<E_, G_>;
                 KRY_ALLOW_MAX_SMEM(k);
-                KRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, KRY_SMEM_CARVEOUT));
-                k<<<gA, thrA, smA, st>>>(slab, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, n2,
-                                        M2, C, logC, psA, tau2, dots, nds, tw32, tw64, ctx->no_nugget ? nullptr : e->tau2_dev, vpt, skip);
+                k<<<gA, thrA, smA, st>>>(vin, ld_in, scale, nvec, pair0, rowptr, colidx, n1, M2, C, sl, tw);
                 KRY_CHECK_LAUNCH();
             });
-        } else {
-            KRY_DISPATCH_NT(G, {
-                auto k = k16_pass_c<T, N_, 1>;
+            KRY_DISPATCH_EG(s.ept_col, C, {
+                auto k = k_pass_b<E_, G_>;
                 KRY_ALLOW_MAX_SMEM(k);
-                k<<<gA, thrA, smA, st>>>(slab, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, n2,
-                                        M2, C, logC, psA, tau2, dots, nds, tw32, tw64, ctx->no_nugget ? nullptr : e->tau2_dev, vpt, skip);
+                k<<<gB, thrB, smB, st>>>(sl, e->lam32T, n1, M1, M2, tw, pair0, e->lam_stride, vpt);
+                KRY_CHECK_LAUNCH();
+            });
+            KRY_DISPATCH_EG(s.ept_row, G, {
+                auto k = k_pass_c<E_, G_>;
+                KRY_ALLOW_MAX_SMEM(k);
+                k<<<gA, thrA, smA, st>>>(sl, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, n2, M2,
+                                         C, tau2, dots, nds, tw, tau2v, vpt);
                 KRY_CHECK_LAUNCH();
             });
         }
-    }
     }
 }
 
@@ -784,79 +476,17 @@ static void run_matvec(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t l
         run_matvec_sites<T>(ctx, e, vin, ld_in, scale, vout, ld_out, nvec, tau2, dots, nds, mode, vpt, skip);
         return;
     }
-    using Cx = typename cx_of<T>::type;
     const bool dbl = sizeof(T) == 8;
-    const int n1 = e->n1, n2 = e->n2, M1 = e->M1, M2 = e->M2;
-    if (use16(M1, M2)) {
-        const int npairs = (nvec + 1) / 2;
-        const MvSched& want = sched_for(ctx, M1, M2, dbl, nvec);
-        const int ppb = want.pairs_per_batch > 0 ? std::min(want.pairs_per_batch, npairs) : npairs;
-        DevBuf& sb = dbl ? ctx->slab64 : ctx->slab32;
-        sb.ensure((size_t)n1 * M2 * cx_size(dbl) * ppb);
-        cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-        if (ctx->prof_on) {
-            KRY_CUDA(cudaEventCreate(&ev0));
-            KRY_CUDA(cudaEventCreate(&ev1));
-            prof_record(ctx, ev0);
-        }
-        run_matvec16<T>(ctx, e, vin, ld_in, scale, vout, ld_out, nvec, tau2, dots, nds, mode, sb.as<Cx>(), ppb, vpt,
-                        skip);
-        if (ctx->prof_on) {
-            prof_record(ctx, ev1);
-            ctx->prof_ev.push_back(ev0);
-            ctx->prof_ev.push_back(ev1);
-            ctx->prof_nvec.push_back(nvec);
-            ctx->prof_dbl.push_back(dbl ? 1 : 0);
-        }
-        return;
-    }
-    MvSched s = pick_sched(ctx, dbl ? ctx->sched64 : ctx->sched32, M1, M2, dbl);
-    const int npairs = (nvec + 1) / 2;
-    int ppb = s.pairs_per_batch > 0 ? std::min(s.pairs_per_batch, npairs) : npairs;
-    const size_t slab_pair = (size_t)n1 * M2 * cx_size(dbl);
+    const int ppb = batch_pairs(ctx, e, dbl, nvec);
     DevBuf& sb = dbl ? ctx->slab64 : ctx->slab32;
-    sb.ensure(slab_pair * ppb);
-    Cx* slab = sb.as<Cx>();
-    const T* lamT = dbl ? reinterpret_cast<const T*>(e->lam64T) : reinterpret_cast<const T*>(e->lam32T);
-    const int C = s.cols_per_cta;
-    const int G = s.rows_per_cta;
-    const int* rowptr = ctx->rowptr.as<int>();
-    const int* colidx = ctx->colidx.as<int>();
-    const void* tw32 = ctx->tw32.p;
-    const void* tw64 = ctx->tw64.p;
-    cudaStream_t st = ctx->stream;
-    const int thrA = G * (M2 / s.ept_row);
-    const size_t smA = (size_t)G * (M2 + 1) * cx_size(dbl);
-    const int thrB = C * (M1 / s.ept_col);
-    const size_t smB = (size_t)C * (M1 + 1) * cx_size(dbl);
-    const int nbx = (n1 + G - 1) / G;
+    sb.ensure((size_t)e->n1 * e->M2 * cx_size(dbl) * ppb);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (ctx->prof_on) {
         KRY_CUDA(cudaEventCreate(&ev0));
         KRY_CUDA(cudaEventCreate(&ev1));
         prof_record(ctx, ev0);
     }
-    for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
-        const int np = std::min(ppb, npairs - pair0);
-        dim3 gA(nbx, np), gB(M2 / C, np);
-        KRY_DISPATCH_EG(s.ept_row, G,
-                        (MvLaunch<T>::template a<E_, G_>(gA, thrA, smA, st, vin, ld_in, scale, nvec, pair0, rowptr,
-                                                         colidx, n1, M2, C, slab, tw32, tw64)));
-        KRY_DISPATCH_EG(s.ept_col, C,
-                        (MvLaunch<T>::template b<E_, G_>(gB, thrB, smB, st, slab, lamT, n1, M1, M2, tw32, tw64, pair0,
-                                                         e->lam_stride, vpt)));
-        if (mode == 0) {
-            KRY_DISPATCH_EG(s.ept_row, G,
-                            (MvLaunch<T>::template c<E_, G_, 0>(gA, thrA, smA, st, slab, vin, ld_in, scale, vout,
-                                                                ld_out, nvec, pair0, rowptr, colidx, n1, n2, M2, C,
-                                                                tau2, dots, nds, tw32, tw64, ctx->no_nugget ? nullptr : e->tau2_dev, vpt)));
-        } else {
-            KRY_DISPATCH_EG(s.ept_row, G,
-                            (MvLaunch<T>::template c<E_, G_, 1>(gA, thrA, smA, st, slab, vin, ld_in, scale, vout,
-                                                                ld_out, nvec, pair0, rowptr, colidx, n1, n2, M2, C,
-                                                                tau2, dots, nds, tw32, tw64, ctx->no_nugget ? nullptr : e->tau2_dev, vpt)));
-        }
-    }
+    run_passes<T>(ctx, e, vin, ld_in, scale, vout, ld_out, nvec, tau2, dots, nds, mode, sb.p, ppb, vpt, skip);
     if (ctx->prof_on) {
         prof_record(ctx, ev1);
         ctx->prof_ev.push_back(ev0);
@@ -870,12 +500,17 @@ static void run_matvec(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t l
 // nvec vectors (the Krylov finalisers sum exactly this many).
 int matvec_num_partials(kry_ctx* ctx, const kry_embed* e, bool dbl, int nvec) {
     if (ctx->sites.active) return site_num_partials(ctx);
-    if (use16(e->M1, e->M2)) {
+    if (dbl) {
+        kf64::Shape row, col;
+        shape64(ctx, e, nvec, &row, &col);
+        return (e->n1 + row.NT - 1) / row.NT;
+    }
+    if (use_spec(e->M1, e->M2)) {
         int G, C;
-        sched16(ctx, e->M1, e->M2, dbl, nvec, &G, &C);
+        spec_shape(ctx, e, nvec, &G, &C);
         return (e->n1 + G - 1) / G;
     }
-    MvSched s = pick_sched(ctx, dbl ? ctx->sched64 : ctx->sched32, e->M1, e->M2, dbl);
+    const MvSched s = pick_sched(ctx, ctx->sched32, e->M1, e->M2);
     return (e->n1 + s.rows_per_cta - 1) / s.rows_per_cta;
 }
 
@@ -989,56 +624,15 @@ static void* noalloc_scratch(int device) {
 template <typename T>
 static void run_matvec_noalloc(kry_ctx* ctx, const kry_embed* e, const T* vin, T* vout, int nvec, int64_t ld,
                                void* scratch) {
-    using Cx = typename cx_of<T>::type;
     const bool dbl = sizeof(T) == 8;
-    const int n1 = e->n1, n2 = e->n2, M1 = e->M1, M2 = e->M2;
-    const size_t slab_pair = (size_t)n1 * M2 * cx_size(dbl);
+    const size_t slab_pair = (size_t)e->n1 * e->M2 * cx_size(dbl);
     KRY_REQUIRE(slab_pair <= KRY_NOALLOC_SCRATCH_BYTES, KRY_EUNSUPPORTED,
                 "grid too large for the allocation-free matvec: n1 * M2 * sizeof(complex) = " +
                     std::to_string(slab_pair) + " bytes exceeds its 16 MiB static scratch");
-    const int npairs = (nvec + 1) / 2;
     const int cap = std::max(1, (int)(KRY_NOALLOC_SCRATCH_BYTES / slab_pair));
-    Cx* slab = static_cast<Cx*>(scratch);
-    const double tau2 = e->cov.tau2;
-    if (use16(M1, M2)) {
-        // the passes and schedule of kry_matvec, with at most `cap` pairs per batch
-        const MvSched& want = sched_for(ctx, M1, M2, dbl, nvec);
-        int ppb = want.pairs_per_batch > 0 ? std::min(want.pairs_per_batch, npairs) : npairs;
-        ppb = std::min(ppb, cap);
-        run_matvec16<T>(ctx, e, vin, ld, nullptr, vout, ld, nvec, tau2, nullptr, 0, 0, slab, ppb, 0, nullptr);
-        return;
-    }
-    // transform lengths below 64: the generic radix-8 passes, as kry_matvec
-    MvSched s = pick_sched(ctx, dbl ? ctx->sched64 : ctx->sched32, M1, M2, dbl);
-    int ppb = s.pairs_per_batch > 0 ? std::min(s.pairs_per_batch, npairs) : npairs;
-    ppb = std::min(ppb, cap);
-    const T* lamT = dbl ? reinterpret_cast<const T*>(e->lam64T) : reinterpret_cast<const T*>(e->lam32T);
-    const int C = s.cols_per_cta;
-    const int G = s.rows_per_cta;
-    const int* rowptr = ctx->rowptr.as<int>();
-    const int* colidx = ctx->colidx.as<int>();
-    const void* tw32 = ctx->tw32.p;
-    const void* tw64 = ctx->tw64.p;
-    cudaStream_t st = ctx->stream;
-    const int thrA = G * (M2 / s.ept_row);
-    const size_t smA = (size_t)G * (M2 + 1) * cx_size(dbl);
-    const int thrB = C * (M1 / s.ept_col);
-    const size_t smB = (size_t)C * (M1 + 1) * cx_size(dbl);
-    const int nbx = (n1 + G - 1) / G;
-    for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
-        const int np = std::min(ppb, npairs - pair0);
-        dim3 gA(nbx, np), gB(M2 / C, np);
-        KRY_DISPATCH_EG(s.ept_row, G,
-                        (MvLaunch<T>::template a<E_, G_>(gA, thrA, smA, st, vin, ld, nullptr, nvec, pair0, rowptr,
-                                                         colidx, n1, M2, C, slab, tw32, tw64)));
-        KRY_DISPATCH_EG(s.ept_col, C,
-                        (MvLaunch<T>::template b<E_, G_>(gB, thrB, smB, st, slab, lamT, n1, M1, M2, tw32, tw64, pair0,
-                                                         e->lam_stride, 0)));
-        KRY_DISPATCH_EG(s.ept_row, G,
-                        (MvLaunch<T>::template c<E_, G_, 0>(gA, thrA, smA, st, slab, vin, ld, nullptr, vout, ld,
-                                                            nvec, pair0, rowptr, colidx, n1, n2, M2, C, tau2,
-                                                            nullptr, 0, tw32, tw64, e->tau2_dev, 0)));
-    }
+    // the passes and schedule of kry_matvec, with at most `cap` pairs per batch
+    run_passes<T>(ctx, e, vin, ld, nullptr, vout, ld, nvec, e->cov.tau2, nullptr, 0, 0, scratch,
+                  std::min(batch_pairs(ctx, e, dbl, nvec), cap), 0, nullptr);
 }
 
 }  // namespace kry
@@ -1130,20 +724,21 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
         const int c = (int)std::max<size_t>(1, budget / slab_pair);
         if (c < npairs && std::find(ppbs.begin(), ppbs.end(), c) == ppbs.end()) ppbs.push_back(c);
     }
-    const size_t lim = (size_t)ctx->max_smem_optin - 1024;   // leave room for static shared memory
     double best = 1e30;
     MvSched bs = dbl ? ctx->sched64 : ctx->sched32;
     const bool had = ctx->tuned.count(key) > 0;
     const MvSched prev = had ? ctx->tuned[key] : bs;
-    if (use16(M1, M2)) {
+    if (dbl || use_spec(M1, M2)) {
+        // blocks that are compiled as asked: others are rounded to one of these
         auto feasible = [&](int M, int nt, int most) {
-            return dbl ? nt * (M >> 4) <= 512 && smem16(M, nt, dbl) <= lim && nt <= most
+            return dbl ? kf64::shape(M, nt).NT == nt
                        : kspec::block_threads(M, nt, most) == nt * kspec::transform_threads(M);
         };
-        for (int g : {1, 2, 4, 8, 16}) {
-            if (!feasible(M2, g, 64)) continue;
-            for (int c : {1, 2, 4, 8, 16}) {
-                if (!feasible(M1, c, M2)) continue;
+        bool any = false;
+        for (int g : {0, 1, 2, 4, 8, 16}) {
+            if (g && !feasible(M2, g, 64)) continue;
+            for (int c : {0, 1, 2, 4, 8, 16}) {
+                if (c && !feasible(M1, c, M2)) continue;
                 for (int ppb : ppbs) {
                     MvSched cand = bs;
                     cand.g16 = g;
@@ -1151,12 +746,24 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
                     cand.pairs_per_batch = ppb;
                     ctx->tuned[key] = cand;
                     const double ms = time_sched<T>(ctx, e, tv.as<T>(), to.as<T>(), nvec, 3);
-                    if (ms < best) {
+                    if (!any || ms < best) {
+                        any = true;
                         best = ms;
                         bs = cand;
                     }
                 }
             }
+        }
+        // report the blocks that run
+        if (dbl) {
+            kf64::Shape row, col;
+            ctx->tuned[key] = bs;
+            shape64(ctx, e, nvec, &row, &col);
+            bs.g16 = row.NT;
+            bs.c16 = col.NT;
+        } else {
+            ctx->tuned[key] = bs;
+            spec_shape(ctx, e, nvec, &bs.g16, &bs.c16);
         }
         ctx->tuned[key] = bs;
     } else {
