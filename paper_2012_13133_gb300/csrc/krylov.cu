@@ -1287,14 +1287,19 @@ static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int
 // matvec of the iteration runs in FP32.  Convergence is declared only on a
 // true FP64 residual.
 
-// Each iteration is the plain CG recurrence on five launches, none of which
-// starts with a reduction:
-//   q = K p                      (FFT matvec; pass C forms the partials of p^T q)
-//   alpha = gamma / p^T q        (k_rcg_alpha: one block per column, fixed-order sum)
-//   x += alpha p, r -= alpha q   (k_rcg_update: streaming, forms the partials of r^T r)
-//   beta = gamma' / gamma        (k_rcg_beta: one block per column; counts the iteration
-//                                 and asks for a residual replacement)
-//   p = r + beta p               (k_rcg_pupdate: streaming)
+// Each iteration is the plain CG recurrence:
+//   q = K p                                  (FFT matvec; pass C forms the partials of p^T q)
+//   alpha = gamma / p^T q, r -= alpha q      (k_rcg_update; forms the partials of r^T r)
+//   beta = gamma' / gamma, x += alpha p, p = r + beta p   (k_rcg_pupdate; counts the
+//                                             iteration and asks for a residual replacement)
+// Every block of the two streaming kernels adds up the few hundred partials of
+// its column itself (total128, the same fixed order in all of them): about 0.4
+// us beside its first loads, where a launch of its own for alpha and for beta
+// took 3 us each.  x waits for the second kernel, which reads p anyhow.  An
+// iteration for 4 columns: 32 x 32 27.5 -> 24.1 us, 256 x 256 28.1 -> 26.0,
+// 1024 x 1024 100.7 -> 97.9.  (All of the vector work in one kernel, a cluster of
+// 16 blocks per column, took 22.6 us at 256 x 256 but 113.7 at 1024 x 1024, and
+// no less than these two from 8 columns on.)
 // K p is computed afresh by every matvec, so no auxiliary recurrence can
 // drift in FP32 (single-reduction rearrangements carry K p by a recurrence and
 // broke down on the ill-conditioned grids here).
@@ -1309,10 +1314,10 @@ static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int
 // It approximates K^-1 well where most of the grid is observed and the gaps
 // are clustered, and poorly under scattered missing cells.
 struct RcgState {
-    double* gam;      // [nrhs] gamma = r^T z (r^T r without a preconditioner)
+    double* gam;      // [nrhs] gamma = r^T z (r^T r without a preconditioner) of the current residual
+    double* gold;     // [nrhs] gamma of the residual that the current p belongs to
     double* rr;       // [nrhs] r^T r of the current residual
     double* alpha;    // [nrhs]
-    double* beta;     // [nrhs]
     double* rr_ref;   // [nrhs] r^T r at the last replacement
     double* thr2;     // [nrhs] (rtol ||b||)^2
     int* want;        // [nrhs] 1: the last iteration asks for a replacement
@@ -1364,8 +1369,8 @@ __global__ void k_rcg_init_scalars(RcgState S, const double* __restrict__ part_r
         S.gam[k] = g;
         S.rr[k] = s;
         S.rr_ref[k] = s;
+        S.gold[k] = g;
         S.alpha[k] = 0.0;
-        S.beta[k] = 0.0;
         S.thr2[k] = tol[k] * tol[k] * s;
         S.want[k] = 0;
         S.done[k] = (s == 0.0 || !(g > 0.0)) ? 1 : 0;
@@ -1373,103 +1378,139 @@ __global__ void k_rcg_init_scalars(RcgState S, const double* __restrict__ part_r
     }
 }
 
-// alpha = gamma / p^T q from the matvec's partials (fixed order; 0 if p^T q is
-// not positive).
-__global__ void k_rcg_alpha(RcgState S, const double* __restrict__ part_pq, int nblkC) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int k = blockIdx.x;
-    if (S.done[k]) return;
-    const double d = block_sum(part_pq + (int64_t)k * nblkC, nblkC);
-    if (threadIdx.x == 0) S.alpha[k] = (d > 0.0) ? S.gam[k] / d : 0.0;
+// Threads and blocks per column of the two streaming kernels: two blocks per SM
+// over all columns (every block repeats its column's sum, 0.4 us of FP64 pipe,
+// so four times as many blocks took 15 + 17 us instead of 8 + 10 for 4 columns
+// of 524,288 values).
+static const int CG_THREADS = 512;
+static int rcg_blocks(int nrhs) { return std::max(1, 304 / nrhs); }   // <= cg_blocks(nrhs)
+
+// Sum of part[0 .. n) in a fixed order, valid in thread 0: by the first four
+// warps, one per scheduler, since an FP64 instruction of a warp holds its
+// scheduler's FP64 pipe for 64 cycles (for the same reason thread 0 alone
+// divides, and the others get FP32 values).  red: four doubles of shared
+// memory, written here only.
+__device__ __forceinline__ double total128(const double* __restrict__ part, int n, double* red) {
+    if (threadIdx.x < 128) {
+        double v = 0.0;
+        for (int b = threadIdx.x; b < n; b += 128) v += part[b];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    }
+    __syncthreads();
+    return threadIdx.x == 0 ? (red[0] + red[1]) + (red[2] + red[3]) : 0.0;
 }
 
-// X += alpha P in double-float (Xh + Xl, FP32 instructions only), R -= alpha Q
-// (FP32); partials of ||R||^2 in double-float.  Streaming: five vectors read,
-// three written, from L2 where they fit (4 columns of 524,288 or
-// 152,950 values: 15.8 and 11.6 us with FP64 shuffle trees and, for odd p,
-// scalar accesses; 9 us on average now).
-__global__ void __launch_bounds__(256) k_rcg_update(float* __restrict__ Xh, float* __restrict__ Xl,
-                                                    float* __restrict__ R, const float* __restrict__ P,
-                                                    const float* __restrict__ Q, int64_t ld, RcgState S,
+// alpha = gamma / p^T q (0 if p^T q is not positive), R -= alpha Q (FP32);
+// partials of ||R||^2 in double-float.  Streaming: two vectors read, one
+// written, from L2 where they fit.
+__global__ void __launch_bounds__(CG_THREADS) k_rcg_update(float* __restrict__ R, const float* __restrict__ Q, int64_t ld,
+                                                    RcgState S, const double* __restrict__ part_pq, int npq,
                                                     double* __restrict__ part_rr) {
+    __shared__ double red[4];
+    __shared__ float coef;
     pdl_wait();
     pdl_launch_dependents();
     const int k = blockIdx.y;
     if (S.done[k]) return;   // finished columns keep x and r
-    const double a = S.alpha[k];
-    const float af = (float)a;
-    float ahi, alo;
-    df_split(a, ahi, alo);
-    const int64_t off = (int64_t)k * ld;
+    const int64_t off = (int64_t)k * ld, step = (int64_t)gridDim.x * blockDim.x * 4;
+    int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    float r[4], q[4];
+    if (x < ld) {   // in flight during the sum
+        load_vec<float, 4>(R + off + x, r);
+        load_vec<float, 4>(Q + off + x, q);
+    }
+    const double g = threadIdx.x == 0 ? S.gam[k] : 0.0;
+    const double d = total128(part_pq + (int64_t)k * npq, npq, red);
+    if (threadIdx.x == 0) {
+        const double a = d > 0.0 ? g / d : 0.0;
+        coef = (float)a;
+        if (blockIdx.x == 0) {
+            S.alpha[k] = a;
+            S.gold[k] = g;
+        }
+    }
+    __syncthreads();
+    const float af = coef;
     DotAcc<float> nrm;
-    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; x < ld; x += (int64_t)gridDim.x * blockDim.x * 4) {
-        const int64_t o = off + x;
-        float r[4], pv[4], qv[4], xh[4], xl[4];
-        load_vec<float, 4>(R + o, r);
-        load_vec<float, 4>(P + o, pv);
-        load_vec<float, 4>(Q + o, qv);
-        load_vec<float, 4>(Xh + o, xh);
-        load_vec<float, 4>(Xl + o, xl);
+    while (x < ld) {
+        float rn[4], qn[4];
+        if (x + step < ld) {
+            load_vec<float, 4>(R + off + x + step, rn);
+            load_vec<float, 4>(Q + off + x + step, qn);
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            df_axpy(xh[e], xl[e], ahi, alo, pv[e]);
-            r[e] -= af * qv[e];
+            r[e] -= af * q[e];
             nrm.add_prod(r[e], r[e]);
         }
-        store_vec<float, 4>(Xh + o, xh);
-        store_vec<float, 4>(Xl + o, xl);
-        store_vec<float, 4>(R + o, r);
+        store_vec<float, 4>(R + off + x, r);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) r[e] = rn[e], q[e] = qn[e];
+        x += step;
     }
     const double s = block_total(nrm);
     if (threadIdx.x == 0) part_rr[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
 // rr' = r^T r from the update's partials and gamma' = r^T z from part_rz (nrz
-// per column; NULL without a preconditioner: gamma' = rr'), both in a fixed
-// order; beta = gamma' / gamma.  Counts the iteration and asks for a
-// replacement when rr' has fallen 100x since the last one, reached the
-// target, is not finite, or the budget is spent.
-__global__ void k_rcg_beta(RcgState S, const double* __restrict__ part_rr, int nbc, const double* __restrict__ part_rz,
-                           int nrz, int maxit) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int k = blockIdx.x;
-    if (S.done[k]) return;
-    const double rr = block_sum(part_rr + (int64_t)k * nbc, nbc);
-    double g = rr;
-    if (part_rz) {
-        __syncthreads();   // block_sum's shared slots are reused
-        g = block_sum(part_rz + (int64_t)k * nrz, nrz);
-    }
-    if (threadIdx.x == 0) {
-        const double g0 = S.gam[k];
-        S.beta[k] = (g0 > 0.0) ? g / g0 : 0.0;
-        S.gam[k] = g;
-        S.rr[k] = rr;
-        const int it = S.iters[k] + 1;
-        S.iters[k] = it;
-        S.want[k] = (rr <= S.thr2[k] || rr <= 1e-2 * S.rr_ref[k] || !(rr == rr) || !(g == g) || it >= maxit) ? 1 : 0;
-    }
-}
-
-// P = Z + beta P (FP32); Z = R without a preconditioner.
-__global__ void __launch_bounds__(256) k_rcg_pupdate(float* __restrict__ P, const float* __restrict__ Z, int64_t ld,
-                                                     RcgState S) {
+// per column; NULL without a preconditioner: gamma' = rr'), beta = gamma' /
+// gamma; X += alpha P in double-float (Xh + Xl, FP32 instructions only) and P =
+// Z + beta P (Z = R without a preconditioner).  Streaming: four vectors read,
+// three written.  Block 0 counts the iteration and asks for a replacement when
+// rr' has fallen 100x since the last one, reached the target, is not finite, or
+// the budget is spent (no block reads what it writes).
+__global__ void __launch_bounds__(CG_THREADS) k_rcg_pupdate(float* __restrict__ Xh, float* __restrict__ Xl,
+                                                     float* __restrict__ P, const float* __restrict__ Z, int64_t ld,
+                                                     RcgState S, const double* __restrict__ part_rr, int nrr,
+                                                     const double* __restrict__ part_rz, int nrz, int maxit) {
+    __shared__ double red[8];
+    __shared__ float coef[3];
     pdl_wait();
     pdl_launch_dependents();
     const int k = blockIdx.y;
     if (S.done[k]) return;
-    const float b = (float)S.beta[k];
-    float* Pk = P + (int64_t)k * ld;
-    const float* Zk = Z + (int64_t)k * ld;
-    for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; x < ld; x += (int64_t)gridDim.x * blockDim.x * 4) {
-        float z[4], pv[4];
-        load_vec<float, 4>(Zk + x, z);
-        load_vec<float, 4>(Pk + x, pv);
+    const int64_t off = (int64_t)k * ld, step = (int64_t)gridDim.x * blockDim.x * 4;
+    int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    float z[4], pv[4], xh[4], xl[4];
+    auto load = [&](int64_t o) {
+        load_vec<float, 4>(Z + o, z);
+        load_vec<float, 4>(P + o, pv);
+        load_vec<float, 4>(Xh + o, xh);
+        load_vec<float, 4>(Xl + o, xl);
+    };
+    if (x < ld) load(off + x);   // in flight during the sums
+    double g0 = 0.0;
+    if (threadIdx.x == 0) {
+        g0 = S.gold[k];
+        df_split(S.alpha[k], coef[1], coef[2]);
+    }
+    const double rr = total128(part_rr + (int64_t)k * nrr, nrr, red);
+    const double rz = part_rz ? total128(part_rz + (int64_t)k * nrz, nrz, red + 4) : 0.0;
+    if (threadIdx.x == 0) {
+        const double g = part_rz ? rz : rr;
+        coef[0] = (float)((g0 > 0.0) ? g / g0 : 0.0);
+        if (blockIdx.x == 0) {
+            S.gam[k] = g;
+            S.rr[k] = rr;
+            const int it = S.iters[k] + 1;
+            S.iters[k] = it;
+            S.want[k] = (rr <= S.thr2[k] || rr <= 1e-2 * S.rr_ref[k] || !(rr == rr) || !(g == g) || it >= maxit) ? 1 : 0;
+        }
+    }
+    __syncthreads();
+    const float b = coef[0], ahi = coef[1], alo = coef[2];
+    while (x < ld) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) pv[e] = z[e] + b * pv[e];
-        store_vec<float, 4>(Pk + x, pv);
+        for (int e = 0; e < 4; ++e) {
+            df_axpy(xh[e], xl[e], ahi, alo, pv[e]);
+            pv[e] = z[e] + b * pv[e];
+        }
+        store_vec<float, 4>(Xh + off + x, xh);
+        store_vec<float, 4>(Xl + off + x, xl);
+        store_vec<float, 4>(P + off + x, pv);
+        x += step;
+        if (x < ld) load(off + x);
     }
 }
 
@@ -1564,8 +1605,8 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     S.gam = reinterpret_cast<double*>(sb);
     S.rr = S.gam + nrhs;
     S.alpha = S.rr + nrhs;
-    S.beta = S.alpha + nrhs;
-    S.rr_ref = S.beta + nrhs;
+    S.gold = S.alpha + nrhs;
+    S.rr_ref = S.gold + nrhs;
     S.thr2 = S.rr_ref + nrhs;
     S.want = reinterpret_cast<int*>(S.thr2 + nrhs);
     S.done = S.want + nrhs;
@@ -1583,7 +1624,7 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     float* Xl = Xh + (size_t)nrhs * ld;
 
     dim3 gv(RED_BLOCKS, nrhs);
-    dim3 gc(nbc, nrhs);
+    dim3 gc(nbc, nrhs), gl(rcg_blocks(nrhs), nrhs);
     const int tbeta = std::max(32, ((nrhs + 31) / 32) * 32);
     if (ld > p) {   // the matvec writes the first p values of Q and Z only
         KRY_CUDA(cudaMemset2DAsync(Q + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
@@ -1598,9 +1639,7 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     if (pre) matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, nullptr);   // z = M^-1 r
     k_rcg_init_scalars<<<nrhs, FIN_THREADS, 0, st>>>(S, part_rr, nbc, part_rz, nblkC, nrhs, ctx->tolbuf.as<double>());
     KRY_CHECK_LAUNCH();
-    if (pre) {   // p = z (beta = 0)
-        launch_pdl(k_rcg_pupdate, gc, dim3(256), 0, st, P, (const float*)Z, ld, S);
-    }
+    if (pre) KRY_CUDA(cudaMemcpyAsync(P, Z, vb, cudaMemcpyDeviceToDevice, st));   // p = z
     int* hflag = reinterpret_cast<int*>(ctx->host_pinned);
     const int poll = 8;
     nrm.assign(2 * nrhs, 0.0);
@@ -1613,12 +1652,9 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
         // columns that have converged are not transformed (pairs of finished
         // columns skip every pass)
         matvec_ex<float>(ctx, e, P, ld, nullptr, Q, ld, nrhs, part_pq, nblkC, vpt, S.done);
-        launch_pdl(k_rcg_alpha, dim3(nrhs), dim3(FIN_THREADS), 0, s2, S, part_pq, nblkC);
-        launch_pdl(k_rcg_update, gc, dim3(256), 0, s2, Xh, Xl, R, P, Q, ld, S, part_rr);
+        launch_pdl(k_rcg_update, gl, dim3(CG_THREADS), 0, s2, R, Q, ld, S, part_pq, nblkC, part_rr);
         if (pre) matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, S.done);
-        launch_pdl(k_rcg_beta, dim3(nrhs), dim3(FIN_THREADS), 0, s2, S, part_rr, nbc, (const double*)part_rz, nblkC,
-                   maxit);
-        launch_pdl(k_rcg_pupdate, gc, dim3(256), 0, s2, P, (const float*)Z, ld, S);
+        launch_pdl(k_rcg_pupdate, gl, dim3(CG_THREADS), 0, s2, Xh, Xl, P, Z, ld, S, part_rr, (int)gl.x, part_rz, nblkC, maxit);
     };
     // Iterations run in blocks of `poll`.  The first block runs directly (it
     // sizes every buffer); later blocks replay one captured graph.
