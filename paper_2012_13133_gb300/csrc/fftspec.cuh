@@ -17,10 +17,9 @@
 // address per two values, and one barrier-separated stage fewer where L =
 // 512 or 8192 (H = 256 = 16^2, 4096 = 16^3).  Measured against one length-L
 // transform per thread group with 8-byte accesses: 4 vectors on 4096^2 2,070 ->
-// 1,263 us, 32 vectors on 512^2 153 -> 121 us, 64 vectors on 1024^2 945 -> 921 us.
-// What bounds the passes now is the shared-memory and L1 pipe (column pass: 860
-// wavefronts per warp, 512 of them the four exchanges, 68% busy), then latency at
-// 16 warps per SM.
+// 1,263 us.  What bounds the passes now is the shared-memory and L1 pipe (column
+// pass of side 2048, before mvwide.cuh took it over: 860 wavefronts per warp, 512
+// of them the four exchanges, 68% busy), then latency at 16 warps per SM.
 //
 // Stages (Stockham after Govindaraju et al., SC 2008): radix R0 = 2^(log2 H
 // mod 4) (16 when that is 1) first, then radix 16; a thread holds 16 packed

@@ -369,12 +369,13 @@ static void run_passes(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t l
             a.nvec = nvec; a.bits = ctx->cellbits.as<uint2>(); a.wpr = (n2 + 31) / 32;
             a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2;
             spec_shape(ctx, e, nvec, &a.G, &a.C);
-            a.logCs = ilog2(std::max(4, a.C));   // tile rows of at least a 32-byte sector
+            a.logCs = ilog2(std::min(32, std::max(4, a.C)));   // tile rows of 1 to 8 32-byte sectors
             a.slab = static_cast<float2*>(slab); a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
             a.tau2 = tau2; a.tau2v = tau2v; a.dots = dots; a.nds = nds;
             a.twf = ctx->spec_tab.as<float4>();
             a.twi = a.twf + kspec::TWF_WORDS;
             a.post = reinterpret_cast<const float2*>(a.twi + kspec::TWI_WORDS);
+            a.tww = a.post + kspec::POST_WORDS;
             a.skip = skip;
             for (a.pair0 = 0; a.pair0 < npairs; a.pair0 += ppb) {
                 a.np = std::min(ppb, npairs - a.pair0);

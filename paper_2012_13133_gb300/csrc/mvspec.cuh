@@ -30,9 +30,9 @@ namespace kspec {
 __host__ __device__ constexpr int lt_of(int B) { return (1 << (B - 1)) / 16; }
 constexpr int nt_of(int B, int TH) { return TH / lt_of(B); }
 // Registers: 64 of a thread's 128 hold the transform: 512 threads per SM.
-// (Measured on the 64-vector 1024^2 call: 96 registers and 640 threads 1195 us
-// against 913 us; 32 values a thread, one shared-memory exchange fewer, but 8
-// warps per SM, 982 us.)
+// (Measured on side 2048 with 16 packed values, 64 vectors: 96 registers and 640
+// threads 1195 us against 913 us; 32 packed values, one shared-memory exchange
+// fewer, but 8 warps per SM, 982 us.)
 constexpr int minb(int B, int TH) { return TH >= 512 ? 1 : 512 / TH; }
 
 // Shared-memory bytes of a block.
@@ -40,11 +40,20 @@ constexpr size_t smem_bytes(int B, int TH) {
     return (size_t)((1 << (B - 1)) + ((1 << (B - 1)) >> pad_shift(1 << (B - 1)))) * nt_of(B, TH) * 16;
 }
 
+// Torus sides whose passes hold 32 values per thread (mvwide.cuh).
+__host__ __device__ constexpr bool is_wide(int B) { return B == 10 || B == 11; }
+
 // Offset within a column of M1 eigenvalues of torus row k1 = 2 k + q, k = t +
 // s lt, lt = threads per transform: word (s/2) lt + t holds (s even: q = 0, 1;
-// s odd: q = 0, 1).
+// s odd: q = 0, 1).  Sides with 32 values per thread: k = t + s lt/2, and word
+// (s/4) lt + 2t + q holds s .. s + 3.
 __host__ __device__ __forceinline__ int lam_slot(int k1, int M1, int lt) {
-    const int q = k1 & 1, k = k1 >> 1, t = k & (lt - 1), s = k / lt;
+    const int q = k1 & 1, k = k1 >> 1;
+    if (M1 == 1024 || M1 == 2048) {
+        const int h = lt >> 1, t = k & (h - 1), s = k / h;
+        return ((s >> 2) * lt + 2 * t + q) * 4 + (s & 3);
+    }
+    const int t = k & (lt - 1), s = k / lt;
     return ((s >> 1) * lt + t) * 4 + (s & 1) * 2 + q;
 }
 
@@ -65,6 +74,28 @@ __device__ __forceinline__ void cell_indices(const uint2* __restrict__ w, int wp
         const unsigned bit = 1u << (j & 31);
         const bool on = live && (b[m].x & bit) != 0u && (j >> 5) < wpr;
         q[m] = on ? (int)(b[m].y + __popc(b[m].x & (bit - 1u))) : -1;
+    }
+}
+
+// Pass C's v . K v partials of a block, in a fixed order and in double-float:
+// FP64 shuffle trees would hold the FP64 pipe (one warp instruction per 64
+// cycles) for longer than the pass's stores take.
+template <int TH>
+__device__ __forceinline__ void block_dots(kry::DFAcc& acc_a, kry::DFAcc& acc_b, float2 (&red)[2][TH / 32], bool has_b,
+                                           double* __restrict__ dots, int ndot_stride, int va, int vb) {
+    kry::df_warp_sum(acc_a.hi, acc_a.lo);
+    kry::df_warp_sum(acc_b.hi, acc_b.lo);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) {
+        red[0][w] = make_float2(acc_a.hi, acc_a.lo);
+        red[1][w] = make_float2(acc_b.hi, acc_b.lo);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 && (threadIdx.x == 0 || has_b)) {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll
+        for (int k = 0; k < TH / 32; ++k) kry::df_add(hi, lo, red[threadIdx.x][k].x, red[threadIdx.x][k].y);
+        dots[(int64_t)(threadIdx.x ? vb : va) * ndot_stride + blockIdx.x] = (double)hi + (double)lo;
     }
 }
 
@@ -283,25 +314,7 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
             }
         }
     }
-    if (dots != nullptr) {
-        // fixed-order block reduction in double-float: FP64 shuffle trees would
-        // hold the FP64 pipe (one warp instruction per 64 cycles) for longer
-        // than the pass's stores take
-        kry::df_warp_sum(acc_a.hi, acc_a.lo);
-        kry::df_warp_sum(acc_b.hi, acc_b.lo);
-        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        if (lane == 0) {
-            red[0][w] = make_float2(acc_a.hi, acc_a.lo);
-            red[1][w] = make_float2(acc_b.hi, acc_b.lo);
-        }
-        __syncthreads();
-        if (threadIdx.x < 2 && (threadIdx.x == 0 || has_b)) {
-            float hi = 0.f, lo = 0.f;
-#pragma unroll
-            for (int k = 0; k < TH / 32; ++k) kry::df_add(hi, lo, red[threadIdx.x][k].x, red[threadIdx.x][k].y);
-            dots[(int64_t)(threadIdx.x ? vb : va) * ndot_stride + blockIdx.x] = (double)hi + (double)lo;
-        }
-    }
+    if (dots != nullptr) block_dots<TH>(acc_a, acc_b, red, has_b, dots, ndot_stride, va, vb);
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -329,6 +342,7 @@ struct SpecArgs {
     const float4* twf;
     const float4* twi;
     const float2* post;
+    const float2* tww;   // twiddles of the 32-value passes
     const int* skip;
 };
 
@@ -349,8 +363,9 @@ bool launch_b(const SpecArgs& a, cudaStream_t st);
 bool launch_c(const SpecArgs& a, cudaStream_t st);
 
 // Words (16 bytes) of the tables that fill_tables writes: forward twiddles,
-// inverse twiddles, post factors (two per word).
-constexpr int TABLE_WORDS = TWF_WORDS + TWI_WORDS + POST_WORDS / 2;
+// inverse twiddles, post factors and the 32-value passes' twiddles (two per word).
+constexpr int TWW_WORDS = 32 + 16 * 32 + 16 * 64;
+constexpr int TABLE_WORDS = TWF_WORDS + TWI_WORDS + POST_WORDS / 2 + TWW_WORDS / 2;
 void fill_tables(float4* tab_dev, cudaStream_t st);
 
 }  // namespace kspec

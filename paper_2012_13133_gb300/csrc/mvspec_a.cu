@@ -2,6 +2,7 @@
 // (log2 M2, threads per block), the block sizes and the twiddle tables.
 #include "kry_internal.cuh"
 #include "mvspec.cuh"
+#include "mvwide.cuh"
 
 namespace kspec {
 
@@ -43,7 +44,7 @@ __global__ void k_tables(float4* __restrict__ tab) {
         const int r = w - 4 * (ns - 2), e = r / ns, k = r - e * ns;
         const float2 a = cos_tan(entry_turns(2 * e, ns, k)), b = cos_tan(entry_turns(2 * e + 1, ns, k));
         tab[i] = make_float4(a.x, a.y, b.x, b.y);
-    } else if (i < TABLE_WORDS) {
+    } else if (i < TWF_WORDS + TWI_WORDS + POST_WORDS / 2) {
         float2 f[2];
         for (int q = 0; q < 2; ++q) {
             const int w = 2 * (i - TWF_WORDS - TWI_WORDS) + q;   // sections of h words from h - 32
@@ -53,6 +54,12 @@ __global__ void k_tables(float4* __restrict__ tab) {
             f[q] = make_float2((float)c, (float)s);
         }
         tab[i] = make_float4(f[0].x, f[0].y, f[1].x, f[1].y);
+    } else if (i < TABLE_WORDS) {
+        const int w = 2 * (i - TWF_WORDS - TWI_WORDS - POST_WORDS / 2);
+        const int ns = w < wide_section(16) ? 1 : w < wide_section(32) ? 16 : 32;
+        const int r = w - wide_section(ns), e = r / (2 * ns), k = (r - e * 2 * ns) >> 1;
+        const float2 a = cos_tan(entry_turns(e, ns, k)), b = cos_tan(entry_turns(e, ns, k + 0.5));
+        tab[i] = make_float4(a.x, a.y, b.x, b.y);
     }
 }
 
@@ -68,11 +75,18 @@ struct RunA {
     template <int B, int TH>
     bool run() const {
         constexpr int NT = nt_of(B, TH);
-        auto k = ks_pass_a<B, TH>;
-        KRY_ALLOW_MAX_SMEM(k);
         dim3 grid((a.n1 + NT - 1) / NT, a.np);
-        launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0, a.bits, a.wpr,
-                   a.n1, a.n2, a.logCs, reinterpret_cast<float4*>(a.slab), a.twf, a.skip);
+        if constexpr (is_wide(B)) {
+            auto k = kw_pass_a<B, TH>;
+            KRY_ALLOW_MAX_SMEM(k);
+            launch_pdl(k, grid, dim3(TH), wide_smem(B, TH), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0, a.bits, a.wpr,
+                       a.n1, a.logCs, a.slab, a.tww, a.skip);
+        } else {
+            auto k = ks_pass_a<B, TH>;
+            KRY_ALLOW_MAX_SMEM(k);
+            launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0, a.bits, a.wpr,
+                       a.n1, a.n2, a.logCs, reinterpret_cast<float4*>(a.slab), a.twf, a.skip);
+        }
         return true;
     }
 };
