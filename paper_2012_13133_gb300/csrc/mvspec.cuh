@@ -33,7 +33,14 @@ constexpr int nt_of(int B, int TH) { return TH / lt_of(B); }
 // (Measured on side 2048 with 16 packed values, 64 vectors: 96 registers and 640
 // threads 1195 us against 913 us; 32 packed values, one shared-memory exchange
 // fewer, but 8 warps per SM, 982 us.)
-constexpr int minb(int B, int TH) { return TH >= 512 ? 1 : 512 / TH; }
+// Sides up to 256 are latency, not throughput: their passes load everything as
+// soon as they may, into up to 255 registers (4 vectors on 128^2 10.7 -> 9.6 us, a
+// CG iteration on them 24.1 -> 22.1 us).
+constexpr bool early(int B) { return B <= 8; }
+constexpr int minb(int B, int TH) {
+    const int resident = early(B) ? 256 : 512;
+    return TH >= resident ? 1 : resident / TH;
+}
 
 // Shared-memory bytes of a block.
 constexpr size_t smem_bytes(int B, int TH) {
@@ -97,6 +104,13 @@ __device__ __forceinline__ void block_dots(kry::DFAcc& acc_a, kry::DFAcc& acc_b,
         for (int k = 0; k < TH / 32; ++k) kry::df_add(hi, lo, red[threadIdx.x][k].x, red[threadIdx.x][k].y);
         dots[(int64_t)(threadIdx.x ? vb : va) * ndot_stride + blockIdx.x] = (double)hi + (double)lo;
     }
+}
+
+// Post factors of a thread's E outputs t + s LT.
+template <int E, int LT>
+__device__ __forceinline__ void load_post(float2 (&f)[E], const float2* __restrict__ pw) {
+#pragma unroll
+    for (int s = 0; s < E; ++s) f[s] = __ldg(pw + s * LT);
 }
 
 // ---------------------------------------------------------------- pass A
@@ -177,6 +191,8 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
     const float4* lam = reinterpret_cast<const float4*>(lamP + theta * lam_stride + (int64_t)col * L) + t;
     const float2* pw = post + (H - 32) + t;
+    float2 f[E];
+    if constexpr (early(B)) load_post<E, LT>(f, pw);
     pdl_wait();   // the slab comes from pass A
     pdl_launch_dependents();
     if (skip) {
@@ -190,11 +206,16 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     auto lds = [&](int c) { return sb[tb + soff<PS, NT>(c)]; };
     auto sts = [&](int bo, int c, c2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
     c2 v[E];
+    float4 lw[E / 2];
     {
         float2 x[E];
 #pragma unroll
         for (int m = 0; m < E; ++m)
             x[m] = (t + m * LT < n1) ? blk[(int64_t)(m * LT) << logCs] : make_float2(0.f, 0.f);
+        if constexpr (early(B)) {
+#pragma unroll
+            for (int s = 0; s < E / 2; ++s) lw[s] = __ldg(lam + s * LT);
+        }
         first_forward<B>(x, t, sts);
     }
     later_stages<B, 1, false>(v, tw1, t, twf, lds, sts);
@@ -202,7 +223,7 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     c2 w[E];
 #pragma unroll
     for (int s = 0; s < E; s += 2) {
-        const float4 l = __ldg(lam + (s >> 1) * LT);
+        const float4 l = early(B) ? lw[s >> 1] : __ldg(lam + (s >> 1) * LT);
         const c2 a = v[brev(s, P::LE)], b = v[brev(s + 1, P::LE)];
         const u64 la = pk(l.x, l.y), lb = pk(l.z, l.w);
         w[s] = {mul2(a.r, la), mul2(a.i, la)};
@@ -216,9 +237,9 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     for (int s = 0; s < E; ++s) {
         if (t + s * LT < n1) {
             const c2 z = v[brev(s, P::LE)];
-            const float2 re = upk(z.r), im = upk(z.i), f = __ldg(pw + s * LT);
-            blk[(int64_t)(s * LT) << logCs] = make_float2(fmaf(f.x, re.y, fmaf(-f.y, im.y, re.x)),
-                                                          fmaf(f.x, im.y, fmaf(f.y, re.y, im.x)));
+            const float2 re = upk(z.r), im = upk(z.i), g = early(B) ? f[s] : __ldg(pw + s * LT);
+            blk[(int64_t)(s * LT) << logCs] = make_float2(fmaf(g.x, re.y, fmaf(-g.y, im.y, re.x)),
+                                                          fmaf(g.x, im.y, fmaf(g.y, re.y, im.x)));
         }
     }
 }
@@ -243,6 +264,8 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     StageTw<16> tw1;   // constant tables: their latency lies behind the kernel before
     load_twiddles<E, P::R0, true>(tw1, twi, t);
     const float2* pw = post + (H - 32) + t;
+    float2 pf[E];
+    if constexpr (early(B)) load_post<E, LT>(pf, pw);
     pdl_wait();   // the slab comes from pass B
     pdl_launch_dependents();
     const int row = blockIdx.x * NT + n;
@@ -255,6 +278,16 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     const int tb = soff<PS, NT>(t);
     auto lds = [&](int c) { return sb[tb + soff<PS, NT>(c)]; };
     auto sts = [&](int bo, int c, c2 z) { sb[soff<PS, NT>(bo) + soff<PS, NT>(c)] = z; };
+    const float* pa = vin + (int64_t)va * ld_in;
+    const float* pb = has_b ? vin + (int64_t)vb * ld_in : pa;
+    const uint2* bw = bits + (int64_t)min(row, n1 - 1) * wpr;
+    int q[E];
+    float2 x[E];
+    auto load_cells = [&]() {
+        cell_indices<LT, E>(bw, wpr, live, t, q);
+#pragma unroll
+        for (int i = 0; i < E; ++i) x[i] = make_float2(pa[max(q[i], 0)], pb[max(q[i], 0)]);
+    };
     c2 v[E];
     {
         const int logk = logCs - 1;
@@ -266,6 +299,7 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
             const float4 f = in[(((int64_t)(k >> logk) * n1 + min(row, n1 - 1)) << logk) + (k & ((1 << logk) - 1))];
             w[s] = {pk(f.x, f.z), pk(f.y, f.w)};
         }
+        if constexpr (early(B)) load_cells();
         first_inverse<B>(w, t, sts);
     }
     later_stages<B, 1, true>(v, tw1, t, twi, lds, sts);
@@ -275,42 +309,32 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
         const float t2 = (float)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
-        const float* pa = vin + (int64_t)va * ld_in;
-        const float* pb = has_b ? vin + (int64_t)vb * ld_in : pa;
         float* oa = vout + (int64_t)va * ld_out;
         float* ob = vout + (int64_t)vb * ld_out;
-        const uint2* w = bits + (int64_t)min(row, n1 - 1) * wpr;
-        constexpr int CH = 16;   // cells at a time (their indices and inputs are live together)
+        if constexpr (!early(B)) load_cells();
+        float2 y[E];
 #pragma unroll
-        for (int s0 = 0; s0 < E; s0 += CH) {
-            int q[CH];
-            cell_indices<LT, CH>(w, wpr, live, t + s0 * LT, q);
-            float2 x[CH], y[CH];
+        for (int i = 0; i < E; ++i) {
+            const c2 z = v[brev(i, P::LE)];
+            const float2 re = upk(z.r), im = upk(z.i), f = early(B) ? pf[i] : __ldg(pw + i * LT);
+            y[i] = make_float2(fmaf(f.x, re.y, fmaf(-f.y, im.y, re.x)), fmaf(f.x, im.y, fmaf(f.y, re.y, im.x)));
+        }
 #pragma unroll
-            for (int i = 0; i < CH; ++i) x[i] = make_float2(pa[max(q[i], 0)], pb[max(q[i], 0)]);
+        for (int i = 0; i < E; ++i) {
+            x[i] = make_float2(x[i].x * sa, x[i].y * sbv);
+            y[i] = make_float2(y[i].x + t2 * x[i].x, y[i].y + t2 * x[i].y);
+        }
 #pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                const c2 z = v[brev(s0 + i, P::LE)];
-                const float2 re = upk(z.r), im = upk(z.i), f = __ldg(pw + (s0 + i) * LT);
-                y[i] = make_float2(fmaf(f.x, re.y, fmaf(-f.y, im.y, re.x)), fmaf(f.x, im.y, fmaf(f.y, re.y, im.x)));
-            }
+        for (int i = 0; i < E; ++i) {
+            if (q[i] >= 0) oa[q[i]] = y[i].x;
+            if (q[i] >= 0 && has_b) ob[q[i]] = y[i].y;
+        }
+        if (dots) {
 #pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                x[i] = make_float2(x[i].x * sa, x[i].y * sbv);
-                y[i] = make_float2(y[i].x + t2 * x[i].x, y[i].y + t2 * x[i].y);
-            }
-#pragma unroll
-            for (int i = 0; i < CH; ++i) {
-                if (q[i] >= 0) oa[q[i]] = y[i].x;
-                if (q[i] >= 0 && has_b) ob[q[i]] = y[i].y;
-            }
-            if (dots) {
-#pragma unroll
-                for (int i = 0; i < CH; ++i) {
-                    const bool on = q[i] >= 0;   // what lies in unobserved cells stays out of the sums
-                    acc_a.add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
-                    acc_b.add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
-                }
+            for (int i = 0; i < E; ++i) {
+                const bool on = q[i] >= 0;   // what lies in unobserved cells stays out of the sums
+                acc_a.add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
+                acc_b.add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
             }
         }
     }
