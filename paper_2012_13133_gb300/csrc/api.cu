@@ -459,7 +459,8 @@ kry_status kry_create(kry_ctx** out, int device, void* cuda_stream) {
         KRY_CUDA(cudaDeviceGetDefaultMemPool(&pool, device));
         uint64_t keep = UINT64_MAX;
         KRY_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        KRY_CUDA(cudaMallocHost(&ctx->host_pinned, 4096 * sizeof(double)));
+        ctx->host_cap = 4096 * sizeof(double);
+        KRY_CUDA(cudaMallocHost(&ctx->host_pinned, ctx->host_cap));
         kry::init_twiddles(ctx);
         KRY_CUDA(cudaStreamSynchronize(ctx->stream));
         return KRY_OK;

@@ -168,7 +168,8 @@ struct kry_ctx {
         DevBuf cellptr, ent_site, ent_w64, ent_w32, cnt;
         DevBuf grid32, grid64;
     } sites;
-    double* host_pinned = nullptr;   // pinned host scratch (4096 doubles)
+    double* host_pinned = nullptr;   // pinned host scratch (4096 doubles at least)
+    size_t host_cap = 0;             // its bytes
     int num_sms = 0;
     int max_smem_optin = 0;
 

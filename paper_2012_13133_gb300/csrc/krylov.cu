@@ -1053,6 +1053,19 @@ void logdet_batched(kry_ctx* ctx, const kry_embed* e, int nprobe, int nsteps, ui
 
 // ------------------------------------------------------------------ CG
 
+// The pinned host scratch as n ints, grown where a batch has more columns than it
+// holds (no copy into it is in flight: every user waits for its own).
+static int* host_ints(kry_ctx* ctx, size_t n) {
+    if (n * sizeof(int) > ctx->host_cap) {
+        double* more = nullptr;
+        KRY_CUDA(cudaMallocHost(&more, n * sizeof(int)));
+        cudaFreeHost(ctx->host_pinned);
+        ctx->host_pinned = more;
+        ctx->host_cap = n * sizeof(int);
+    }
+    return reinterpret_cast<int*>(ctx->host_pinned);
+}
+
 struct CgState {
     double* rr;      // [nrhs] r^T r
     double* alpha;   // [nrhs]
@@ -1187,7 +1200,7 @@ static int cg_inner(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t l
     KRY_CHECK_LAUNCH();
     k_cg_init_scalars<<<nrhs, FIN_THREADS, 0, st>>>(S, part, RED_BLOCKS, nrhs, tol_dev);
     KRY_CHECK_LAUNCH();
-    int* hdone = reinterpret_cast<int*>(ctx->host_pinned);
+    int* hdone = host_ints(ctx, nrhs);
     int it = 0;
     const int poll = 8;
     for (; it < maxit; ++it) {
@@ -1654,7 +1667,6 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
 
     dim3 gv(RED_BLOCKS, nrhs);
     dim3 gc(nbc, nrhs), gl(rcg_blocks(nrhs), nrhs);
-    const int tbeta = std::max(32, ((nrhs + 31) / 32) * 32);
     if (ld > p) {   // the matvec writes the first p values of Q and Z only
         KRY_CUDA(cudaMemset2DAsync(Q + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
         if (pre) KRY_CUDA(cudaMemset2DAsync(Z + p, ld * sizeof(float), 0, (ld - p) * sizeof(float), nrhs, st));
@@ -1669,7 +1681,7 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
     k_rcg_init_scalars<<<nrhs, FIN_THREADS, 0, st>>>(S, part_rr, nbc, part_rz, nblkC, nrhs, ctx->tolbuf.as<double>());
     KRY_CHECK_LAUNCH();
     if (pre) KRY_CUDA(cudaMemcpyAsync(P, Z, vb, cudaMemcpyDeviceToDevice, st));   // p = z
-    int* hflag = reinterpret_cast<int*>(ctx->host_pinned);
+    int* hflag = host_ints(ctx, nrhs);
     const int poll = 8;
     *fresh = false;
     // one CG iteration on ctx->stream (the capture stream while capturing)
@@ -1708,7 +1720,7 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
             // the columns that ask for it, and the FP64 matvec transforms only
             // their pairs.
             const int all = nrhs <= 8 ? 1 : 0;
-            k_rcg_select<<<1, tbeta, 0, st>>>(S, nrhs, sel, all);
+            k_rcg_select<<<(nrhs + 255) / 256, 256, 0, st>>>(S, nrhs, sel, all);
             KRY_CHECK_LAUNCH();
             to_f64(sel);
             true_residual(ctx, e, B, ldb, X, ldx, nrhs, R64, ctx->kxbuf.as<double>(), vpt, sel);

@@ -64,3 +64,32 @@ def test_preconditioned_residuals(n1, n2, nrhs):
         assert bool(torch.all(rn <= 1e-6 * 1.001 * B.norm(dim=1)))
     assert pre[1] < plain[1]
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ncov,settings", [(1, 600), (8, 900)])
+def test_search_of_many_columns(ncov, settings):
+    """Batches past 1024 columns (a block's most threads) and past 8192 (the host flags' first size):
+    every setting's result is the one that it has alone."""
+    import torch
+
+    from paper_2012_13133_gb300 import inputs as I
+    from paper_2012_13133_gb300 import kry
+    n1, n2 = 12, 10
+    g = torch.Generator().manual_seed(ncov)
+    mask = np.random.default_rng(3).random((n1, n2)) >= 0.2
+    ctx = kry.Context(0)
+    p = ctx.set_mask(torch.from_numpy(mask.astype(np.uint8)).cuda())
+    y = torch.randn(p, generator=g, dtype=torch.float64).cuda()
+    X = torch.randn((ncov, p), generator=g, dtype=torch.float64).cuda()
+    thetas = [I.Cov(1.0, 0.05 + 0.1 * k / settings, 0.5, 0.3) for k in range(settings)]
+    opts = kry.Opts(prec=kry.KRY_F32, nprobe=2, nsteps=10, seed=1, rtol=RTOL, maxit=200, reorth=1)
+    assert settings * (ncov + 1) > (1024 if ncov == 1 else 8192)
+    r = ctx.profile_loglik(y, X, thetas, opts)
+    assert r["status"] == kry.KRY_OK
+    for k in (0, settings // 2, settings - 1):
+        one = ctx.profile_loglik(y, X, [thetas[k]], opts)
+        # solves to 1e-8 of a system of condition number below 100, at most 9 columns: 1e-5 of the quadratic form
+        assert abs(r["loglik"][k] - one["loglik"][0]) <= 1e-5 * abs(one["loglik"][0]) + 1e-5
+        assert abs(r["logdet"][k] - one["logdet"][0]) <= 1e-5 * p
+    ctx.close()
