@@ -483,8 +483,9 @@ void kry_server_destroy(kry_server* server);
  * per batch (all, or chunks whose FFT intermediate fits ~32/64 MB of L2) --
  * and keeps the fastest for (M1, M2, precision, batch-size bucket) in ctx;
  * every later matvec, log-det, solve and likelihood on ctx with that shape
- * uses it.  Reports the best time per call (ms) and the chosen schedule
- * (host pointers, each may be NULL).  Allocates and frees two test buffers
+ * uses it.  Reports the best time per call (ms) and the chosen schedule in
+ * the form that kry_set_schedule takes (host pointers, each may be NULL; 0 =
+ * library default).  Allocates and frees two test buffers
  * of nvec * p values.  Synchronises the stream. */
 kry_status kry_autotune(kry_ctx* ctx, const kry_embed* e, int32_t nvec, double* best_ms,
                         int32_t* rows_per_block, int32_t* cols_per_block, int32_t* pairs_per_batch);

@@ -755,7 +755,7 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
                 }
             }
         }
-        // report the blocks that run
+        // pin the blocks that run, and report them
         if (dbl) {
             kf64::Shape row, col;
             ctx->tuned[key] = bs;
@@ -767,6 +767,10 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
             spec_shape(ctx, e, nvec, &bs.g16, &bs.c16);
         }
         ctx->tuned[key] = bs;
+        // the default blocks of the shortest tori hold more transforms than kry_set_schedule takes:
+        // reported as 0, which names the same blocks
+        for (int* b : {&bs.g16, &bs.c16})
+            if (*b > 16) *b = 0;
     } else {
         if (had) ctx->tuned[key] = prev;
         best = time_sched<T>(ctx, e, tv.as<T>(), to.as<T>(), nvec, 3);

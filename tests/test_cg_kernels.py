@@ -84,7 +84,7 @@ def test_search_of_many_columns(ncov, settings):
     X = torch.randn((ncov, p), generator=g, dtype=torch.float64).cuda()
     thetas = [I.Cov(1.0, 0.05 + 0.1 * k / settings, 0.5, 0.3) for k in range(settings)]
     opts = kry.Opts(prec=kry.KRY_F32, nprobe=2, nsteps=10, seed=1, rtol=RTOL, maxit=200, reorth=1)
-    assert settings * (ncov + 1) > (1024 if ncov == 1 else 8192)
+    assert settings * ((ncov + 2) & ~1) > (1024 if ncov == 1 else 8192)   # columns [y, X] in pairs
     r = ctx.profile_loglik(y, X, thetas, opts)
     assert r["status"] == kry.KRY_OK
     for k in (0, settings // 2, settings - 1):
