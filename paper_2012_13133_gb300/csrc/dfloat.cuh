@@ -43,13 +43,74 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float ohi, float ol
     lo = __fadd_rn(__fadd_rn(lo, olo), t);
 }
 
-// Sum of (hi, lo) over a warp's lanes in a fixed tree order; valid in lane 0.
-__device__ __forceinline__ void df_warp_sum(float& hi, float& lo) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h = __shfl_down_sync(0xffffffffu, hi, o), l = __shfl_down_sync(0xffffffffu, lo, o);
-        df_add(hi, lo, h, l);
+// A sum across threads as three floats a + b + c.  Adding two of them with exact
+// first and second components leaves an error of about 2^-70 of the sum, so a tree
+// of these loses less than one of FP64 additions (2^-53), without the FP64 pipe.
+struct TFloat {
+    float a, b, c;
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+__device__ __forceinline__ void tf_add(TFloat& x, const TFloat& y) {
+    float s, e, t, f, u, g;
+    two_sum(x.a, y.a, s, e);
+    two_sum(x.b, y.b, t, f);
+    two_sum(t, e, u, g);
+    x = {s, u, __fadd_rn(__fadd_rn(x.c, y.c), __fadd_rn(f, g))};
+}
+
+__device__ __forceinline__ TFloat tf_xor(const TFloat& x, int o) {
+    return {__shfl_xor_sync(0xffffffffu, x.a, o), __shfl_xor_sync(0xffffffffu, x.b, o),
+            __shfl_xor_sync(0xffffffffu, x.c, o)};
+}
+
+// Block sums of N = 1 or 2 running dot products over a block of at most WARPS warps
+// in a fixed order: thread k WARPS returns the k-th, k < N.  Added as three floats;
+// where finite sums leave the FP32 range together, in FP64 (a warp's FP64
+// instruction holds its scheduler's FP64 pipe for 64 cycles on GB300: an FP64
+// shuffle tree in every block of a streaming kernel takes longer than the
+// streaming).  Two sums share a tree, each half a warp's lanes.
+template <int N, int WARPS>
+__device__ __forceinline__ double block_sums(const DFAcc (&acc)[N]) {
+    static_assert(N <= 2 && N * WARPS <= 32 && (WARPS & (WARPS - 1)) == 0, "a warp adds the warps' sums");
+    __shared__ __align__(16) TFloat red[N][WARPS];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    constexpr int HALF = 32 / N;
+    TFloat x = {acc[0].hi, acc[0].lo, 0.f};
+    if constexpr (N == 2) {
+        const TFloat y = {acc[1].hi, acc[1].lo, 0.f};
+        const bool second = lane >= 16;
+        const TFloat keep = second ? y : x, give = second ? x : y;
+        x = keep;
+        tf_add(x, tf_xor(give, 16));
     }
+#pragma unroll
+    for (int o = HALF / 2; o > 0; o >>= 1) tf_add(x, tf_xor(x, o));
+    const bool mine = (lane & (HALF - 1)) == 0;
+    if (mine) red[lane / HALF][w] = x;
+    if (!__syncthreads_or(mine && !isfinite(x.a))) {
+        if (w != 0) return 0.0;
+        const int k = min(lane / WARPS, N - 1), v = lane & (WARPS - 1);
+        x = v < nw ? red[k][v] : TFloat{0.f, 0.f, 0.f};
+#pragma unroll
+        for (int o = WARPS / 2; o > 0; o >>= 1) tf_add(x, tf_xor(x, o));
+        if (v != 0) return 0.0;
+        if (isfinite(x.a)) return x.value();
+        double s = 0.0;
+        for (int i = 0; i < nw; ++i) s += red[k][i].value();
+        return s;
+    }
+    double* red64 = reinterpret_cast<double*>(&red[0][0]);   // nobody reads red on this path
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        double v = acc[k].value();
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) red64[k * WARPS + w] = v;
+    }
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < N * WARPS && (threadIdx.x & (WARPS - 1)) == 0)
+        for (int i = 0; i < nw; ++i) s += red64[threadIdx.x + i];
+    return s;
 }
 
 // Dot-product accumulator of the vector precision: double-float for FP32

@@ -7,9 +7,11 @@
 //     x-hat, Eq. act_xhat, by Woodbury) and simple-kriging variances (the
 //     quantity the bootstrap of Sec. 3.5 estimates).
 //
-// Vectors are FP32 (or FP64 for FP64 embeddings); every dot product is
-// accumulated in FP64 per block and reduced in a fixed order by one small
-// kernel, so results do not depend on scheduling.
+// Vectors are FP32 (or FP64 for FP64 embeddings).  Dot products are summed in a
+// fixed order, so results do not depend on scheduling: a thread's in double-float
+// (FP64 for FP64 vectors), a block's to FP64's precision and range (block_sums),
+// the blocks' partials in FP64, by a small kernel or, in FP32 CG, by every block
+// of the kernel that needs the sum.
 #include <cuda_fp16.h>
 #include <math.h>
 #include <string.h>
@@ -230,30 +232,21 @@ __device__ __forceinline__ void store_vec(T* __restrict__ dst, const T (&in)[VW]
     }
 }
 
-// Block sum of a running dot product in a fixed order (valid in thread 0):
-// double-float through FP32 shuffles for FP32 vectors, FP64 for FP64 ones.  A
-// warp's FP64 instruction holds its scheduler's FP64 pipe for 64 cycles on
-// GB300, so an FP64 shuffle tree in every block of a streaming kernel costs
-// more than the streaming (k_lanczos_update, 32 vectors of 183,501 values: 31
-// us, now 17.5 us with the FP16 store that took another 11).
+// Block sum of a running dot product over THREADS threads in a fixed order, valid
+// in thread 0.
+template <int THREADS>
 __device__ __forceinline__ double block_total(const DotAcc<float>& acc) {
-    __shared__ float2 red[32];
-    float hi = acc.a.hi, lo = acc.a.lo;
-    df_warp_sum(hi, lo);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(hi, lo);
-    __syncthreads();
-    if (threadIdx.x != 0) return 0.0;
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) df_add(hi, lo, red[w].x, red[w].y);
-    return (double)hi + (double)lo;
+    return block_sums<1, THREADS / 32>({acc.a});
 }
+template <int THREADS>
 __device__ __forceinline__ double block_total(const DotAcc<double>& acc) {
-    __shared__ double red[32];
+    __shared__ double red[THREADS / 32];
     double v = acc.s;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x != 0) return 0.0;
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v += red[w];
+    for (int w = 1; w < THREADS / 32; ++w) v += red[w];
     return v;
 }
 
@@ -389,7 +382,7 @@ __global__ void k_lanczos_update(const T* __restrict__ U, const T* __restrict__ 
             }
         }
     }
-    const double s = block_total(nrm);
+    const double s = block_total<256>(nrm);
     if (threadIdx.x == 0) part[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
@@ -443,6 +436,13 @@ struct Pair {
 };
 __device__ __forceinline__ void pair_add(Pair<float>& a, Pair<float> b) { df_add(a.hi, a.lo, b.hi, b.lo); }
 __device__ __forceinline__ void pair_add(Pair<double>& a, Pair<double> b) { a.hi += b.hi; }
+// a += x y: the product rounded to T, FP32 sums kept exactly but for the last bits of lo.
+__device__ __forceinline__ void pair_add_prod(Pair<float>& a, float x, float y) {
+    float s, t;
+    two_sum(a.hi, __fmul_rn(x, y), s, t);
+    a = {s, __fadd_rn(a.lo, t)};
+}
+__device__ __forceinline__ void pair_add_prod(Pair<double>& a, double x, double y) { a.hi = fma(x, y, a.hi); }
 __device__ __forceinline__ double pair_value(Pair<float> a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ double pair_value(Pair<double> a) { return a.hi; }
 template <typename T>
@@ -453,14 +453,11 @@ __device__ __forceinline__ Pair<T> pair_xor(Pair<T> a, int o) {
     return b;
 }
 
-// Sums of eight values over a warp: lanes 4a .. 4a + 3 return the sum of v[a].
+// Sums of eight values over a warp: lanes 4a .. 4a + 3 return the sum of s[a].
 // Each of the first three exchanges hands half of the values over, so that it
 // takes 9 exchanges instead of 40.
 template <typename T>
-__device__ __forceinline__ Pair<T> warp_sum8(const T (&v)[8], int lane) {
-    Pair<T> s[8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) s[a] = {v[a], (T)0};
+__device__ __forceinline__ Pair<T> warp_sum8(Pair<T> (&s)[8], int lane) {
 #pragma unroll
     for (int h = 4; h >= 1; h >>= 1) {
         const bool up = lane & (4 * h);
@@ -567,12 +564,13 @@ __device__ __forceinline__ bool reorth_now(const LanczosState& S, int k, int pas
 }
 
 // Partial dot products W_i^T w (i = 0..j) of each flagged vector against the
-// basis store Q (T, or FP16 for FP32 vectors).  A block holds its 8192 values
-// of w in registers and sweeps the basis eight vectors at a time, so every
-// thread has 32 independent 16-byte loads in flight; products and the sums of
-// a thread's 32 terms are in the vector precision T (a coefficient only needs
-// a few correct digits: it removes a component of size <= sqrt(eps)), sums
-// across threads in double-float (FP64 for FP64 vectors).  dpart rows are
+// basis store Q (T, or FP16 for FP32 vectors).  A block holds its 8192 values of
+// w (FP64: 2048) in registers and sweeps the basis eight vectors at a time, so
+// every thread has 32 (FP64: 8 times four) independent 16-byte loads in flight.
+// Products are in the vector precision T (a coefficient only needs a few correct
+// digits: it removes a component of size <= sqrt(eps)), FP32 ones added in
+// double-float throughout, so that the coefficient is as exact as its products
+// are; FP64 ones in FP64.  dpart rows are
 // [nvec][nsteps + 8][gridDim.x] (hi, lo) pairs: a sweep's rows past j (zeros)
 // stay in the vector's padding.  What held the pass before: one FP64 shuffle
 // tree of eight values per block and sweep (64 cycles an instruction) for 2 to
@@ -605,17 +603,17 @@ __global__ void __launch_bounds__(256) k_reorth_dots(const Sq* __restrict__ Q, c
             for (int e = 0; e < 8; ++e) w[c][e] = in[c] ? w[c][e] : (T)0;
         }
         for (int i0 = 0, sweep = 0; i0 <= j; i0 += 8, ++sweep) {
-            T acc[8];
+            Pair<T> acc[8];
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
-                acc[a] = 0;
+                acc[a] = {(T)0, (T)0};
                 const Sq* q = Q + (int64_t)min(i0 + a, j) * vs;
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     T qv[8];
                     load8(q + x[c], qv);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[a] += qv[e] * w[c][e];
+                    for (int e = 0; e < 8; ++e) pair_add_prod(acc[a], qv[e], w[c][e]);
                 }
             }
             Pair<T> tot = warp_sum8<T>(acc, lane);   // of acc[lane >> 2] over the warp
@@ -688,7 +686,7 @@ __global__ void __launch_bounds__(256) k_reorth_apply(const Sq* __restrict__ Q, 
         }
         store8(w + x, r);
     }
-    const double s = block_total(nrm);
+    const double s = block_total<256>(nrm);
     if (threadIdx.x == 0) part[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 
@@ -1286,7 +1284,7 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_update(float* __restrict__ R
         for (int e = 0; e < 4; ++e) r[e] = rn[e], q[e] = qn[e];
         x += step;
     }
-    const double s = block_total(nrm);
+    const double s = block_total<CG_THREADS>(nrm);
     if (threadIdx.x == 0) part_rr[(int64_t)k * gridDim.x + blockIdx.x] = s;
 }
 

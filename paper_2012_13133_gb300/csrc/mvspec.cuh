@@ -84,28 +84,6 @@ __device__ __forceinline__ void cell_indices(const uint2* __restrict__ w, int wp
     }
 }
 
-// Pass C's v . K v partials of a block, in a fixed order and in double-float:
-// FP64 shuffle trees would hold the FP64 pipe (one warp instruction per 64
-// cycles) for longer than the pass's stores take.
-template <int TH>
-__device__ __forceinline__ void block_dots(kry::DFAcc& acc_a, kry::DFAcc& acc_b, float2 (&red)[2][TH / 32], bool has_b,
-                                           double* __restrict__ dots, int ndot_stride, int va, int vb) {
-    kry::df_warp_sum(acc_a.hi, acc_a.lo);
-    kry::df_warp_sum(acc_b.hi, acc_b.lo);
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-        red[0][w] = make_float2(acc_a.hi, acc_a.lo);
-        red[1][w] = make_float2(acc_b.hi, acc_b.lo);
-    }
-    __syncthreads();
-    if (threadIdx.x < 2 && (threadIdx.x == 0 || has_b)) {
-        float hi = 0.f, lo = 0.f;
-#pragma unroll
-        for (int k = 0; k < TH / 32; ++k) kry::df_add(hi, lo, red[threadIdx.x][k].x, red[threadIdx.x][k].y);
-        dots[(int64_t)(threadIdx.x ? vb : va) * ndot_stride + blockIdx.x] = (double)hi + (double)lo;
-    }
-}
-
 // Post factors of a thread's E outputs t + s LT.
 template <int E, int LT>
 __device__ __forceinline__ void load_post(float2 (&f)[E], const float2* __restrict__ pw) {
@@ -259,7 +237,6 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     using P = Plan<B>;
     constexpr int H = P::H, E = P::E, LT = P::LT, NT = nt_of(B, TH), PS = pad_shift(H);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float2 red[2][TH / 32];
     const int n = threadIdx.x & (NT - 1), t = threadIdx.x / NT;
     StageTw<16> tw1;   // constant tables: their latency lies behind the kernel before
     load_twiddles<E, P::R0, true>(tw1, twi, t);
@@ -304,7 +281,7 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     }
     later_stages<B, 1, true>(v, tw1, t, twi, lds, sts);
 
-    kry::DFAcc acc_a, acc_b;
+    kry::DFAcc acc[2];
     {
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
@@ -333,12 +310,16 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
 #pragma unroll
             for (int i = 0; i < E; ++i) {
                 const bool on = q[i] >= 0;   // what lies in unobserved cells stays out of the sums
-                acc_a.add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
-                acc_b.add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
+                acc[0].add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
+                acc[1].add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
             }
         }
     }
-    if (dots != nullptr) block_dots<TH>(acc_a, acc_b, red, has_b, dots, ndot_stride, va, vb);
+    if (dots != nullptr) {
+        const double s = kry::block_sums<2, TH / 32>(acc);
+        if (threadIdx.x == 0) dots[(int64_t)va * ndot_stride + blockIdx.x] = s;
+        if (threadIdx.x == TH / 32 && has_b) dots[(int64_t)vb * ndot_stride + blockIdx.x] = s;
+    }
 }
 
 // ---------------------------------------------------------------- dispatch

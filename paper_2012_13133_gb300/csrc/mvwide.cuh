@@ -346,7 +346,6 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
     using P = Wide<B>;
     constexpr int LT = P::LT, NT = wide_nt(B, TH);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float2 red[2][TH / 32];
     const int q = threadIdx.x & 1, n = (threadIdx.x >> 1) & (NT - 1), t = threadIdx.x / (2 * NT);
     pdl_wait();   // the slab comes from pass B
     pdl_launch_dependents();
@@ -371,7 +370,7 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
         wide_inverse<B>(w, v, reinterpret_cast<float2*>(smem_raw) + n * 2 + q, t, q, 2 * NT, tw);
         wide_post<B>(v, y, t, q, post);
     }
-    kry::DFAcc acc_a, acc_b;
+    kry::DFAcc acc[2];
     {
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
@@ -399,12 +398,16 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const bool on = c[i] >= 0;   // what lies in unobserved cells stays out of the sums
-                acc_a.add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
-                acc_b.add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
+                acc[0].add_prod(on ? x[i].x : 0.f, on ? y[i].x : 0.f);
+                acc[1].add_prod(on ? x[i].y : 0.f, on ? y[i].y : 0.f);
             }
         }
     }
-    if (dots != nullptr) block_dots<TH>(acc_a, acc_b, red, has_b, dots, ndot_stride, va, vb);
+    if (dots != nullptr) {
+        const double s = kry::block_sums<2, TH / 32>(acc);
+        if (threadIdx.x == 0) dots[(int64_t)va * ndot_stride + blockIdx.x] = s;
+        if (threadIdx.x == TH / 32 && has_b) dots[(int64_t)vb * ndot_stride + blockIdx.x] = s;
+    }
 }
 
 }  // namespace kspec
