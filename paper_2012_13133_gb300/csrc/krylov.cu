@@ -1359,43 +1359,74 @@ __global__ void k_df_to_f64(const float* __restrict__ Xh, const float* __restric
         X[(int64_t)k * ldx + i] = (double)Xh[(int64_t)k * ld + i] + (double)Xl[(int64_t)k * ld + i];
 }
 
+// The kept direction belongs to the recursive residual.  Where a block of
+// iterations gains more digits than FP32 holds (rr below 1e-12 rr_ref; condition
+// numbers below about 2), the recursion goes on below the true residual, of norm
+// rn, and the step along the then far shorter direction would overshoot by the
+// square of the ratio: the column starts again from its residual.  Slower systems,
+// whose recursion drifts by rounding, keep their direction.  S.rr and S.rr_ref are
+// the recursive r^T r and that of the last replacement until k_round_end.
+__device__ __forceinline__ bool rcg_restart(const RcgState& S, int k, double rn) {
+    return S.rr[k] < 1e-12 * S.rr_ref[k] && rn * rn > 16.0 * S.rr[k];
+}
+
 // Residual replacement of the running columns of the round: R = (float) R64,
-// rr = rr_ref = ||R64||^2 and, without a preconditioner, gamma = rr (P is
-// kept); done when ||R64|| <= rtol ||B|| or the iteration budget is spent (a
-// non-finite residual also ends the column; the caller reports it).
-__global__ void k_rcg_replace(const double* __restrict__ R64, float* __restrict__ R, int64_t p, int64_t ld,
-                              const double* __restrict__ norms, RcgState S, int maxit, int precond,
+// and without a preconditioner P = R where the column starts again.
+__global__ void k_rcg_replace(const double* __restrict__ R64, float* __restrict__ R, float* __restrict__ P, int64_t p,
+                              int64_t ld, const double* __restrict__ norms, RcgState S, int precond,
                               const int* __restrict__ sel) {
     const int k = blockIdx.y;
     if (S.done[k] || sel[k]) return;   // only the columns of the round (the others' norms are stale)
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x)
-        R[(int64_t)k * ld + i] = (float)R64[(int64_t)k * p + i];
-    if (blockIdx.x == 0 && threadIdx.x == 0) {   // (want is cleared by k_count_done, after every block)
-        const double rn = norms[2 * k];
-        if (!precond) S.gam[k] = rn * rn;
-        S.rr[k] = rn * rn;
-        S.rr_ref[k] = rn * rn;
-        if (rn * rn <= S.thr2[k] || S.iters[k] >= maxit || !(rn == rn)) S.done[k] = 1;
+    const bool again = !precond && rcg_restart(S, k, norms[2 * k]);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x) {
+        const float r = (float)R64[(int64_t)k * p + i];
+        R[(int64_t)k * ld + i] = r;
+        if (again) P[(int64_t)k * ld + i] = r;
     }
 }
 
-// gamma = r^T z after a replacement (preconditioned runs): the fixed-order sum
-// of the preconditioner matvec's partials.
-__global__ void k_rcg_regamma(RcgState S, const double* __restrict__ part_rz, int nrz, const int* __restrict__ sel) {
-    const int k = blockIdx.x;
+// Preconditioned runs after a replacement: gamma = r^T z, the fixed-order sum of
+// the preconditioner matvec's partials (block 0 of a column), and P = Z where the
+// column starts again.
+__global__ void k_rcg_regamma(RcgState S, const float* __restrict__ Z, float* __restrict__ P, int64_t ld,
+                              const double* __restrict__ norms, const double* __restrict__ part_rz, int nrz,
+                              const int* __restrict__ sel) {
+    const int k = blockIdx.y;
     if (S.done[k] || sel[k]) return;
-    const double g = block_sum(part_rz + (int64_t)k * nrz, nrz);
-    if (threadIdx.x == 0) S.gam[k] = g;
+    if (blockIdx.x == 0) {
+        const double g = block_sum(part_rz + (int64_t)k * nrz, nrz);
+        if (threadIdx.x == 0) S.gam[k] = g;
+    }
+    if (!rcg_restart(S, k, norms[2 * k])) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ld; i += (int64_t)gridDim.x * blockDim.x)
+        P[(int64_t)k * ld + i] = Z[(int64_t)k * ld + i];
 }
 
-// Ends a replacement round: counts the finished columns and clears the requests.
-__global__ void k_count_done(RcgState S, int nrhs) {
+// Ends a replacement round (one block).  Its running columns: rr = rr_ref =
+// ||R64||^2 and, without a preconditioner, gamma = rr; done when ||R64|| <= rtol
+// ||B|| or the iteration budget is spent (a non-finite residual also ends the
+// column; the caller reports it).  Counts the finished columns and clears the
+// requests.
+__global__ void k_round_end(RcgState S, int nrhs, const double* __restrict__ norms, int maxit, int precond,
+                            const int* __restrict__ sel) {
+    __shared__ int finished;
+    if (threadIdx.x == 0) finished = 0;
+    __syncthreads();
     int d = 0;
-    for (int k = 0; k < nrhs; ++k) {
+    for (int k = threadIdx.x; k < nrhs; k += blockDim.x) {
+        if (!S.done[k] && !sel[k]) {
+            const double rn = norms[2 * k], rr = rn * rn;
+            if (!precond) S.gam[k] = rr;
+            S.rr[k] = rr;
+            S.rr_ref[k] = rr;
+            if (rr <= S.thr2[k] || S.iters[k] >= maxit || !(rn == rn)) S.done[k] = 1;
+        }
         d += S.done[k];
         S.want[k] = 0;
     }
-    *S.ndone = d;
+    atomicAdd(&finished, d);
+    __syncthreads();
+    if (threadIdx.x == 0) *S.ndone = finished;
 }
 
 static void true_residual(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t ldb, const double* X,
@@ -1519,14 +1550,14 @@ static int cg_reliable(kry_ctx* ctx, const kry_embed* e, const double* B, int64_
             to_f64(sel);
             true_residual(ctx, e, B, ldb, X, ldx, nrhs, R64, ctx->kxbuf.as<double>(), vpt, sel);
             double* dn = ctx->red.as<double>() + (size_t)nrhs * RED_BLOCKS * 2;   // device norms
-            k_rcg_replace<<<gc, 256, 0, st>>>(R64, R, p, ld, dn, S, maxit, pre ? 1 : 0, sel);
+            k_rcg_replace<<<gc, 256, 0, st>>>(R64, R, P, p, ld, dn, S, pre ? 1 : 0, sel);
             KRY_CHECK_LAUNCH();
             if (pre) {   // z = M^-1 r and gamma = r^T z for the replaced r
                 matvec_ex<float>(ctx, pre, R, ld, nullptr, Z, ld, nrhs, part_rz, nblkC, vpt, sel);
-                k_rcg_regamma<<<nrhs, FIN_THREADS, 0, st>>>(S, part_rz, nblkC, sel);
+                k_rcg_regamma<<<gc, FIN_THREADS, 0, st>>>(S, Z, P, ld, dn, part_rz, nblkC, sel);
                 KRY_CHECK_LAUNCH();
             }
-            k_count_done<<<1, 1, 0, st>>>(S, nrhs);
+            k_round_end<<<1, 256, 0, st>>>(S, nrhs, dn, maxit, pre ? 1 : 0, sel);
             KRY_CHECK_LAUNCH();
             KRY_CUDA(cudaMemcpyAsync(hflag, S.ndone, sizeof(int), cudaMemcpyDeviceToHost, st));
             KRY_CUDA(cudaStreamSynchronize(st));

@@ -93,3 +93,27 @@ def test_search_of_many_columns(ncov, settings):
         assert abs(r["loglik"][k] - one["loglik"][0]) <= 1e-5 * abs(one["loglik"][0]) + 1e-5
         assert abs(r["logdet"][k] - one["logdet"][0]) <= 1e-5 * p
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n1,n2,nrhs", [(600, 90, 3), (40, 520, 2), (300, 300, 1), (64, 64, 12), (20, 20, 2)])
+@pytest.mark.parametrize("cells", [0.05, 0.3, 0.7])
+@pytest.mark.parametrize("precond", [False, True])
+def test_systems_that_converge_within_a_block_of_iterations(n1, n2, nrhs, cells, precond):
+    """Ranges below a cell: the recursive residual passes FP32's resolution before the first replacement."""
+    import torch
+
+    from paper_2012_13133_gb300 import inputs as I
+    from paper_2012_13133_gb300 import kry
+    cov = I.Cov(1.0, cells / max(n1, n2), 0.5, 0.5)
+    mask = np.random.default_rng(n1).random((n1, n2)) >= 0.2
+    ctx = kry.Context(0)
+    p = ctx.set_mask(torch.from_numpy(mask.astype(np.uint8)).cuda())
+    B = torch.randn((nrhs, p), generator=torch.Generator().manual_seed(n2), dtype=torch.float64).cuda()
+    X, iters, _, st = ctx.solve(ctx.embed(cov, kry.KRY_F32), B, rtol=RTOL, maxit=500, precond=precond)
+    assert st == kry.KRY_OK
+    rn, kappa = residual_norms(ctx, kry, cov, B, X)   # the largest row sum over tau2 bounds the condition number
+    assert bool(torch.all(rn <= RTOL * 1.001 * B.norm(dim=1)))
+    # CG's bound, with a block of 8 more after each of the (at most 9) replacements
+    assert iters <= 0.5 * math.sqrt(kappa / 0.5) * math.log(2.0 * kappa / 0.5 / RTOL) + 8 * 9
+    ctx.close()
