@@ -503,7 +503,7 @@ void bccb_logdet(kry_ctx* ctx, const kry_cov& cov, bool deriv, double* logdet, d
 }
 
 // lamT[j][k] = lam[k][j] * scale (FP64 and optionally FP32), 32 x 32 tiles.
-// With t32p != NULL also the column-permuted FP32 copy (kspec::lam_slot).
+// With t32p != NULL also the column-permuted FP32 copy (kspec::lam_slot), scaled by 1 / FWD_SCALE more.
 __global__ void k_transpose_scale(const double* __restrict__ lam, int M1, int M2, double scale,
                                   double* __restrict__ t64, float* __restrict__ t32, float* __restrict__ t32p,
                                   int lt) {
@@ -520,7 +520,7 @@ __global__ void k_transpose_scale(const double* __restrict__ lam, int M1, int M2
             const double v = tile[threadIdx.x][r] * scale;
             t64[(int64_t)j * M1 + k] = v;
             if (t32) t32[(int64_t)j * M1 + k] = (float)v;
-            if (t32p) t32p[(int64_t)j * M1 + kspec::lam_slot(k, M1, lt)] = (float)v;
+            if (t32p) t32p[(int64_t)j * M1 + kspec::lam_slot(k, M1, lt)] = (float)(v * (1.0 / kspec::FWD_SCALE));
         }
     }
 }

@@ -14,7 +14,8 @@
 //  * E = 16 for long transforms, E = 4 up to 512 points: a thread's serial chain is
 //    a quarter as long, and small grids have too few warps for the chip's 608
 //    schedulers otherwise.
-// Where cos = 0 the table holds +-2^-55 for it (see fftspec.cuh).
+// Where cos = 0 the table holds +-2^-55 for it (what this adds is an eighth of a unit
+// roundoff), so intermediate values are to stay below 2^969.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -33,9 +33,16 @@
 // whole radix-16 stage are then 8 pairs (c, T) (the other seven are these
 // times -i), all from a table; the products that formed 12 of 15 twiddles
 // before are gone.  Rounding: u carries a relative error of |T| eps |b|, which
-// the factor c scales back to eps |sin| |b|, so a large T costs no accuracy;
-// where cos = 0 the table holds +-2^-27 for it (the part of b that this adds
-// is an eighth of a unit roundoff).
+// the factor c scales back to eps |sin| |b|, so a large T costs no accuracy.  Level
+// 1, whose angles reach half a turn, takes p = a + w b with (cos, sin) in its table
+// entry and 2 a - p (8 operations); from level 2 on they stay below a quarter turn.
+//
+// Range: T reaches R NS / 2 pi at the last level of a stage of radix R and stride NS, 652
+// at side 8192, so intermediate values are to stay below 2^118.  Forward they can be
+// as large as the sum over the grid; pass A therefore scales its input by FWD_SCALE
+// and the eigenvalues of pass B take it back, both exactly.  What is left of it: a
+// result K v beyond 2^118 overflows.  ((cos, sin), or tangents of at most one, at
+// every level: no limit, but 25% more error on ordinary values.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -127,6 +134,16 @@ __device__ __forceinline__ constexpr float tan32(int m) {
     return t[m];
 }
 
+// One radix-2 butterfly (a, b) -> (a + w b, a - w b) in both lanes, w = c -+ i s
+// (forward / inverse).
+template <bool INV>
+__device__ __forceinline__ void bfly_cs(c2& a, c2& b, u64 c, u64 s) {
+    const u64 ns = neg2(s);
+    const u64 pr = fma2(INV ? ns : s, b.i, fma2(c, b.r, a.r)), pi = fma2(INV ? s : ns, b.r, fma2(c, b.i, a.i));
+    b = {sub2(add2(a.r, a.r), pr), sub2(add2(a.i, a.i), pi)};   // a - w b = 2 a - (a + w b)
+    a = {pr, pi};
+}
+
 // One radix-2 butterfly (a, b) -> (a + w b, a - w b) in both lanes, w = c (1 -+ i T)
 // (forward / inverse), times -+i with ROT.
 template <bool INV, bool ROT>
@@ -168,7 +185,7 @@ __device__ __forceinline__ void bfly1(c2& a, c2& b) {
 // 2^{l-2} times -+i).  Output s of the tree ends in slot bitrev(s).
 __host__ __device__ constexpr int tw_base(int l) { return l == 1 ? 0 : 1 << (l - 2); }
 
-// Twiddles of one level: MODE 0 from the registers (c, T); MODE 1 the first
+// Twiddles of one level: MODE 0 from the registers (c, T) (level 1: (c, s)); MODE 1 the first
 // forward stage's (lane 0: W_{2^l}^s, lane 1: that times omega^D, omega =
 // W_{2R}); MODE 2 the first inverse stage's (both lanes W_{2^l}^s).
 template <int R, int LEV, bool INV, int MODE>
@@ -184,6 +201,10 @@ __device__ __forceinline__ void level(c2* v, const u64* c, const u64* T) {
         if constexpr (MODE == 0) {
             cc = c[tw_base(LEV) + e];
             tt = T[tw_base(LEV) + e];
+            if constexpr (LEV == 1) {
+                bfly_cs<INV>(v[p], v[p + D], cc, tt);
+                continue;
+            }
         } else {
             const int m0 = e * (32 >> LEV), m1 = MODE == 1 ? m0 + (16 >> LEV) : m0;
             if (MODE == 2 && e == 0) {
@@ -220,10 +241,14 @@ __device__ __forceinline__ void first_pair(float2 a, float2 b, c2& p, c2& m) {
 // with consecutive k = t mod NS read consecutive 16-byte words:
 //   forward  word 8 (NS - 2) + e NS + k      = (c, c', T, T')  lanes k, k + 1/2
 //   inverse  word 4 (NS - 2) + (e/2) NS + k  = (c_e, T_e, c_{e+1}, T_{e+1})
+// with sin instead of tan for entry 0 (level 1).
 constexpr int TWF_WORDS = 8 * 510, TWI_WORDS = 4 * 510;
 // Post factors exp(+2 pi i j / L) of the inverse: word L/2 - 32 + j, j < L/2
 // (64 <= L <= 8192).
 constexpr int POST_WORDS = 8160;
+
+// What pass A scales its input by, and the eigenvalues of pass B (lam32P) by its inverse.
+constexpr float FWD_SCALE = 0x1p-10f;
 
 // Twiddles of one radix-E stage.
 template <int E>

@@ -9,7 +9,7 @@
 //    tiles slab[pair][tile][i][c], c < Cs, tile = column / Cs (Cs even, so the
 //    two columns 2k, 2k + 1 that a row transform produces in its two lanes
 //    are one 16-byte word);
-//  * lamP: eigenvalues per column j at j M1, scaled by 1 / (M1 M2), permuted
+//  * lamP: eigenvalues per column j at j M1, scaled by 1 / (M1 M2 FWD_SCALE), permuted
 //    so that the values a column-pass thread multiplies are 16-byte words
 //    consecutive over threads (lam_slot);
 //  * bits: per 32 cells of a grid row, the observation bits and the index of
@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
 
     float2 x[E];
     {
-        const float sa = scale ? (float)scale[va] : 1.f;
-        const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
+        const float sa = FWD_SCALE * (scale ? (float)scale[va] : 1.f);
+        const float sbv = FWD_SCALE * ((scale && has_b) ? (float)scale[vb] : 1.f);
         const float* pa = vin + (int64_t)va * ld;
         const float* pb = has_b ? vin + (int64_t)vb * ld : pa;
         int q[E];

@@ -16,19 +16,14 @@ int block_threads(int M, int nt, int most) {
     return th;
 }
 
-// cos of the twiddle angle with its zero replaced by +-2^-27 (fftspec.cuh) and the tangent that goes with it.
-__device__ __forceinline__ float2 cos_tan(double turns) {
-    double s, c;
-    sincospi(2.0 * turns, &s, &c);
-    float cf = (float)c;
-    if (fabsf(cf) < 7.450580596923828e-9f) cf = c < 0.0 ? -7.450580596923828e-9f : 7.450580596923828e-9f;
-    return make_float2(cf, (float)(s / (double)cf));
-}
-
-// Angle (in turns) of entry e = s + 2^{l-2} of level l at stride ns, frequency k.
-__device__ __forceinline__ double entry_turns(int e, int ns, double k) {
+// Entry e = s + 2^{l-2} of level l at stride ns, frequency k: (cos, tan) of its angle,
+// (k / ns + s) / 2^l of a turn, the tangent that goes with the rounded cosine; entry
+// 0 (level 1): (cos, sin).
+__device__ __forceinline__ float2 entry(int e, int ns, double k) {
     const int l = e == 0 ? 1 : 2 + (31 - __clz(e));
-    return (k / ns + (e - tw_base(l))) / (double)(1 << l);
+    double s, c;
+    sincospi(2.0 * (k / ns + (e - tw_base(l))) / (double)(1 << l), &s, &c);
+    return make_float2((float)c, (float)(e == 0 ? s : s / (double)(float)c));
 }
 
 __global__ void k_tables(float4* __restrict__ tab) {
@@ -36,13 +31,13 @@ __global__ void k_tables(float4* __restrict__ tab) {
     if (i < TWF_WORDS) {
         const int ns = 1 << (31 - __clz(i / 8 + 2));   // sections of 8 ns words from 8 (ns - 2)
         const int r = i - 8 * (ns - 2), e = r / ns, k = r - e * ns;
-        const float2 a = cos_tan(entry_turns(e, ns, k)), b = cos_tan(entry_turns(e, ns, k + 0.5));
+        const float2 a = entry(e, ns, k), b = entry(e, ns, k + 0.5);
         tab[i] = make_float4(a.x, b.x, a.y, b.y);
     } else if (i < TWF_WORDS + TWI_WORDS) {
         const int w = i - TWF_WORDS;
         const int ns = 1 << (31 - __clz(w / 4 + 2));
         const int r = w - 4 * (ns - 2), e = r / ns, k = r - e * ns;
-        const float2 a = cos_tan(entry_turns(2 * e, ns, k)), b = cos_tan(entry_turns(2 * e + 1, ns, k));
+        const float2 a = entry(2 * e, ns, k), b = entry(2 * e + 1, ns, k);
         tab[i] = make_float4(a.x, a.y, b.x, b.y);
     } else if (i < TWF_WORDS + TWI_WORDS + POST_WORDS / 2) {
         float2 f[2];
@@ -58,7 +53,7 @@ __global__ void k_tables(float4* __restrict__ tab) {
         const int w = 2 * (i - TWF_WORDS - TWI_WORDS - POST_WORDS / 2);
         const int ns = w < wide_section(16) ? 1 : w < wide_section(32) ? 16 : 32;
         const int r = w - wide_section(ns), e = r / (2 * ns), k = (r - e * 2 * ns) >> 1;
-        const float2 a = cos_tan(entry_turns(e, ns, k)), b = cos_tan(entry_turns(e, ns, k + 0.5));
+        const float2 a = entry(e, ns, k), b = entry(e, ns, k + 0.5);
         tab[i] = make_float4(a.x, a.y, b.x, b.y);
     }
 }

@@ -79,6 +79,17 @@ __device__ __forceinline__ void wbfly1(cx& a, cx& b) {
     }
 }
 
+// Level 1 on two packed partners: bfly_cs of fftspec.cuh by way of u = w b, which is
+// the faster form here (64 vectors on 1024^2 799 us against 810; both forms' error is
+// 1.7e-7).
+template <bool INV>
+__device__ __forceinline__ void wbfly_cs(c2& a, c2& b, u64 c, u64 s) {
+    const u64 ns = neg2(s);
+    const u64 ur = fma2(INV ? ns : s, b.i, mul2(c, b.r)), ui = fma2(INV ? s : ns, b.r, mul2(c, b.i));
+    b = {sub2(a.r, ur), sub2(a.i, ui)};
+    a = {add2(a.r, ur), add2(a.i, ui)};
+}
+
 // Levels LEV .. log2 R of a radix-R tree (level of fftspec.cuh): twiddle entry
 // e at tw[e stride], or (CONST) the constants of a first inverse stage. sign =
 // -1 swaps outputs s and s + R/2.
@@ -109,7 +120,8 @@ __device__ __forceinline__ void wlevels(cx* v, const float2* __restrict__ tw, in
                     else bfly1<INV, false>(a, b);
                 } else {
                     const float c = CONST ? cos32(e * (32 >> LEV)) : w[e].x, T = CONST ? tan32(e * (32 >> LEV)) : w[e].y;
-                    if (rot) bfly<INV, true>(a, b, pk(c, c), pk(T, T));
+                    if (LEV == 1) wbfly_cs<INV>(a, b, pk(c, c), pk(T, T));
+                    else if (rot) bfly<INV, true>(a, b, pk(c, c), pk(T, T));
                     else bfly<INV, false>(a, b, pk(c, c), pk(T, T));
                 }
                 const float2 ar = upk(a.r), ai = upk(a.i), br = upk(b.r), bi = upk(b.i);
@@ -133,7 +145,7 @@ __device__ __forceinline__ void wlevels(cx* v, const float2* __restrict__ tw, in
 }
 
 // Twiddle table: for stride NS = 1, 16 and 32, entry e of thread (k, q) at
-// section + e 2 NS + 2 k + q: (cos, tan) of (k + q / 2) / NS + s over 2^l turns.
+// section + e 2 NS + 2 k + q: (cos, tan) of (k + q / 2) / NS + s over 2^l turns (entry 0: (cos, sin)).
 // Inverse stages take q = 0.
 constexpr int wide_section(int NS) { return NS == 1 ? 0 : NS == 16 ? 32 : 32 + 16 * 32; }
 
@@ -242,8 +254,8 @@ __global__ void __launch_bounds__(TH, minb(B, TH))
 
     float2 own[16];   // cells t + (i + 16 q) LT; the other half comes from the neighbouring thread
     {
-        const float sa = scale ? (float)scale[va] : 1.f;
-        const float sbv = (scale && has_b) ? (float)scale[vb] : 1.f;
+        const float sa = FWD_SCALE * (scale ? (float)scale[va] : 1.f);
+        const float sbv = FWD_SCALE * ((scale && has_b) ? (float)scale[vb] : 1.f);
         const float* pa = vin + (int64_t)va * ld;
         const float* pb = has_b ? vin + (int64_t)vb * ld : pa;
         int c[16];
