@@ -10,7 +10,6 @@
 // are averaged, which keeps c symmetric under j -> -j (and Lambda real) for
 // anisotropic covariances too.  Lambda = FFT2(c) in FP64.
 #include <algorithm>
-#include <cfloat>
 
 #include "fft64.cuh"
 #include "kry_internal.cuh"

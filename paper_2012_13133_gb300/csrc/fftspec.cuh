@@ -94,7 +94,7 @@ __device__ __forceinline__ u64 neg2(u64 a) { return a ^ 0x8000000080000000ull; }
 // 16-byte wavefront).  For every stage pad(x + c) = pad(x) + pad(c), so an
 // access is one per-thread base plus an immediate.
 __host__ __device__ constexpr int pad_shift(int H) {
-    return H == 1024 ? 2 : H == 128 || H == 512 || H == 2048 ? 3 : 4;
+    return H == 128 || H == 2048 ? 3 : 4;
 }
 
 __host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x >> 1); }

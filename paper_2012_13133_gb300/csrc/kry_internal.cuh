@@ -100,18 +100,13 @@ struct DevBuf {
     T* as() const { return static_cast<T*>(p); }
 };
 
-// Matvec launch schedule: elements per thread in the row passes and the
-// column pass, rows per CTA in the row passes, columns per CTA in the column
-// pass (= the column-tile width of the intermediate slab), and the number of
-// complex vector pairs per batch.
+// Matvec launch schedule: rows per block in the row passes, columns per block in
+// the column pass, and the number of complex vector pairs per batch (0: the
+// default, all pairs).
 struct MvSched {
-    int ept_row = 8;
-    int rows_per_cta = 1;
-    int ept_col = 8;
-    int cols_per_cta = 4;
-    int pairs_per_batch = 0;   // 0 = all pairs at once
-    int g16 = 0;               // radix-16 path: rows per block (0 = default)
-    int c16 = 0;               // radix-16 path: columns per block / slab tile width (0 = default)
+    int pairs_per_batch = 0;
+    int rows = 0;
+    int cols = 0;
 };
 
 struct kry_ctx {
@@ -173,7 +168,7 @@ struct kry_ctx {
     int num_sms = 0;
     int max_smem_optin = 0;
 
-    MvSched sched32, sched64;
+    MvSched sched;   // the default
     // autotuned / user-set schedules keyed by (M1, M2, precision, batch bucket)
     std::map<uint64_t, MvSched> tuned;
 
@@ -288,7 +283,6 @@ void genhybr(kry_ctx* ctx, const kry_cov& cov, kry_prec prec, const double* b, i
 // deriv, of its range derivative (Sec. 3.3, Appendix A).
 void bccb_logdet(kry_ctx* ctx, const kry_cov& cov, bool deriv, double* logdet, double* dlogdet);
 
-int smem_limit(kry_ctx* ctx);
 
 // Record a profiling event on the context stream; inside a stream capture it
 // becomes an external event-record node, so it still times the graph replay.

@@ -20,7 +20,6 @@
 #include <vector>
 
 #include "dfloat.cuh"
-#include "fft.cuh"
 #include "kry_internal.cuh"
 #include "matern.cuh"
 #include "quadrature.cuh"
@@ -207,29 +206,14 @@ __device__ __forceinline__ double block_sum(const double* __restrict__ part, int
 
 static const int FIN_THREADS = 256;   // block size of the per-vector finalisers
 
-// VW consecutive elements of type T through one 16-byte access (VW = 16 /
-// sizeof(T)), or one element (VW = 1).  The caller guarantees alignment.
-template <typename T, int VW>
-__device__ __forceinline__ void load_vec(const T* __restrict__ src, T (&out)[VW]) {
-    if constexpr (VW * sizeof(T) == 16) {
-        const int4 q = *reinterpret_cast<const int4*>(src);
-        memcpy(out, &q, 16);
-    } else {
-#pragma unroll
-        for (int e = 0; e < VW; ++e) out[e] = src[e];
-    }
+// Four consecutive FP32 values through one 16-byte access (the caller guarantees
+// the alignment).
+__device__ __forceinline__ void load4(const float* __restrict__ src, float (&out)[4]) {
+    const float4 a = *reinterpret_cast<const float4*>(src);
+    out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
 }
-
-template <typename T, int VW>
-__device__ __forceinline__ void store_vec(T* __restrict__ dst, const T (&in)[VW]) {
-    if constexpr (VW * sizeof(T) == 16) {
-        int4 q;
-        memcpy(&q, in, 16);
-        *reinterpret_cast<int4*>(dst) = q;
-    } else {
-#pragma unroll
-        for (int e = 0; e < VW; ++e) dst[e] = in[e];
-    }
+__device__ __forceinline__ void store4(float* __restrict__ dst, const float (&v)[4]) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
 // Block sum of a running dot product over THREADS threads in a fixed order, valid
@@ -304,7 +288,6 @@ struct LanczosState {
     // partial reorthogonalisation only (all NULL without it)
     double* s_hist;   // [nprobe][nsteps] scale of every stored basis vector: q_i = s_hist[i] * W_i
     double* omega;    // [3][nprobe][nsteps + 1] estimates of q_j^T q_k for j-1, j, j+1 (buffer j mod 3)
-    double* coef;     // [nprobe][nsteps] s_i * q_i^T w of the vector being reorthogonalised
     int* flag;        // [nprobe] 1: reorthogonalise the new vector of this step
     int* force;       // [nprobe] 1: the next new vector is reorthogonalised too
     int* again;       // [nprobe] 1: a flagged vector takes a second Gram-Schmidt pass
@@ -736,7 +719,7 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
     ctx->work[4].ensure((size_t)nvec * nred * sizeof(double));
     double* part = ctx->work[4].as<double>();
     const size_t nsc = (size_t)nvec * (2 * nsteps + 4) + nvec;
-    const size_t npro = reorth ? (size_t)nvec * (2 * nsteps + 3 * (nsteps + 1) + 1) : 0;
+    const size_t npro = reorth ? (size_t)nvec * (nsteps + 3 * (nsteps + 1) + 1) : 0;
     ctx->scal.ensure((nsc + npro) * sizeof(double));
     double* sc = ctx->scal.as<double>();
     LanczosState S;
@@ -747,13 +730,12 @@ static void lanczos_logdet(kry_ctx* ctx, const kry_embed* e, int nvec, int nprob
     double* res = S.beta + (size_t)nvec * nsteps;
     ctx->work[5].ensure((size_t)nvec * 4 * sizeof(int));
     S.m_eff = ctx->work[5].as<int>();
-    S.s_hist = S.omega = S.coef = S.pre2 = nullptr;
+    S.s_hist = S.omega = S.pre2 = nullptr;
     S.flag = S.force = S.again = nullptr;
     Pair<T>* dpart = nullptr;
     if (reorth) {
         S.s_hist = sc + nsc;
-        S.coef = S.s_hist + (size_t)nvec * nsteps;
-        S.omega = S.coef + (size_t)nvec * nsteps;
+        S.omega = S.s_hist + (size_t)nvec * nsteps;
         S.pre2 = S.omega + (size_t)3 * nvec * (nsteps + 1);
         S.flag = S.m_eff + nvec;
         S.force = S.flag + nvec;
@@ -1016,7 +998,6 @@ static int cg_inner(kry_ctx* ctx, const kry_embed* e, const double* B, int64_t l
             }
         }
     }
-    std::vector<int> its(nrhs);
     KRY_CUDA(cudaMemcpyAsync(hdone, S.iters, nrhs * sizeof(int), cudaMemcpyDeviceToHost, st));
     KRY_CUDA(cudaStreamSynchronize(st));
     int mx = 0;
@@ -1213,8 +1194,8 @@ __global__ void k_rcg_init_scalars(RcgState S, const double* __restrict__ part_r
     }
 }
 
-// Threads and blocks per column of the two streaming kernels: two blocks per SM
-// over all columns (every block repeats its column's sum, 0.4 us of FP64 pipe,
+// Threads and blocks per column of the two streaming kernels: two blocks per SM of
+// GB300 over all columns (every block repeats its column's sum, 0.4 us of FP64 pipe,
 // so four times as many blocks took 15 + 17 us instead of 8 + 10 for 4 columns
 // of 524,288 values).
 static const int CG_THREADS = 512;
@@ -1252,8 +1233,8 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_update(float* __restrict__ R
     int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     float r[4], q[4];
     if (x < ld) {   // in flight during the sum
-        load_vec<float, 4>(R + off + x, r);
-        load_vec<float, 4>(Q + off + x, q);
+        load4(R + off + x, r);
+        load4(Q + off + x, q);
     }
     const double g = threadIdx.x == 0 ? S.gam[k] : 0.0;
     const double d = total128(part_pq + (int64_t)k * npq, npq, red);
@@ -1271,15 +1252,15 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_update(float* __restrict__ R
     while (x < ld) {
         float rn[4], qn[4];
         if (x + step < ld) {
-            load_vec<float, 4>(R + off + x + step, rn);
-            load_vec<float, 4>(Q + off + x + step, qn);
+            load4(R + off + x + step, rn);
+            load4(Q + off + x + step, qn);
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             r[e] -= af * q[e];
             nrm.add_prod(r[e], r[e]);
         }
-        store_vec<float, 4>(R + off + x, r);
+        store4(R + off + x, r);
 #pragma unroll
         for (int e = 0; e < 4; ++e) r[e] = rn[e], q[e] = qn[e];
         x += step;
@@ -1309,10 +1290,10 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_pupdate(float* __restrict__ 
     int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     float z[4], pv[4], xh[4], xl[4];
     auto load = [&](int64_t o) {
-        load_vec<float, 4>(Z + o, z);
-        load_vec<float, 4>(P + o, pv);
-        load_vec<float, 4>(Xh + o, xh);
-        load_vec<float, 4>(Xl + o, xl);
+        load4(Z + o, z);
+        load4(P + o, pv);
+        load4(Xh + o, xh);
+        load4(Xl + o, xl);
     };
     if (x < ld) load(off + x);   // in flight during the sums
     double g0 = 0.0;
@@ -1341,9 +1322,9 @@ __global__ void __launch_bounds__(CG_THREADS) k_rcg_pupdate(float* __restrict__ 
             df_axpy(xh[e], xl[e], ahi, alo, pv[e]);
             pv[e] = z[e] + b * pv[e];
         }
-        store_vec<float, 4>(Xh + off + x, xh);
-        store_vec<float, 4>(Xl + off + x, xl);
-        store_vec<float, 4>(P + off + x, pv);
+        store4(Xh + off + x, xh);
+        store4(Xl + off + x, xl);
+        store4(P + off + x, pv);
         x += step;
         if (x < ld) load(off + x);
     }

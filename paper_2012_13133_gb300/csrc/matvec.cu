@@ -8,19 +8,18 @@
 // the real and imaginary parts of one complex field; that is exact because
 // Lambda is real and even.  The 2-D transform is split into three kernels:
 //
-//   pass A  per grid row i < n1: scatter the observed values of the row into
-//           a zero row of length M2 in shared memory, forward FFT, store the
-//           row into the intermediate slab (n1 x M2 complex per pair);
-//   pass B  per tile of C columns: load the n1 nonzero rows of each column,
-//           forward FFT of length M1, multiply by Lambda (scaled by
-//           1/(M1 M2)), inverse FFT, store the first n1 rows back;
-//   pass C  per grid row: inverse FFT of length M2, gather the observed
-//           columns, add the nugget term, and (optionally) accumulate the
-//           FP64 dot product of input and output for the Krylov loops.
+//   pass A  grid rows i < n1: the observed values of a row, zeros elsewhere,
+//           forward FFT of length M2 into the intermediate slab (n1 x M2
+//           complex per pair);
+//   pass B  columns: the n1 nonzero rows of a column, forward FFT of length
+//           M1, times Lambda (scaled by 1/(M1 M2)), inverse FFT, the first n1
+//           rows back in place;
+//   pass C  grid rows: inverse FFT of length M2, the observed columns, plus
+//           the nugget term, and (optionally) the partials of the dot product
+//           of input and output for the Krylov loops.
 //
-// The slab is laid out in column tiles, slab[pair][tile][i][c] with
-// c < C, so that pass B reads and writes one contiguous block per CTA and
-// passes A and C touch G*C contiguous elements per tile for G rows per CTA.
+// The slab is laid out in column tiles, slab[pair][tile][i][c], whose width each
+// kind of pass chooses so that the column pass reads and writes whole sectors.
 #include <algorithm>
 #include <mutex>
 #include <string>
@@ -34,72 +33,54 @@
 namespace kry {
 
 // The specialised FP32 passes (mvspec.cuh) cover torus sides from 64, the FP64
-// ones (mv64.cu) every side; the three kernels below run FP32 on the shorter
-// tori, radix 8 in shared memory (fft.cuh).
+// ones (mv64.cu) every side; the three kernels below run FP32 on tori with a
+// shorter side, radix 8 in shared memory (fft.cuh), 8 values per thread.
 
 // ------------------------------------------------------------------ pass A
 
-template <int EPT, int G>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_a(const float* __restrict__ vin, int64_t ld, const double* __restrict__ scale,
-                                                 int nvec, int pair0, const int* __restrict__ rowptr,
-                                                 const int* __restrict__ colidx, int n1, int M2, int C,
-                                                 float2* __restrict__ slab, const float2* __restrict__ tw) {
+// One row: the observed values into a zero row in shared memory, forward FFT.
+__global__ void __launch_bounds__(1024) k_pass_a(const float* __restrict__ vin, int64_t ld,
+                                                 const double* __restrict__ scale, int nvec, int pair0,
+                                                 const int* __restrict__ rowptr, const int* __restrict__ colidx,
+                                                 int n1, int M2, int C, float2* __restrict__ slab,
+                                                 const float2* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
-    const int L = M2;
-    const int stride = L + 1;
-    const int LT = L / EPT;
-    const int g = threadIdx.x / LT;
-    const int tl = threadIdx.x - g * LT;
-    const int row0 = blockIdx.x * G;
-    const int row = row0 + g;
-    const int pair = pair0 + blockIdx.y;
-    const int va = 2 * pair, vb = 2 * pair + 1;
+    const int L = M2, LT = L / 8, tl = threadIdx.x, row = blockIdx.x;
+    const int va = 2 * (pair0 + (int)blockIdx.y), vb = va + 1;
     const bool has_b = vb < nvec;
-    float2* rb = buf + g * stride;
 
-    for (int k = tl; k < L; k += LT) rb[k] = make_float2(0.f, 0.f);
+    for (int k = tl; k < L; k += LT) buf[k] = make_float2(0.f, 0.f);
     __syncthreads();
-    if (row < n1) {
-        const float sa = scale ? (float)scale[va] : 1.f;
-        const float sb = (scale && has_b) ? (float)scale[vb] : 1.f;
-        const float* pa = vin + (int64_t)va * ld;
-        const float* pb = vin + (int64_t)vb * ld;
-        const int q1 = rowptr[row + 1];
-        for (int q = rowptr[row] + tl; q < q1; q += LT) {
-            const int c = colidx[q];
-            const float a = pa[q] * sa;
-            const float b = has_b ? pb[q] * sb : 0.f;
-            rb[c] = make_float2(a, b);
-        }
-    }
+    const float sa = scale ? (float)scale[va] : 1.f;
+    const float sb = (scale && has_b) ? (float)scale[vb] : 1.f;
+    const float* pa = vin + (int64_t)va * ld;
+    const float* pb = vin + (int64_t)vb * ld;
+    const int q1 = rowptr[row + 1];
+    for (int q = rowptr[row] + tl; q < q1; q += LT) buf[colidx[q]] = make_float2(pa[q] * sa, has_b ? pb[q] * sb : 0.f);
     __syncthreads();
-    fft_smem<float2, false, EPT>(rb, L, tl, tw);
+    fft_smem<false>(buf, L, tl, tw);
 
     // store: slab[pair][tile][row][c]
     float2* out = slab + (int64_t)blockIdx.y * n1 * M2;
-    const int GC = G * C;
-    for (int e = threadIdx.x; e < G * L; e += blockDim.x) {
-        const int tile = e / GC;
-        const int rem = e - tile * GC;
-        const int gg = rem / C;
-        const int c = rem - gg * C;
-        const int r = row0 + gg;
-        if (r < n1) out[(int64_t)tile * n1 * C + (int64_t)r * C + c] = buf[gg * stride + tile * C + c];
+    for (int e = tl; e < L; e += LT) {
+        const int tile = e / C;
+        out[((int64_t)tile * n1 + row) * C + (e - tile * C)] = buf[e];
     }
 }
 
 // ------------------------------------------------------------------ pass B
 
-template <int EPT, int CC>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(float2* __restrict__ slab, const float* __restrict__ lamT,
-                                                 int n1, int M1, int M2, const float2* __restrict__ tw,
-                                                 int pair0, int64_t lam_stride, int vpt) {
+// CC columns, the slab's tile width.
+template <int CC>
+__global__ void __launch_bounds__(1024) k_pass_b(float2* __restrict__ slab, const float* __restrict__ lamT, int n1,
+                                                 int M1, int M2, const float2* __restrict__ tw, int pair0,
+                                                 int64_t lam_stride, int vpt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
     const int L = M1;
     const int stride = L + 1;
-    const int LT = L / EPT;
+    const int LT = L / 8;
     const int g = threadIdx.x / LT;
     const int tl = threadIdx.x - g * LT;
     const int tile = blockIdx.x;
@@ -118,7 +99,7 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(float2* __res
     }
     __syncthreads();
     float2* cb = buf + g * stride;
-    fft_smem<float2, false, EPT>(cb, L, tl, tw);
+    fft_smem<false>(cb, L, tl, tw);
     const int theta = vpt ? (2 * (pair0 + (int)blockIdx.y)) / vpt : 0;
     const float* lam = lamT + theta * lam_stride + (int64_t)(tile * CC + g) * L;
     for (int k = tl; k < L; k += LT) {
@@ -127,7 +108,7 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(float2* __res
         cb[k] = make_float2(z.x * l, z.y * l);
     }
     __syncthreads();
-    fft_smem<float2, true, EPT>(cb, L, tl, tw);
+    fft_smem<true>(cb, L, tl, tw);
     for (int e = threadIdx.x; e < nload; e += blockDim.x) {
         const int i = e / CC;
         const int c = e - i * CC;
@@ -137,46 +118,31 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_b(float2* __res
 
 // ------------------------------------------------------------------ pass C
 
-// Gathers the observed cells, adds tau2 * (scaled input), optional dot.
-template <int EPT, int G>
-__global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const float2* __restrict__ slab, const float* __restrict__ vin,
-                                                 int64_t ld_in, const double* __restrict__ scale, float* __restrict__ vout,
-                                                 int64_t ld_out, int nvec, int pair0, const int* __restrict__ rowptr,
-                                                 const int* __restrict__ colidx, int n1, int n2, int M2, int C,
-                                                 double tau2, double* __restrict__ dots, int ndot_stride,
-                                                 const float2* __restrict__ tw, const double* __restrict__ tau2v,
-                                                 int vpt) {
+// One row: inverse FFT, the observed cells, tau2 * (scaled input), optional dot.
+__global__ void __launch_bounds__(1024) k_pass_c(const float2* __restrict__ slab, const float* __restrict__ vin,
+                                                 int64_t ld_in, const double* __restrict__ scale,
+                                                 float* __restrict__ vout, int64_t ld_out, int nvec, int pair0,
+                                                 const int* __restrict__ rowptr, const int* __restrict__ colidx,
+                                                 int n1, int M2, int C, double tau2, double* __restrict__ dots,
+                                                 int ndot_stride, const float2* __restrict__ tw,
+                                                 const double* __restrict__ tau2v, int vpt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* buf = reinterpret_cast<float2*>(smem_raw);
     __shared__ double red[2][32];
-    const int L = M2;
-    const int stride = L + 1;
-    const int LT = L / EPT;
-    const int g = threadIdx.x / LT;
-    const int tl = threadIdx.x - g * LT;
-    const int row0 = blockIdx.x * G;
-    const int pair = pair0 + blockIdx.y;
-    const int va = 2 * pair, vb = 2 * pair + 1;
+    const int L = M2, LT = L / 8, tl = threadIdx.x, row = blockIdx.x;
+    const int va = 2 * (pair0 + (int)blockIdx.y), vb = va + 1;
     const bool has_b = vb < nvec;
 
     const float2* in = slab + (int64_t)blockIdx.y * n1 * M2;
-    const int GC = G * C;
-    for (int e = threadIdx.x; e < G * L; e += blockDim.x) {
-        const int tile = e / GC;
-        const int rem = e - tile * GC;
-        const int gg = rem / C;
-        const int c = rem - gg * C;
-        const int r = row0 + gg;
-        buf[gg * stride + tile * C + c] =
-            (r < n1) ? in[(int64_t)tile * n1 * C + (int64_t)r * C + c] : make_float2(0.f, 0.f);
+    for (int e = tl; e < L; e += LT) {
+        const int tile = e / C;
+        buf[e] = in[((int64_t)tile * n1 + row) * C + (e - tile * C)];
     }
     __syncthreads();
-    float2* rb = buf + g * stride;
-    fft_smem<float2, true, EPT>(rb, L, tl, tw);
+    fft_smem<true>(buf, L, tl, tw);
 
-    const int row = row0 + g;
     DotAcc<float> acc_a, acc_b;
-    if (row < n1) {
+    {
         const float sa = scale ? (float)scale[va] : 1.f;
         const float sb = (scale && has_b) ? (float)scale[vb] : 1.f;
         const float t2 = (float)(tau2v ? tau2v[vpt ? va / vpt : 0] : tau2);
@@ -186,7 +152,7 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const float2*
         float* ob = vout + (int64_t)vb * ld_out;
         const int q1 = rowptr[row + 1];
         for (int q = rowptr[row] + tl; q < q1; q += LT) {
-            const float2 z = rb[colidx[q]];
+            const float2 z = buf[colidx[q]];
             const float xa = pa[q] * sa;
             const float ya = z.x + t2 * xa;
             oa[q] = ya;
@@ -235,41 +201,9 @@ __global__ void __launch_bounds__(EPT >= 16 ? 512 : 1024) k_pass_c(const float2*
 
 static size_t cx_size(bool dbl) { return dbl ? sizeof(double2) : sizeof(float2); }
 
-int smem_limit(kry_ctx* ctx) { return ctx->max_smem_optin; }
-
-#define KRY_DISPATCH_EG(EPTV, GV, ...)                                                \
-    do {                                                                              \
-        if (EPTV == 8) {                                                              \
-            if (GV == 1) { constexpr int E_ = 8, G_ = 1; __VA_ARGS__; }                       \
-            else if (GV == 2) { constexpr int E_ = 8, G_ = 2; __VA_ARGS__; }                  \
-            else if (GV == 4) { constexpr int E_ = 8, G_ = 4; __VA_ARGS__; }                  \
-            else if (GV == 8) { constexpr int E_ = 8, G_ = 8; __VA_ARGS__; }                  \
-            else throw KryError{KRY_EUNSUPPORTED, "bad group count"};                \
-        } else if (EPTV == 16) {                                                      \
-            if (GV == 1) { constexpr int E_ = 16, G_ = 1; __VA_ARGS__; }                      \
-            else if (GV == 2) { constexpr int E_ = 16, G_ = 2; __VA_ARGS__; }                 \
-            else if (GV == 4) { constexpr int E_ = 16, G_ = 4; __VA_ARGS__; }                 \
-            else if (GV == 8) { constexpr int E_ = 16, G_ = 8; __VA_ARGS__; }                 \
-            else throw KryError{KRY_EUNSUPPORTED, "bad group count"};                \
-        } else                                                                        \
-            throw KryError{KRY_EUNSUPPORTED, "bad elements per thread"};              \
-    } while (0)
-
-// Schedule of the short FP32 passes that fits shared memory and the block limits.
-static MvSched pick_sched(kry_ctx* ctx, const MvSched& want, int M1, int M2) {
-    MvSched s = want;
-    const size_t lim = (size_t)ctx->max_smem_optin - 1024;   // leave room for static shared memory
-    auto fix = [&](int& ept, int& grp, int L) {
-        if (ept != 8 && ept != 16) ept = 8;
-        if (L < ept) ept = 8;
-        if (L / ept > 1024) ept = 16;
-        const int maxthr = (ept >= 16) ? 512 : 1024;
-        while (grp > 1 && ((size_t)grp * (L + 1) * sizeof(float2) > lim || grp * (L / ept) > maxthr)) grp /= 2;
-    };
-    fix(s.ept_row, s.rows_per_cta, M2);
-    fix(s.ept_col, s.cols_per_cta, M1);
-    return s;
-}
+// Columns per block (= slab tile width) of the short FP32 column pass: four, fewer
+// where their transforms exceed a block's threads.
+static int short_cols(int M1) { return M1 <= 2048 ? 4 : M1 == 4096 ? 2 : 1; }
 
 void prof_record(kry_ctx* ctx, cudaEvent_t ev) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -298,13 +232,14 @@ uint64_t sched_key(int M1, int M2, bool dbl, int nvec) {
 const MvSched& sched_for(kry_ctx* ctx, int M1, int M2, bool dbl, int nvec) {
     auto it = ctx->tuned.find(sched_key(M1, M2, dbl, nvec));
     if (it != ctx->tuned.end()) return it->second;
-    return dbl ? ctx->sched64 : ctx->sched32;
+    return ctx->sched;
 }
 
 // Rows per block (passes A and C) and columns per block (pass B) of the
 // specialised FP32 passes.  Blocks of 128 threads (four and more per SM, so that
 // one block's loads run behind another's butterflies), 256 for the longest
-// columns, whose slab rows would otherwise be read 8 bytes at a time; down to
+// columns: two of side 4096, or one of side 8192, which alone needs 256 threads
+// and reads and writes 8 bytes of each of its tile rows of 32.  Down to
 // two warps (one for columns) while the launch has fewer blocks than two per SM
 // (128^2, 4 vectors: 11.0 us, with 128 threads 12).  The rows per block group pass
 // C's dot partials, so they do not depend on the batch.
@@ -316,8 +251,8 @@ static void spec_shape(kry_ctx* ctx, const kry_embed* e, int nvec, int* G, int* 
         while (th > least && th > lt && transforms * lt / th < 2 * ctx->num_sms) th /= 2;
         return std::max(1, th / lt);
     };
-    const int g = want.g16 > 0 ? want.g16 : fill(ltr, 128, 64, M1 / 2);
-    const int c = want.c16 > 0 ? want.c16 : fill(ltc, M1 >= 4096 ? 256 : 128, 32, (int64_t)M2 * np);
+    const int g = want.rows > 0 ? want.rows : fill(ltr, 128, 64, M1 / 2);
+    const int c = want.cols > 0 ? want.cols : fill(ltc, M1 >= 4096 ? 256 : 128, 32, (int64_t)M2 * np);
     *G = kspec::block_threads(M2, g, 64) / ltr;
     *C = kspec::block_threads(M1, c, M2) / ltc;
 }
@@ -325,15 +260,15 @@ static void spec_shape(kry_ctx* ctx, const kry_embed* e, int nvec, int* G, int* 
 // Row and column transforms of the FP64 passes.
 static void shape64(kry_ctx* ctx, const kry_embed* e, int nvec, kf64::Shape* row, kf64::Shape* col) {
     const MvSched& want = sched_for(ctx, e->M1, e->M2, true, nvec);
-    *row = kf64::shape(e->M2, want.g16);
-    *col = kf64::shape(e->M1, want.c16);
+    *row = kf64::shape(e->M2, want.rows);
+    *col = kf64::shape(e->M1, want.cols);
 }
 
 // Complex pairs per batch: all, unless the schedule says otherwise.
 static int batch_pairs(kry_ctx* ctx, const kry_embed* e, bool dbl, int nvec) {
     const int npairs = (nvec + 1) / 2;
-    const MvSched& want =
-        dbl || use_spec(e->M1, e->M2) ? sched_for(ctx, e->M1, e->M2, dbl, nvec) : ctx->sched32;
+    if (!dbl && !use_spec(e->M1, e->M2)) return npairs;
+    const MvSched& want = sched_for(ctx, e->M1, e->M2, dbl, nvec);
     return want.pairs_per_batch > 0 ? std::min(want.pairs_per_batch, npairs) : npairs;
 }
 
@@ -367,7 +302,7 @@ static void run_passes(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t l
             kspec::SpecArgs a{};
             a.vin = vin; a.ld_in = ld_in; a.scale = scale; a.vout = vout; a.ld_out = ld_out;
             a.nvec = nvec; a.bits = ctx->cellbits.as<uint2>(); a.wpr = (n2 + 31) / 32;
-            a.n1 = n1; a.n2 = n2; a.M1 = M1; a.M2 = M2;
+            a.n1 = n1; a.M1 = M1; a.M2 = M2;
             spec_shape(ctx, e, nvec, &a.G, &a.C);
             a.logCs = ilog2(std::min(32, std::max(4, a.C)));   // tile rows of 1 to 8 32-byte sectors
             a.slab = static_cast<float2*>(slab); a.lamP = e->lam32P; a.lam_stride = e->lam_stride; a.vpt = vpt;
@@ -384,36 +319,26 @@ static void run_passes(kry_ctx* ctx, const kry_embed* e, const T* vin, int64_t l
             }
             return;
         }
-        const MvSched s = pick_sched(ctx, ctx->sched32, M1, M2);
-        const int C = s.cols_per_cta, G = s.rows_per_cta;
+        const int C = short_cols(M1);
         const int* rowptr = ctx->rowptr.as<int>();
         const int* colidx = ctx->colidx.as<int>();
         const float2* tw = ctx->tw32.as<float2>();
         float2* sl = static_cast<float2*>(slab);
-        const int thrA = G * (M2 / s.ept_row), thrB = C * (M1 / s.ept_col), nbx = (n1 + G - 1) / G;
-        const size_t smA = (size_t)G * (M2 + 1) * sizeof(float2), smB = (size_t)C * (M1 + 1) * sizeof(float2);
+        const size_t smA = (size_t)(M2 + 1) * sizeof(float2), smB = (size_t)C * (M1 + 1) * sizeof(float2);
+        auto pass_b = C == 4 ? k_pass_b<4> : C == 2 ? k_pass_b<2> : k_pass_b<1>;
+        KRY_ALLOW_MAX_SMEM(k_pass_a);
+        KRY_ALLOW_MAX_SMEM(pass_b);
+        KRY_ALLOW_MAX_SMEM(k_pass_c);
         for (int pair0 = 0; pair0 < npairs; pair0 += ppb) {
             const int np = std::min(ppb, npairs - pair0);
-            const dim3 gA(nbx, np), gB(M2 / C, np);
-            KRY_DISPATCH_EG(s.ept_row, G, {
-                auto k = k_pass_a<E_, G_>;
-                KRY_ALLOW_MAX_SMEM(k);
-                k<<<gA, thrA, smA, st>>>(vin, ld_in, scale, nvec, pair0, rowptr, colidx, n1, M2, C, sl, tw);
-                KRY_CHECK_LAUNCH();
-            });
-            KRY_DISPATCH_EG(s.ept_col, C, {
-                auto k = k_pass_b<E_, G_>;
-                KRY_ALLOW_MAX_SMEM(k);
-                k<<<gB, thrB, smB, st>>>(sl, e->lam32T, n1, M1, M2, tw, pair0, e->lam_stride, vpt);
-                KRY_CHECK_LAUNCH();
-            });
-            KRY_DISPATCH_EG(s.ept_row, G, {
-                auto k = k_pass_c<E_, G_>;
-                KRY_ALLOW_MAX_SMEM(k);
-                k<<<gA, thrA, smA, st>>>(sl, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, n2, M2,
-                                         C, tau2, dots, nds, tw, tau2v, vpt);
-                KRY_CHECK_LAUNCH();
-            });
+            const dim3 gA(n1, np), gB(M2 / C, np);
+            k_pass_a<<<gA, M2 / 8, smA, st>>>(vin, ld_in, scale, nvec, pair0, rowptr, colidx, n1, M2, C, sl, tw);
+            KRY_CHECK_LAUNCH();
+            pass_b<<<gB, C * (M1 / 8), smB, st>>>(sl, e->lam32T, n1, M1, M2, tw, pair0, e->lam_stride, vpt);
+            KRY_CHECK_LAUNCH();
+            k_pass_c<<<gA, M2 / 8, smA, st>>>(sl, vin, ld_in, scale, vout, ld_out, nvec, pair0, rowptr, colidx, n1, M2,
+                                              C, tau2, dots, nds, tw, tau2v, vpt);
+            KRY_CHECK_LAUNCH();
         }
     }
 }
@@ -511,8 +436,7 @@ int matvec_num_partials(kry_ctx* ctx, const kry_embed* e, bool dbl, int nvec) {
         spec_shape(ctx, e, nvec, &G, &C);
         return (e->n1 + G - 1) / G;
     }
-    const MvSched s = pick_sched(ctx, ctx->sched32, e->M1, e->M2);
-    return (e->n1 + s.rows_per_cta - 1) / s.rows_per_cta;
+    return e->n1;   // the short passes take a row per block
 }
 
 template <typename T>
@@ -671,7 +595,7 @@ extern "C" kry_status kry_matvec_noalloc(kry_ctx* ctx, const kry_embed* e, const
 
 // ------------------------------------------------------------------ schedule autotuner
 //
-// Times every feasible radix-16 schedule (rows per block for the row passes,
+// Times every feasible schedule (rows per block for the row passes,
 // columns per block = slab tile width for the column pass, complex pairs per
 // batch: all at once, or chunks whose slab stays within ~32 or ~64 MB of L2)
 // on the caller's embedding and batch width, and caches the fastest for
@@ -726,7 +650,7 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
         if (c < npairs && std::find(ppbs.begin(), ppbs.end(), c) == ppbs.end()) ppbs.push_back(c);
     }
     double best = 1e30;
-    MvSched bs = dbl ? ctx->sched64 : ctx->sched32;
+    MvSched bs = ctx->sched;
     const bool had = ctx->tuned.count(key) > 0;
     const MvSched prev = had ? ctx->tuned[key] : bs;
     if (dbl || use_spec(M1, M2)) {
@@ -742,8 +666,8 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
                 if (c && !feasible(M1, c, M2)) continue;
                 for (int ppb : ppbs) {
                     MvSched cand = bs;
-                    cand.g16 = g;
-                    cand.c16 = c;
+                    cand.rows = g;
+                    cand.cols = c;
                     cand.pairs_per_batch = ppb;
                     ctx->tuned[key] = cand;
                     const double ms = time_sched<T>(ctx, e, tv.as<T>(), to.as<T>(), nvec, 3);
@@ -760,16 +684,16 @@ static double autotune_t(kry_ctx* ctx, const kry_embed* e, int nvec, MvSched* be
             kf64::Shape row, col;
             ctx->tuned[key] = bs;
             shape64(ctx, e, nvec, &row, &col);
-            bs.g16 = row.NT;
-            bs.c16 = col.NT;
+            bs.rows = row.NT;
+            bs.cols = col.NT;
         } else {
             ctx->tuned[key] = bs;
-            spec_shape(ctx, e, nvec, &bs.g16, &bs.c16);
+            spec_shape(ctx, e, nvec, &bs.rows, &bs.cols);
         }
         ctx->tuned[key] = bs;
         // the default blocks of the shortest tori hold more transforms than kry_set_schedule takes:
         // reported as 0, which names the same blocks
-        for (int* b : {&bs.g16, &bs.c16})
+        for (int* b : {&bs.rows, &bs.cols})
             if (*b > 16) *b = 0;
     } else {
         if (had) ctx->tuned[key] = prev;
@@ -800,8 +724,8 @@ extern "C" kry_status kry_autotune(kry_ctx* ctx, const kry_embed* e, int32_t nve
         MvSched b;
         const double ms = kry::autotune(ctx, e, nvec, &b);
         if (best_ms) *best_ms = ms;
-        if (rows_per_block) *rows_per_block = b.g16;
-        if (cols_per_block) *cols_per_block = b.c16;
+        if (rows_per_block) *rows_per_block = b.rows;
+        if (cols_per_block) *cols_per_block = b.cols;
         if (pairs_per_batch) *pairs_per_batch = b.pairs_per_batch;
         return KRY_OK;
     } catch (const KryError& err) {
@@ -823,9 +747,9 @@ extern "C" kry_status kry_set_schedule(kry_ctx* ctx, const kry_embed* e, int32_t
                         cols_per_block <= 16 && pairs_per_batch >= 0,
                     KRY_EINVAL, "rows/cols per block must be 0 (default) or a power of two <= 16; pairs >= 0");
         const bool dbl = e->prec == KRY_F64;
-        MvSched s = dbl ? ctx->sched64 : ctx->sched32;
-        s.g16 = rows_per_block;
-        s.c16 = cols_per_block;
+        MvSched s = ctx->sched;
+        s.rows = rows_per_block;
+        s.cols = cols_per_block;
         s.pairs_per_batch = pairs_per_batch;
         ctx->tuned[kry::sched_key(e->M1, e->M2, dbl, nvec)] = s;
         return KRY_OK;

@@ -99,7 +99,7 @@ __device__ __forceinline__ void load_post(float2 (&f)[E], const float2* __restri
 template <int B, int TH>
 __global__ void __launch_bounds__(TH, minb(B, TH))
     ks_pass_a(const float* __restrict__ vin, int64_t ld, const double* __restrict__ scale, int nvec, int pair0,
-              const uint2* __restrict__ bits, int wpr, int n1, int n2, int logCs, float4* __restrict__ slab,
+              const uint2* __restrict__ bits, int wpr, int n1, int logCs, float4* __restrict__ slab,
               const float4* __restrict__ twf, const int* __restrict__ skip) {
     using P = Plan<B>;
     constexpr int H = P::H, E = P::E, LT = P::LT, NT = nt_of(B, TH), PS = pad_shift(H);
@@ -230,7 +230,7 @@ template <int B, int TH>
 __global__ void __launch_bounds__(TH, minb(B, TH))
     ks_pass_c(const float4* __restrict__ slab, const float* __restrict__ vin, int64_t ld_in,
               const double* __restrict__ scale, float* __restrict__ vout, int64_t ld_out, int nvec, int pair0,
-              const uint2* __restrict__ bits, int wpr, int n1, int n2, int logCs, double tau2,
+              const uint2* __restrict__ bits, int wpr, int n1, int logCs, double tau2,
               double* __restrict__ dots, int ndot_stride, const float4* __restrict__ twi,
               const float2* __restrict__ post, const double* __restrict__ tau2v, int vpt,
               const int* __restrict__ skip) {
@@ -334,7 +334,7 @@ struct SpecArgs {
     int nvec, pair0, np;
     const uint2* bits;
     int wpr;
-    int n1, n2, M1, M2;
+    int n1, M1, M2;
     int G, C, logCs;   // rows per block (A, C), columns per block (B), log2 of the slab tile width
     float2* slab;
     const float* lamP;   // column-permuted FP32 eigenvalues (kry_embed::lam32P)

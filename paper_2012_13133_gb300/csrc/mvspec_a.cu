@@ -80,7 +80,7 @@ struct RunA {
             auto k = ks_pass_a<B, TH>;
             KRY_ALLOW_MAX_SMEM(k);
             launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, a.vin, a.ld_in, a.scale, a.nvec, a.pair0, a.bits, a.wpr,
-                       a.n1, a.n2, a.logCs, reinterpret_cast<float4*>(a.slab), a.twf, a.skip);
+                       a.n1, a.logCs, reinterpret_cast<float4*>(a.slab), a.twf, a.skip);
         }
         return true;
     }

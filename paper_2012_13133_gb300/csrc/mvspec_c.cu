@@ -23,7 +23,7 @@ struct RunC {
             auto k = ks_pass_c<B, TH>;
             KRY_ALLOW_MAX_SMEM(k);
             launch_pdl(k, grid, dim3(TH), smem_bytes(B, TH), st, reinterpret_cast<const float4*>(a.slab), a.vin, a.ld_in,
-                       a.scale, a.vout, a.ld_out, a.nvec, a.pair0, a.bits, a.wpr, a.n1, a.n2, a.logCs, a.tau2, a.dots,
+                       a.scale, a.vout, a.ld_out, a.nvec, a.pair0, a.bits, a.wpr, a.n1, a.logCs, a.tau2, a.dots,
                        a.nds, a.twi, a.post, a.tau2v, a.vpt, a.skip);
         }
         return true;
