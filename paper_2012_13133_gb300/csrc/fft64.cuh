@@ -14,8 +14,9 @@
 //  * E = 16 for long transforms, E = 4 up to 512 points: a thread's serial chain is
 //    a quarter as long, and small grids have too few warps for the chip's 608
 //    schedulers otherwise.
-// Where cos = 0 the table holds +-2^-55 for it (what this adds is an eighth of a unit
-// roundoff), so intermediate values are to stay below 2^969.
+// Level 1, whose angles reach half a turn (cos = 0), takes p = a + w b with (cos,
+// sin) in its table entry, and 2 a - p: 6 instructions too.  The other levels' T
+// goes up to 1304 (side 8192), so intermediate values are to stay below 2^1013.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -76,6 +77,14 @@ __device__ __forceinline__ void bfly(double2& a, double2& b, double c, double T)
     if constexpr (!PLUS) b = m;
 }
 
+// The same for w = c -+ i s.
+template <bool INV, bool PLUS>
+__device__ __forceinline__ void bfly_cs(double2& a, double2& b, double c, double s) {
+    const double2 p = make_double2(fma(INV ? -s : s, b.y, fma(c, b.x, a.x)), fma(INV ? s : -s, b.x, fma(c, b.y, a.y)));
+    if constexpr (!PLUS) b = make_double2(fma(2.0, a.x, -p.x), fma(2.0, a.y, -p.y));
+    a = p;
+}
+
 // w = 1 (ROT: w = -+i)
 template <bool INV, bool ROT, bool PLUS>
 __device__ __forceinline__ void bfly1(double2& a, double2& b) {
@@ -112,7 +121,8 @@ __device__ __forceinline__ void level(double2* v, const double2* w) {
         }
         const double c = CONST ? cos16(e * (16 >> LEV)) : w[tw_base(LEV) + e].x;
         const double T = CONST ? tan16(e * (16 >> LEV)) : w[tw_base(LEV) + e].y;
-        if (rot) bfly<INV, true, PLUS>(v[p], v[p + D], c, T);
+        if (!CONST && LEV == 1) bfly_cs<INV, PLUS>(v[p], v[p + D], c, T);
+        else if (rot) bfly<INV, true, PLUS>(v[p], v[p + D], c, T);
         else bfly<INV, false, PLUS>(v[p], v[p + D], c, T);
     }
 }
@@ -127,7 +137,7 @@ __device__ __forceinline__ void levels(double2* v, const double2* w) {
 
 // Twiddle table: section 8 (NS - 2) of stage stride NS (a power of two in [2,
 // 512]), word e NS + k = (c, T) of entry e = s + 2^{l-2} of level l at frequency
-// k, angle (k / NS + s) / 2^l turns.
+// k, angle (k / NS + s) / 2^l turns; entry 0 (level 1): (cos, sin).
 constexpr int TW_WORDS = 8 * 1022;
 
 template <class P, int NT, int R, int NS>
