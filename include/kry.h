@@ -188,7 +188,9 @@ void kry_embed_free(kry_embed* e);
 
 /* out = K v for nvec vectors (K = sigma2 A Sigma A^T + tau2 I, Sec. 3).  v_dev
  * and out_dev are FP32 (prec KRY_F32) or FP64 (KRY_F64) arrays of nvec columns
- * with leading dimension ld.  Asynchronous.  v_dev and out_dev must not overlap. */
+ * with leading dimension ld.  Asynchronous.  v_dev and out_dev must not overlap.
+ * Range: FP32 results up to 2^118, and sums of a column's magnitudes over the grid
+ * within FP32; FP64 both up to 2^1012.  Beyond it a result can be Inf or NaN. */
 kry_status kry_matvec(kry_ctx* ctx, const kry_embed* e, const void* v_dev, void* out_dev,
                       int32_t nvec, int64_t ld);
 

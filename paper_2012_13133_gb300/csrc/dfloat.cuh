@@ -68,7 +68,9 @@ __device__ __forceinline__ TFloat tf_xor(const TFloat& x, int o) {
 // where finite sums leave the FP32 range together, in FP64 (a warp's FP64
 // instruction holds its scheduler's FP64 pipe for 64 cycles on GB300: an FP64
 // shuffle tree in every block of a streaming kernel takes longer than the
-// streaming).  Two sums share a tree, each half a warp's lanes.
+// streaming).  Two sums share a tree, each half a warp's lanes.  Against sums in
+// double-float, whose 48 bits and FP32 range are less than FP64's, a CG iteration
+// for 4 columns takes 25.4 -> 26.3 us on 128^2, 49.6 -> 50.4 us on 500^2.
 template <int N, int WARPS>
 __device__ __forceinline__ double block_sums(const DFAcc (&acc)[N]) {
     static_assert(N <= 2 && N * WARPS <= 32 && (WARPS & (WARPS - 1)) == 0, "a warp adds the warps' sums");

@@ -1113,7 +1113,7 @@ static std::vector<double> residual_norms(kry_ctx* ctx, int nrhs) {
 // us beside its first loads, where a launch of its own for alpha and for beta
 // took 3 us each.  x waits for the second kernel, which reads p anyhow.  An
 // iteration for 4 columns: 32 x 32 27.5 -> 24.1 us, 256 x 256 28.1 -> 26.0,
-// 1024 x 1024 100.7 -> 97.9.  (All of the vector work in one kernel, a cluster of
+// 1024 x 1024 100.7 -> 97.9 (both with sums in double-float; block_sums).  (All of the vector work in one kernel, a cluster of
 // 16 blocks per column, took 22.6 us at 256 x 256 but 113.7 at 1024 x 1024, and
 // no less than these two from 8 columns on.)
 // K p is computed afresh by every matvec, so no auxiliary recurrence can
@@ -1218,7 +1218,7 @@ __device__ __forceinline__ double total128(const double* __restrict__ part, int 
 }
 
 // alpha = gamma / p^T q (0 if p^T q is not positive), R -= alpha Q (FP32);
-// partials of ||R||^2 in double-float.  Streaming: two vectors read, one
+// partials of ||R||^2 (block_sums).  Streaming: two vectors read, one
 // written, from L2 where they fit.
 __global__ void __launch_bounds__(CG_THREADS) k_rcg_update(float* __restrict__ R, const float* __restrict__ Q, int64_t ld,
                                                     RcgState S, const double* __restrict__ part_pq, int npq,

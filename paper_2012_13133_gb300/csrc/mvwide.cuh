@@ -14,8 +14,8 @@
 // two to an instruction (21 -> 18 million warp instructions, no faster: issue is
 // not what bounds).
 // Measured against 16 packed values: 4 vectors on 1024^2 69.7 -> 57.5 us (passes
-// 15.3 + 36.3 + 20.0 -> 13.5 + 30.3 + 16.6), 64 vectors 921 -> 795 us, 32 vectors
-// on 512^2 121 -> 99 us, 5 vectors on 363 x 730 46.5 -> 37.8 us.  What is left:
+// 15.3 + 36.3 + 20.0 -> 13.5 + 30.3 + 16.6), 64 vectors 921 -> 799 us, 32 vectors
+// on 512^2 121 -> 99 us, 5 vectors on 363 x 730 46.5 -> 37.4 us.  What is left:
 // the L1 pipe 69% busy while the SMs are, FMA pipe 50%, and 15% (columns) to
 // 25% (rows) of a launch's time to start and to run out.
 //
